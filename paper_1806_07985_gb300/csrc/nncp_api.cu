@@ -283,8 +283,8 @@ cudaError_t update_mode(nncp_ctx* c, int n, cudaStream_t st) {
     }
     cudaError_t e = launch_apg_update(c->H[n], c->Mbuf, c->dims[n], c->R, c->nls_iters, c->st, st);
     if (e != cudaSuccess) return e;
-    return launch_finalize(c->H[n], c->dims[n], c->R, c->N, n, (n + 1) % c->N,
-                           hals_gram_blocks(c->dims[n]), n == c->N - 1, 0, 0.0, c->st, st);
+    return launch_finish(c->H[n], c->dims[n], c->R, c->N, n, (n + 1) % c->N, n == c->N - 1, c->st,
+                         c->red_part, st);
   }
   if (c->nls == NNCP_NLS_ADMM) {
     if (cluster_update_ok(c->dims[n], c->R)) {
@@ -297,9 +297,8 @@ cudaError_t update_mode(nncp_ctx* c, int n, cudaStream_t st) {
     cudaError_t e = launch_admm_update(c->H[n], c->U[n], c->Mbuf, c->dims[n], c->R,
                                        c->nls_iters, c->st, st);
     if (e != cudaSuccess) return e;
-    return launch_finalize(c->H[n], c->dims[n], c->R, c->N, n, (n + 1) % c->N,
-                           hals_gram_blocks(c->dims[n]), n == c->N - 1, 0, 0.0, c->st, st,
-                           c->U[n]);
+    return launch_finish(c->H[n], c->dims[n], c->R, c->N, n, (n + 1) % c->N, n == c->N - 1, c->st,
+                         c->red_part, st, c->U[n]);
   }
   if (c->nls == NNCP_NLS_BPP) {
     if (cluster_update_ok(c->dims[n], c->R)) {
@@ -310,8 +309,8 @@ cudaError_t update_mode(nncp_ctx* c, int n, cudaStream_t st) {
     }
     cudaError_t e = launch_bpp_update(c->H[n], c->Mbuf, c->dims[n], c->R, c->st, c->num_sms, st);
     if (e != cudaSuccess) return e;
-    return launch_finalize(c->H[n], c->dims[n], c->R, c->N, n, (n + 1) % c->N,
-                           hals_gram_blocks(c->dims[n]), n == c->N - 1, 0, 0.0, c->st, st);
+    return launch_finish(c->H[n], c->dims[n], c->R, c->N, n, (n + 1) % c->N, n == c->N - 1, c->st,
+                         c->red_part, st);
   }
   if (cluster_update_ok(c->dims[n], c->R))
     return launch_update_cluster(c->H[n], c->Mbuf, c->dims[n], c->R, c->N, n, (n + 1) % c->N,
@@ -321,8 +320,8 @@ cudaError_t update_mode(nncp_ctx* c, int n, cudaStream_t st) {
                                n == c->N - 1, c->st, c->upd_part, st);
   cudaError_t e = launch_hals_gram(c->H[n], c->Mbuf, c->dims[n], c->R, c->st, st);
   if (e != cudaSuccess) return e;
-  return launch_finalize(c->H[n], c->dims[n], c->R, c->N, n, (n + 1) % c->N,
-                         hals_gram_blocks(c->dims[n]), n == c->N - 1, 0, 0.0, c->st, st);
+  return launch_finish(c->H[n], c->dims[n], c->R, c->N, n, (n + 1) % c->N, n == c->N - 1, c->st,
+                       c->red_part, st);
 }
 
 // Node {a..last} held in T (half h, depth d): leaf M(a), update, child node.
@@ -417,18 +416,9 @@ nncp_status end_on_work(nncp_ctx* c) {
 
 nncp_status solve_init(nncp_ctx* c, double tol) {
   cudaStream_t st = c->work;
-  const int R = c->R, N = c->N;
-  CK(launch_solve_reset(c->st, R, tol, st));
-  for (int n = 0; n < N; ++n)
-    CK(cudaMemsetAsync(c->U[n], 0, (size_t)c->dims[n] * R * sizeof(float), st));
-  CK(launch_sumsq(c->X, c->precision == NNCP_BF16_STORED, c->I, c->red_part, c->red_nparts,
-                  c->st.scalars, nullptr, st));
-  for (int n = 0; n < N; ++n) {
-    CK(launch_gram_only(c->H[n], c->dims[n], R, c->st, st));
-    CK(launch_finalize(c->H[n], c->dims[n], R, N, n, -1, hals_gram_blocks(c->dims[n]), 0, 1,
-                       0.0, c->st, st));
-  }
-  CK(launch_compute_S(c->st, N, R, 0, st));
+  CK(launch_sumsq_partials(c->X, c->precision == NNCP_BF16_STORED, c->I, c->red_part, c->red_nparts, st));
+  CK(launch_solve_init(c->N, c->dims, c->R, c->H, c->U, tol, c->red_part, c->red_nparts, c->st,
+                       c->partials, c->part_cap, st));
   c->initialised = true;
   return NNCP_OK;
 }

@@ -151,7 +151,10 @@ cudaError_t launch_mttv_first(const float* T, int64_t I, int64_t J, const float*
 
 // sum of squares of n float32 (or bf16) values into *out (float64), deterministic.
 cudaError_t launch_sumsq(const void* X, int bf16, int64_t n, double* partials, int nparts,
-                         double* out, const int* flags, cudaStream_t st);
+                         double* out, cudaStream_t st);
+// its partials alone
+cudaError_t launch_sumsq_partials(const void* X, int bf16, int64_t n, double* partials, int nparts,
+                                  cudaStream_t st);
 
 // float32 -> bf16 (round to nearest even).
 cudaError_t launch_to_bf16(const float* X, uint16_t* Y, int64_t n, cudaStream_t st);
@@ -191,7 +194,7 @@ cudaError_t launch_update_multi(float* H, const float* M, int64_t In, int R, int
 // Block principal pivoting NLS update (R <= 32): W = argmin_{W >= 0} of the
 // row-wise least squares with S = st.S and M, written to H unnormalised,
 // followed by the Gram partials and <M, W> into st.gram_part (then
-// launch_finalize, as after launch_hals_gram).
+// launch_finish, as after launch_hals_gram).
 cudaError_t launch_bpp_update(float* H, const float* M, int64_t In, int R, SolveState st,
                               int num_sms, cudaStream_t stream);
 // The row solves alone (W into H, unnormalised), for launch_update_cluster(sweep = 0).
@@ -200,7 +203,7 @@ cudaError_t launch_bpp_rows(float* H, const float* M, int64_t In, int R, SolveSt
 
 // AO-ADMM NLS update (R <= 32): `iters` ADMM iterations on every row from
 // z = H diag(lam), u = U diag(lam); z into H (unnormalised W), u into U.  The
-// _update form adds the Gram partials and <M, W> (then launch_finalize with
+// _update form adds the Gram partials and <M, W> (then launch_finish with
 // U); the _rows form is for launch_update_cluster(sweep = 0, U).
 cudaError_t launch_admm_rows(float* H, float* U, const float* M, int64_t In, int R, int iters,
                             SolveState st, cudaStream_t stream);
@@ -209,7 +212,7 @@ cudaError_t launch_admm_update(float* H, float* U, const float* M, int64_t In, i
 
 // Accelerated projected gradient NLS update (R <= 32): `iters` FISTA steps on
 // every row from W = H diag(lam), W into H (unnormalised).  The _update form
-// adds the Gram partials and <M, W> (then launch_finalize); the _rows form is
+// adds the Gram partials and <M, W> (then launch_finish); the _rows form is
 // for launch_update_cluster(sweep = 0).
 cudaError_t launch_apg_rows(float* H, const float* M, int64_t In, int R, int iters,
                            SolveState st, cudaStream_t stream);
@@ -224,21 +227,23 @@ cudaError_t launch_scale_columns(float* H, int64_t rows, int R, const float* inv
 cudaError_t launch_gram_only(const float* H, int64_t In, int R, SolveState st,
                              cudaStream_t stream);
 
-// Single-CTA finalise of a mode update:
+// The rest of a mode update after launch_hals_gram (or an NLS update's rows):
 //   W^T W = sum of the partials; lam = sqrt(diag); G_n = D^-1 W^T W D^-1;
 //   H_n = W / lam (in place); if is_last: fit from the Sec. IV-B identity;
-//   S for mode next_mode.  init = 1: lam *= column norms instead of replacing.
+//   S for mode next_mode.
+//   gscr: kFinishScratch doubles of device scratch.
 //   U non-null: the rows' ADMM duals, divided by the new lambda along with H.
-cudaError_t launch_finalize(float* H, int64_t In, int R, int N, int n, int next_mode,
-                            int nblocks, int is_last, int init, double tol, SolveState st,
-                            cudaStream_t stream, float* U = nullptr);
+constexpr int kFinishScratch = 304;
+cudaError_t launch_finish(float* H, int64_t In, int R, int N, int n, int next_mode, int is_last,
+                          SolveState st, double* gscr, cudaStream_t stream, float* U = nullptr);
 
-// lambda = 1, flags and fit counter cleared, tolerance stored (before initialisation).
-cudaError_t launch_solve_reset(SolveState st, int R, double tol, cudaStream_t stream);
-
-// S = Hadamard of every Gram but mode's, in float64 (st.S + mode R^2) and as
-// the float32 copy st.S32.
-cudaError_t launch_compute_S(SolveState st, int N, int R, int mode, cudaStream_t stream);
+// Start of a solve: every factor normalised, lambda = the product of its column
+// norms, the Grams, S of mode 1 (st.S32 and float64), alpha = the sum of the
+// nalpha partials, the ADMM duals zero, flags and fit counter cleared, the
+// tolerance stored.  scratch: device floats the partial Grams may use.
+cudaError_t launch_solve_init(int N, const int64_t* dims, int R, float* const* H, float* const* U,
+                              double tol, const double* alpha_part, int nalpha, SolveState st,
+                              float* scratch, size_t scratch_floats, cudaStream_t stream);
 
 // Explicit residual ||X - [[lam; H]]||^2 accumulated in float64 into out[0];
 // out[1] = ||X||^2.

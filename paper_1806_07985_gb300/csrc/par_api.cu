@@ -240,7 +240,7 @@ nncp_status nncp_par_alpha_local(nncp_par* p, const float* X_local, double* loca
   if (!p->ws) return pfail(p, NNCP_ERR_INVALID_ARG, "workspace not set");
   int64_t n = 1;
   for (int k = 0; k < p->N; ++k) n *= p->block_rows[k];
-  PCK(launch_sumsq(X_local, 0, n, p->red, kRedParts, p->red + kRedParts, nullptr, p->stream));
+  PCK(launch_sumsq(X_local, 0, n, p->red, kRedParts, p->red + kRedParts, p->stream));
   PCK(cudaMemcpyAsync(p->host_part, p->red + kRedParts, sizeof(double), cudaMemcpyDeviceToHost,
                       p->stream));
   PCK(cudaStreamSynchronize(p->stream));

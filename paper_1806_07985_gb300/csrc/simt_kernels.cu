@@ -415,56 +415,90 @@ __global__ void k_mttv_first(const float* __restrict__ T, long long I, const flo
   }
 }
 
-__device__ __forceinline__ double block_sum_double(double v, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += sh[i];
-  return t;  // valid in thread 0
-}
+// Sum of squares: four (float32) or two (bf16) squares at a time in float32,
+// accumulated as float-float pairs (TwoSum: no rounding is lost down to ~2^-48),
+// which cost a few float32 operations per 16 bytes, and added up in float64 once
+// per eight loads; one float64 addition per load had held the pass to 3.8 TB/s
+// on a GB300, float64 issuing at about a sixtieth of the float32 rate there.
+struct SumFF {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float v) {
+    const float s = hi + v, t = s - hi;
+    lo += (hi - (s - t)) + (v - t);
+    hi = s;
+  }
+};
 
-__global__ void k_sumsq_partial(const void* __restrict__ Xv, int bf16, long long n,
-                                double* __restrict__ partials, const int* flags) {
-  if (flags && flags[0]) return;
-  __shared__ double sh[32];
+__global__ void __launch_bounds__(256)
+k_sumsq_partial(const void* __restrict__ Xv, int bf16, long long n, double* __restrict__ partials) {
+  __shared__ double sh[8];
+  const long long stride = (long long)gridDim.x * 256;
+  const long long t0 = (long long)blockIdx.x * 256 + threadIdx.x;
+  const int per = bf16 ? 8 : 4;  // elements per 16 bytes
+  const long long nv = n / per;
+  const uint4* V = reinterpret_cast<const uint4*>(Xv);
+  SumFF a0, a1;
+  auto square = [&](const uint4& v) {
+    if (bf16) {
+      // products of bf16 values are exact in float32
+      const unsigned u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float x = __uint_as_float(u[i] << 16), y = __uint_as_float(u[i] & 0xffff0000u);
+        a0.add(x * x);
+        a1.add(y * y);
+      }
+    } else {
+      const float x = __uint_as_float(v.x), y = __uint_as_float(v.y), z = __uint_as_float(v.z),
+                  w = __uint_as_float(v.w);
+      float s = x * x;
+      s = fmaf(y, y, s);
+      s = fmaf(z, z, s);
+      s = fmaf(w, w, s);
+      a0.add(s);
+    }
+  };
+  // into float64 after every eight loads, which keeps float32's range out of
+  // the sum; an infinite square stays infinite
   double acc = 0.0;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (!bf16) {
-    const float* X = static_cast<const float*>(Xv);
-    const long long n4 = n / 4;
-    const float4* X4 = reinterpret_cast<const float4*>(X);
-    for (long long t = t0; t < n4; t += stride) {
-      float4 v = __ldg(X4 + t);
-      float s = v.x * v.x;
-      s = fmaf(v.y, v.y, s);
-      s = fmaf(v.z, v.z, s);
-      s = fmaf(v.w, v.w, s);
-      acc += (double)s;
-    }
-    for (long long t = n4 * 4 + t0; t < n; t += stride) acc += (double)X[t] * X[t];
-  } else {
-    const __nv_bfloat16* X = static_cast<const __nv_bfloat16*>(Xv);
-    for (long long t = t0; t < n; t += stride) {
-      float v = __bfloat162float(X[t]);
-      acc += (double)(v * v);
-    }
+  auto flush = [&]() {
+    const float h = a0.hi + a1.hi;
+    acc += isfinite(h) ? ((double)a0.hi + (double)a1.hi) + (double)(a0.lo + a1.lo) : (double)h;
+    a0 = a1 = SumFF();
+  };
+  long long t = t0;
+  for (; t + 7 * stride < nv; t += 8 * stride) {  // eight loads in flight
+    uint4 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = __ldcs(V + t + q * stride);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) square(v[q]);
+    flush();
   }
-  double tot = block_sum_double(acc, sh);
-  if (threadIdx.x == 0) partials[blockIdx.x] = tot;
+  for (; t < nv; t += stride) square(__ldcs(V + t));
+  flush();
+  for (long long e = nv * per + t0; e < n; e += stride) {
+    const float x = bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(Xv)[e])
+                         : static_cast<const float*>(Xv)[e];
+    a0.add(x * x);
+  }
+  flush();
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double tot = 0.0;
+    for (int i = 0; i < 8; ++i) tot += sh[i];
+    partials[blockIdx.x] = tot;
+  }
 }
 
-__global__ void k_sum_partials(const double* __restrict__ partials, int n, double* out,
-                               const int* flags) {
-  if (flags && flags[0]) return;
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += partials[i];
-    out[0] = s;
-  }
+__global__ void k_sum_partials(const double* __restrict__ partials, int n, double* out) {
+  double s = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += 32) s += partials[i];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (threadIdx.x == 0) out[0] = s;
 }
 
 __global__ void k_to_bf16(const float* __restrict__ X, __nv_bfloat16* __restrict__ Y, long long n) {
@@ -602,10 +636,17 @@ cudaError_t launch_mttv_first(const float* T, int64_t I, int64_t J, const float*
                        dim3(threads), smem, st, T, (long long)I, H, R, G, out);
 }
 
+cudaError_t launch_sumsq_partials(const void* X, int bf16, int64_t n, double* partials, int nparts,
+                                  cudaStream_t st) {
+  k_sumsq_partial<<<nparts, 256, 0, st>>>(X, bf16, n, partials);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_sumsq(const void* X, int bf16, int64_t n, double* partials, int nparts,
-                         double* out, const int* flags, cudaStream_t st) {
-  k_sumsq_partial<<<nparts, 256, 0, st>>>(X, bf16, n, partials, flags);
-  k_sum_partials<<<1, 32, 0, st>>>(partials, nparts, out, flags);
+                         double* out, cudaStream_t st) {
+  const cudaError_t e = launch_sumsq_partials(X, bf16, n, partials, nparts, st);
+  if (e != cudaSuccess) return e;
+  k_sum_partials<<<1, 32, 0, st>>>(partials, nparts, out);
   return cudaGetLastError();
 }
 

@@ -5,9 +5,10 @@
 // Grams for the next mode.  Three forms by mode length:
 //   k_update_cluster  I_n <= 1024: one launch on a thread-block cluster that
 //                     exchanges its partials through distributed shared memory;
-//   k_update_multi    I_n <= 16384: CTAs of 128 rows, the last CTA (atomic
+//   k_update_multi    I_n R < 131072: CTAs of 128 rows, the last CTA (atomic
 //                     ticket) finishes;
-//   k_hals_gram + k_finalize  otherwise (and for the solve's initialisation).
+//   k_hals_gram + k_finish  otherwise (rows over every SM, then the rest over as
+//                     many CTAs); the solve's initialisation shares their code.
 // The factors, the HALS arithmetic, the Grams and S are float32.  The sums the
 // fit needs to more than float32 precision (<M, W> and lambda^T (S * G) lambda)
 // are float-float (unevaluated hi + lo pairs added with the error-free TwoSum),
@@ -15,8 +16,10 @@
 // 60x slower than float32 on this GPU, so it is kept off every per-element path.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "nncp_internal.cuh"
 
@@ -26,11 +29,6 @@ namespace {
 
 constexpr int kRowsPerBlock = 64;
 constexpr int kHalsThreads = 256;
-
-__device__ __forceinline__ float warp_sum(float v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // 1 / sqrt(g) and sqrt(g) in float64 for a float32 g: a float32 estimate
 // refined by two steps of Newton's iteration for the reciprocal square root,
@@ -60,94 +58,225 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// One HALS sweep per row, one warp per row; lane holds columns lane + 32*j.
-// Then the block's partial W^T W (float32 over <= 64 rows, stored as double)
-// and partial <M, W>.
+// Rows of a mode of any length and rank: the HALS sweep (Sec. II-B) and the
+// partial W^T W and <M, W>, 64 rows at a time, four lanes per row.  Lane q of a
+// row's quad holds columns 16 j + 4 q .. + 3 in registers (all indices static)
+// and the matching part of every dot product, which two shuffles complete; the
+// quads of a warp read the same row of S, four neighbouring 16-byte chunks, so
+// the reads are broadcasts without bank conflicts.  Then W^T W from small
+// register tiles.  A column step is a chain of R / 16 x 4 FMAs, two shuffles and
+// the update (~150 cycles), so the sweep is bound by its R dependent columns;
+// a row per quad gives four times the threads that a row per thread would, and
+// one of S's rows is read for eight matrix rows at once.  (A warp per row with a
+// five-step shuffle sum per column took 285 us for 220 rows at R = 100 on a GB300.)
+template <int RMAX>
+struct RowsCfg {
+  static constexpr int NJ = RMAX / 16;       // chunks of four columns per lane
+  static constexpr int RP = RMAX + 4;        // padded row stride in shared memory
+  static constexpr int TB = RMAX <= 32 ? 2 : 4;  // W^T W tile of a thread
+};
+
+template <int RMAX>
+__device__ __forceinline__ void rows_block(float* __restrict__ H, const float* __restrict__ M,
+                                           long long In, int R, const float* __restrict__ S,
+                                           const double* __restrict__ lam, double* __restrict__ gp,
+                                           int do_hals, int block, int nblocks, float* sm,
+                                           bool write_beta = true) {
+  using C = RowsCfg<RMAX>;
+  constexpr int NJ = C::NJ, RP = C::RP;
+  float* Ws = sm;                               // kRowsPerBlock x RP
+  float* Ss = Ws + kRowsPerBlock * RP;          // R x RMAX (sweeps only)
+  __shared__ double wbeta[kHalsThreads / 32];
+  __shared__ float lamf[RMAX], srr_s[RMAX], sinv[RMAX];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int q = tid & 3, row = tid >> 2;
+  const bool vec = (R & 3) == 0 &&
+                   ((reinterpret_cast<uintptr_t>(H) | reinterpret_cast<uintptr_t>(M)) & 15) == 0;
+  if (do_hals == 1) {
+    // columns past R are zero; S is symmetric, so row r serves as column r
+    for (int e = tid; e < R * (RMAX / 4); e += kHalsThreads) {
+      const int r = e / (RMAX / 4), c = 4 * (e - r * (RMAX / 4));
+      float4 v;
+      v.x = c < R ? __ldg(S + r * R + c) : 0.0f;
+      v.y = c + 1 < R ? __ldg(S + r * R + c + 1) : 0.0f;
+      v.z = c + 2 < R ? __ldg(S + r * R + c + 2) : 0.0f;
+      v.w = c + 3 < R ? __ldg(S + r * R + c + 3) : 0.0f;
+      *reinterpret_cast<float4*>(Ss + r * RMAX + c) = v;
+    }
+    for (int r = tid; r < R; r += kHalsThreads) {
+      const float d = __ldg(S + r * R + r);
+      srr_s[r] = d;
+      sinv[r] = d != 0.0f ? 1.0f / d : 0.0f;
+      lamf[r] = (float)lam[r];
+    }
+    __syncthreads();
+  }
+  constexpr int TB = C::TB;
+  const int nb4 = (R + 3) >> 2, nt = (R + TB - 1) / TB, tiles = nt * nt;
+  double beta = 0.0;
+  bool first = true;
+  for (long long row0 = (long long)block * kRowsPerBlock; row0 < In;
+       row0 += (long long)nblocks * kRowsPerBlock) {
+    const int nrows = (int)min((long long)kRowsPerBlock, In - row0);
+    const long long i = row0 + row;
+    const bool in = row < nrows;
+    float w[NJ][4], m[NJ][4];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const int c = 16 * j + 4 * q;
+      float4 h = make_float4(0.0f, 0.0f, 0.0f, 0.0f), mm = h;
+      if (in && c < R) {
+        const float* hp = H + i * R + c;
+        const float* mp = M + i * R + c;
+        if (vec) {
+          h = *reinterpret_cast<const float4*>(hp);
+          if (do_hals) mm = *reinterpret_cast<const float4*>(mp);
+        } else {
+          h.x = hp[0];
+          if (c + 1 < R) h.y = hp[1];
+          if (c + 2 < R) h.z = hp[2];
+          if (c + 3 < R) h.w = hp[3];
+          if (do_hals) {
+            mm.x = mp[0];
+            if (c + 1 < R) mm.y = mp[1];
+            if (c + 2 < R) mm.z = mp[2];
+            if (c + 3 < R) mm.w = mp[3];
+          }
+        }
+      }
+      w[j][0] = h.x; w[j][1] = h.y; w[j][2] = h.z; w[j][3] = h.w;
+      m[j][0] = mm.x; m[j][1] = mm.y; m[j][2] = mm.z; m[j][3] = mm.w;
+    }
+    if (do_hals == 1) {
+#pragma unroll
+      for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const int c = 16 * j + 4 * q + t;
+          w[j][t] = c < R ? w[j][t] * lamf[c] : 0.0f;
+        }
+#pragma unroll 1
+      for (int r4 = 0; r4 < nb4; ++r4) {
+        const int jr = r4 >> 2;
+        const bool own = (r4 & 3) == q;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const int r = 4 * r4 + t;
+          if (r >= R) break;
+          const float4* srow = reinterpret_cast<const float4*>(Ss + r * RMAX) + q;
+          float d0 = 0.0f, d1 = 0.0f, d2 = 0.0f, d3 = 0.0f;
+          float wr = 0.0f, mr = 0.0f;
+#pragma unroll
+          for (int j = 0; j < NJ; ++j) {
+            const float4 sv = srow[4 * j];
+            d0 = fmaf(w[j][0], sv.x, d0);
+            d1 = fmaf(w[j][1], sv.y, d1);
+            d2 = fmaf(w[j][2], sv.z, d2);
+            d3 = fmaf(w[j][3], sv.w, d3);
+            if (j == jr) {
+              wr = w[j][t];
+              mr = m[j][t];
+            }
+          }
+          float dot = (d0 + d1) + (d2 + d3);
+          dot += __shfl_xor_sync(0xffffffffu, dot, 1);
+          dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+          // (m - dot) / s_rr: the product with the reciprocal, corrected once
+          const float num = mr - dot, si = sinv[r];
+          float step = num * si;
+          step = fmaf(fmaf(-srr_s[r], step, num), si, step);
+          const float upd = fmaxf(0.0f, wr + step);
+          if (own && si != 0.0f) {  // S_rr = 0: column left as it is
+#pragma unroll
+            for (int j = 0; j < NJ; ++j)
+              if (j == jr) w[j][t] = upd;
+          }
+        }
+      }
+    }
+    float b = 0.0f;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const int c = 16 * j + 4 * q;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) b = fmaf(m[j][t], w[j][t], b);
+      *reinterpret_cast<float4*>(Ws + row * RP + c) = make_float4(w[j][0], w[j][1], w[j][2], w[j][3]);
+      if (do_hals == 1 && in && c < R) {
+        float* hp = H + i * R + c;
+        if (vec) {
+          *reinterpret_cast<float4*>(hp) = make_float4(w[j][0], w[j][1], w[j][2], w[j][3]);
+        } else {
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            if (c + t < R) hp[t] = w[j][t];
+        }
+      }
+    }
+    if (do_hals) {
+      b += __shfl_xor_sync(0xffffffffu, b, 1);
+      b += __shfl_xor_sync(0xffffffffu, b, 2);
+      beta += q == 0 ? (double)b : 0.0;
+    }
+    __syncthreads();
+    // W^T W of these rows, every output over the rows in order: a thread per
+    // TB x TB tile
+#pragma unroll 1
+    for (int tile = tid; tile < tiles; tile += kHalsThreads) {
+      const int a0 = (tile / nt) * TB, b0 = (tile % nt) * TB;
+      float acc[TB][TB];
+#pragma unroll
+      for (int x = 0; x < TB; ++x)
+#pragma unroll
+        for (int y = 0; y < TB; ++y) acc[x][y] = 0.0f;
+#pragma unroll 4
+      for (int rr = 0; rr < nrows; ++rr) {
+        using V = typename std::conditional<TB == 4, float4, float2>::type;
+        const V qa = *reinterpret_cast<const V*>(Ws + rr * RP + a0);
+        const V qb = *reinterpret_cast<const V*>(Ws + rr * RP + b0);
+        const float* va = reinterpret_cast<const float*>(&qa);
+        const float* vb = reinterpret_cast<const float*>(&qb);
+#pragma unroll
+        for (int x = 0; x < TB; ++x)
+#pragma unroll
+          for (int y = 0; y < TB; ++y) acc[x][y] = fmaf(va[x], vb[y], acc[x][y]);
+      }
+#pragma unroll
+      for (int x = 0; x < TB; ++x)
+#pragma unroll
+        for (int y = 0; y < TB; ++y)
+          if (a0 + x < R && b0 + y < R) {
+            double* o = gp + (a0 + x) * R + b0 + y;
+            *o = first ? (double)acc[x][y] : *o + (double)acc[x][y];
+          }
+    }
+    __syncthreads();
+    first = false;
+  }
+  if (!write_beta) return;
+  beta = warp_sum_d(beta);
+  if (lane == 0) wbeta[warp] = beta;
+  __syncthreads();
+  if (tid == 0) {
+    double bsum = 0.0;
+    for (int k = 0; k < kHalsThreads / 32; ++k) bsum += wbeta[k];
+    gp[R * R] = bsum;
+  }
+}
+
+// do_hals: 1 = HALS sweep on W = H diag(lam), then the partials; 0 = the
+// partials of W = H alone (no <M, W>); 2 = W given in H (an NLS solve of the
+// rows): the partials and <M, W>, no sweep.
+template <int RMAX>
 __global__ void __launch_bounds__(kHalsThreads)
 k_hals_gram(float* __restrict__ H, const float* __restrict__ M, long long In, int R,
             const float* __restrict__ S, const double* __restrict__ lam,
             double* __restrict__ gram_part, const int* __restrict__ flags, int do_hals) {
-  // do_hals: 1 = HALS sweep on W = H diag(lam), then the partials; 0 = the
-  // partials of W = H alone (no <M, W>); 2 = W given in H (the block
-  // principal pivoting update): the partials and <M, W>, no sweep
   pdl_wait();
   pdl_trigger();
   if (flags && flags[0]) return;
-  extern __shared__ float sm[];
-  float* Ss = sm;                        // R x R
-  float* Ws = Ss + R * R;                // kRowsPerBlock x (R + 1)
-  __shared__ double wbeta[kHalsThreads / 32];
-  const int RP = R + 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long row0 = (long long)blockIdx.x * kRowsPerBlock;
-  const int nrows = (int)min((long long)kRowsPerBlock, In - row0);
-
-  if (do_hals)
-    for (int t = threadIdx.x; t < R * R; t += blockDim.x) Ss[t] = S[t];
-  __syncthreads();
-
-  double beta_acc = 0.0;
-  for (int rr = warp; rr < nrows; rr += kHalsThreads / 32) {
-    const long long i = row0 + rr;
-    float w[4], m[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int c = lane + 32 * j;
-      w[j] = 0.0f;
-      m[j] = 0.0f;
-      if (c < R) {
-        w[j] = H[i * R + c];
-        if (do_hals) {
-          if (do_hals == 1) w[j] = w[j] * (float)lam[c];
-          m[j] = M[i * R + c];
-        }
-      }
-    }
-    if (do_hals == 1) {
-      for (int r = 0; r < R; ++r) {
-        const float srr = Ss[r * R + r];
-        if (srr == 0.0f) continue;  // warp-uniform
-        float part = 0.0f;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          int c = lane + 32 * j;
-          if (c < R) part = fmaf(w[j], Ss[c * R + r], part);
-        }
-        const float dot = warp_sum(part);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (lane + 32 * j == r) w[j] = fmaxf(0.0f, w[j] + (m[j] - dot) / srr);
-      }
-    }
-    if (do_hals) {
-      float bp = 0.0f;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bp = fmaf(m[j], w[j], bp);
-      beta_acc += (double)warp_sum(bp);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int c = lane + 32 * j;
-      if (c < R) {
-        if (do_hals == 1) H[i * R + c] = w[j];
-        Ws[rr * RP + c] = w[j];
-      }
-    }
-  }
-  if (lane == 0) wbeta[warp] = beta_acc;
-  __syncthreads();
-  double* gp = gram_part + (long long)blockIdx.x * (R * R + 1);
-  for (int t = threadIdx.x; t < R * R; t += blockDim.x) {
-    const int a = t / R, b = t % R;
-    float s = 0.0f;
-    for (int rr = 0; rr < nrows; ++rr) s = fmaf(Ws[rr * RP + a], Ws[rr * RP + b], s);
-    gp[t] = (double)s;
-  }
-  if (threadIdx.x == 0) {
-    double bsum = 0.0;
-    for (int w = 0; w < kHalsThreads / 32; ++w) bsum += wbeta[w];
-    gp[R * R] = bsum;
-  }
+  extern __shared__ __align__(16) float sm[];
+  rows_block<RMAX>(H, M, In, R, S, lam, gram_part + (long long)blockIdx.x * (R * R + 1), do_hals,
+                   blockIdx.x, gridDim.x, sm);
 }
 
 // fit = 1 - eps, eps^2 = (alpha - 2 beta + gamma) / alpha clamped at 0 (Sec. IV-B);
@@ -174,71 +303,218 @@ __device__ void record_fit(SolveState st, double beta, double gamma) {
 }
 
 
-// Single CTA (1024 threads).  Shared: GW (R*R doubles) + c (R doubles).
-__global__ void __launch_bounds__(1024)
-k_finalize(float* __restrict__ H, long long In, int R, int N, int n, int next_mode,
-           int nblocks, int is_last, int init, SolveState st, float* __restrict__ U) {
+// Column sums over the row blocks' partials: part(b) = W^T W of block b, pitch
+// doubles apart.  A warp per output over many blocks (fixed butterfly), a
+// thread per output over few.
+constexpr int kFewBlocks = 16;
+__device__ __forceinline__ double sum_blocks_thread(const double* p, long long pitch, int nblocks) {
+  double s = 0.0;
+#pragma unroll 4
+  for (int b = 0; b < nblocks; ++b) s += p[b * pitch];
+  return s;
+}
+__device__ __forceinline__ double sum_blocks_warp(const double* p, long long pitch, int nblocks) {
+  double s = 0.0;
+#pragma unroll 4
+  for (int b = threadIdx.x & 31; b < nblocks; b += 32) s += p[b * pitch];
+  return warp_sum_d(s);
+}
+
+// The rest of a mode update after k_hals_gram, over gridDim.x CTAs: every CTA
+// forms all column norms from the partials' diagonals (the same bits in each),
+// scales its share of the rows of H (and of the ADMM duals U) and owns a slice
+// of the R x R outputs G_n and S of the next mode; at n = N the CTAs' shares of
+// gamma are added in CTA order by the last one to arrive (ticket st.flags[8]),
+// which records the fit.  gscr: gridDim.x doubles of scratch.
+// (One CTA for all of it took 500 us for 40,000 rows at R = 16 on a GB300.)
+constexpr int kFinishThreads = 256;
+constexpr int kFinishMax = 304;
+
+__global__ void __launch_bounds__(kFinishThreads)
+k_finish(float* __restrict__ H, long long In, int R, int N, int n, int next_mode, int nblocks,
+         int is_last, SolveState st, float* __restrict__ U, double* __restrict__ gscr) {
   pdl_wait();
   pdl_trigger();
   if (st.flags[0]) return;
-  extern __shared__ double dsm[];
-  double* GW = dsm;          // R x R
-  double* c = GW + R * R;    // R
-  __shared__ double red[32];
-  const int R2 = R * R;
-  const int tid = threadIdx.x;
-
-  for (int t = tid; t < R2; t += blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += st.gram_part[(long long)b * (R2 + 1) + t];
-    GW[t] = s;
-  }
-  __syncthreads();
-  for (int r = tid; r < R; r += blockDim.x) {
-    double v = sqrt(GW[r * R + r]);
-    c[r] = v;
-    if (init) st.lam[r] *= v;
-    else st.lam[r] = v;
-  }
-  __syncthreads();
   __shared__ double cinv[kMaxRank];
-  for (int r = tid; r < R; r += blockDim.x) cinv[r] = c[r] > 0.0 ? 1.0 / c[r] : 0.0;
-  __syncthreads();
-  double* Gn = st.G + (long long)n * R2;
-  for (int t = tid; t < R2; t += blockDim.x) {
-    const int a = t / R, b = t % R;
-    Gn[t] = GW[t] * cinv[a] * cinv[b];
-  }
-  for (long long t = tid; t < In * R; t += blockDim.x) {
-    const int r = (int)(t % R);
-    H[t] = c[r] > 0.0 ? H[t] / (float)c[r] : 0.0f;
-    if (U) U[t] = c[r] > 0.0 ? U[t] / (float)c[r] : 0.0f;  // ADMM dual, same frame as H
-  }
-  if (is_last) {
-    // gamma = lam^T (S * G_N) lam = sum_ab S_ab (W^T W)_ab
-    const double* Sn = st.S + (long long)n * R2;
-    double g = 0.0;
-    for (int t = tid; t < R2; t += blockDim.x) g += Sn[t] * GW[t];
-    for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-    if ((tid & 31) == 0) red[tid >> 5] = g;
-    __syncthreads();
-    if (tid == 0) {
-      double gamma = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) gamma += red[w];
-      double beta = 0.0;
-      for (int b = 0; b < nblocks; ++b) beta += st.gram_part[(long long)b * (R2 + 1) + R2];
-      record_fit(st, beta, gamma);
+  __shared__ float cf[kMaxRank];
+  __shared__ double red[kFinishThreads / 32];
+  __shared__ int last_sh;
+  constexpr int T = kFinishThreads;
+  const int R2 = R * R, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const long long pitch = R2 + 1;
+  const bool few = nblocks <= kFewBlocks;
+  auto column = [&](int r, double g) {
+    const double v = sqrt(g);
+    cinv[r] = v > 0.0 ? 1.0 / v : 0.0;
+    cf[r] = (float)v;
+    if (blockIdx.x == 0) st.lam[r] = v;
+  };
+  if (few) {
+    for (int r = tid; r < R; r += T) column(r, sum_blocks_thread(st.gram_part + r * R + r, pitch, nblocks));
+  } else {
+    for (int r = warp; r < R; r += T / 32) {
+      const double g = sum_blocks_warp(st.gram_part + r * R + r, pitch, nblocks);
+      if (lane == 0) column(r, g);
     }
   }
   __syncthreads();
-  // S for the next mode: Hadamard of every Gram but next_mode's (float64)
-  if (next_mode >= 0) {
-    for (int t = tid; t < R2; t += blockDim.x) {
-      double s = 1.0;
-      for (int k = 0; k < N; ++k)
-        if (k != next_mode) s *= st.G[(long long)k * R2 + t];
-      st.S[(long long)next_mode * R2 + t] = s;
-      st.S32[t] = (float)s;
+  // this CTA's slice of G_n and of S for the next mode: Hadamard of every Gram
+  // but next_mode's, in mode order (mode n's is the new one)
+  const int ssz = (R2 + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int s0 = min(R2, (int)blockIdx.x * ssz), s1 = min(R2, s0 + ssz);
+  double* Gn = st.G + (long long)n * R2;
+  double gamma = 0.0;
+  auto output = [&](int e, double g) {
+    const double gn = g * cinv[e / R] * cinv[e % R];
+    Gn[e] = gn;
+    // gamma = lam^T (S * G_N) lam = sum_ab S_ab (W^T W)_ab
+    if (is_last) gamma += st.S[(long long)n * R2 + e] * g;
+    double s = 1.0;
+    for (int k = 0; k < N; ++k)
+      if (k != next_mode) s *= k == n ? gn : st.G[(long long)k * R2 + e];
+    st.S[(long long)next_mode * R2 + e] = s;
+    st.S32[e] = (float)s;
+  };
+  if (few) {
+    for (int e = s0 + tid; e < s1; e += T) output(e, sum_blocks_thread(st.gram_part + e, pitch, nblocks));
+  } else {
+    for (int e = s0 + warp; e < s1; e += T / 32) {
+      const double g = sum_blocks_warp(st.gram_part + e, pitch, nblocks);
+      if (lane == 0) output(e, g);
+    }
+  }
+  // this CTA's share of H = W / lambda
+  const long long tot = In * R, stride = (long long)gridDim.x * T;
+  for (long long t = (long long)blockIdx.x * T + tid; t < tot; t += stride) {
+    const float c = cf[t % R];
+    H[t] = c > 0.0f ? H[t] / c : 0.0f;
+    if (U) U[t] = c > 0.0f ? U[t] / c : 0.0f;  // ADMM dual, same frame as H
+  }
+  if (is_last) {
+    gamma = warp_sum_d(gamma);
+    if (lane == 0) red[warp] = gamma;
+    __syncthreads();
+    if (tid == 0) {
+      double g = 0.0;
+      for (int w = 0; w < T / 32; ++w) g += red[w];
+      gscr[blockIdx.x] = g;
+      __threadfence();
+      last_sh = atomicAdd(&st.flags[8], 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last_sh && warp == 0) {
+      __threadfence();
+      const double g = sum_blocks_warp(gscr, 1, gridDim.x);
+      const double beta = sum_blocks_warp(st.gram_part + R2, pitch, nblocks);
+      if (lane == 0) {
+        st.flags[8] = 0;  // ticket reset for the next launch
+        record_fit(st, beta, g);
+      }
+    }
+  }
+}
+
+// ---- initialisation of a solve (Alg. 3): every factor normalised, the norms
+// folded into lambda, the Grams, S for mode 1 and alpha.  Two launches after the
+// tensor's sum of squares: the Gram partials of every mode at once, then all the
+// rest.  (A Gram and a single-CTA finalise per mode, a serial sum of alpha's
+// partials and a memset per dual took 100 to 500 us per solve on a GB300.)
+struct InitArgs {
+  int N, R;
+  float* H[kMaxModes];
+  float* U[kMaxModes];
+  long long rows[kMaxModes];
+  int first[kMaxModes + 1];  // first partial of each mode (and the total)
+  double* part[kMaxModes];   // partial b of mode n at part[n] + b (R^2 + 1)
+};
+
+template <int RMAX>
+__global__ void __launch_bounds__(kHalsThreads) k_init_gram(const __grid_constant__ InitArgs a) {
+  extern __shared__ __align__(16) float sm[];
+  int n = 0;
+  while ((int)blockIdx.x >= a.first[n + 1]) ++n;
+  const int b = blockIdx.x - a.first[n], nb = a.first[n + 1] - a.first[n];
+  rows_block<RMAX>(a.H[n], nullptr, a.rows[n], a.R, nullptr, nullptr,
+                   a.part[n] + (long long)b * (a.R * a.R + 1), 0, b, nb, sm, false);
+}
+
+__global__ void __launch_bounds__(kFinishThreads)
+k_init_finish(const __grid_constant__ InitArgs a, SolveState st, double tol,
+              const double* __restrict__ alpha_part, int nalpha) {
+  extern __shared__ double dsm[];
+  double* cn = dsm;                                       // N x R column norms
+  double* cinv = cn + a.N * a.R;                          // and their reciprocals
+  float* cf = reinterpret_cast<float*>(cinv + a.N * a.R);
+  constexpr int T = kFinishThreads;
+  const int N = a.N, R = a.R, R2 = R * R, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  bool few = true;
+  for (int n = 0; n < N; ++n) few = few && a.first[n + 1] - a.first[n] <= kFewBlocks;
+  auto column = [&](int x, double g) {
+    const double v = sqrt(g);
+    cn[x] = v;
+    cinv[x] = v > 0.0 ? 1.0 / v : 0.0;
+    cf[x] = (float)v;
+  };
+  if (few) {
+    for (int x = tid; x < N * R; x += T) {
+      const int n = x / R, r = x - n * R;
+      column(x, sum_blocks_thread(a.part[n] + r * R + r, R2 + 1, a.first[n + 1] - a.first[n]));
+    }
+  } else {
+    for (int x = warp; x < N * R; x += T / 32) {
+      const int n = x / R, r = x - n * R;
+      const double g = sum_blocks_warp(a.part[n] + r * R + r, R2 + 1, a.first[n + 1] - a.first[n]);
+      if (lane == 0) column(x, g);
+    }
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    for (int r = tid; r < R; r += T) {
+      double l = 1.0;
+      for (int n = 0; n < N; ++n) l *= cn[n * R + r];
+      st.lam[r] = l;
+    }
+    if (warp == 0) {
+      const double alpha = sum_blocks_warp(alpha_part, 1, nalpha);
+      if (lane == 0) {
+        st.scalars[0] = alpha;
+        st.scalars[4] = tol;
+        st.scalars[5] = 0.0;
+      }
+      if (lane < 16) st.flags[lane] = 0;
+    }
+  }
+  // Grams of the normalised factors, and S for mode 1
+  const int ssz = (R2 + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int s0 = min(R2, (int)blockIdx.x * ssz), s1 = min(R2, s0 + ssz);
+  const int per = few ? 1 : 32;
+  for (int e = s0 + tid / per; e < s1; e += T / per) {
+    double s = 1.0;
+    for (int n = 0; n < N; ++n) {
+      const double* p = a.part[n] + e;
+      const int nb = a.first[n + 1] - a.first[n];
+      const double g = (few ? sum_blocks_thread(p, R2 + 1, nb) : sum_blocks_warp(p, R2 + 1, nb)) *
+                       cinv[n * R + e / R] * cinv[n * R + e % R];
+      if (few || lane == 0) st.G[(long long)n * R2 + e] = g;
+      if (n > 0) s *= g;
+    }
+    if (few || lane == 0) {
+      st.S[e] = s;
+      st.S32[e] = (float)s;
+    }
+  }
+  // rows of every factor; the ADMM duals start at zero
+  const long long stride = (long long)gridDim.x * T;
+  for (int n = 0; n < N; ++n) {
+    const long long tot = a.rows[n] * R;
+    float* H = a.H[n];
+    float* U = a.U[n];
+    const float* c = cf + n * R;
+    for (long long t = (long long)blockIdx.x * T + tid; t < tot; t += stride) {
+      const float v = c[t % R];
+      H[t] = v > 0.0f ? H[t] / v : 0.0f;
+      U[t] = 0.0f;
     }
   }
 }
@@ -1589,30 +1865,6 @@ k_apg_rows(float* __restrict__ W, const float* __restrict__ M, int In, int R,
   }
 }
 
-__global__ void k_solve_reset(SolveState st, int R, double tol) {
-  for (int r = threadIdx.x; r < R; r += blockDim.x) st.lam[r] = 1.0;
-  if (threadIdx.x == 0) {
-    st.flags[0] = 0;
-    st.flags[1] = 0;
-    st.flags[2] = 0;
-    st.flags[3] = 0;
-    st.flags[8] = 0;
-    st.scalars[4] = tol;
-    st.scalars[5] = 0.0;
-  }
-}
-
-__global__ void k_compute_S(SolveState st, int N, int R, int mode) {
-  const int R2 = R * R;
-  for (int t = threadIdx.x; t < R2; t += blockDim.x) {
-    double s = 1.0;
-    for (int k = 0; k < N; ++k)
-      if (k != mode) s *= st.G[(long long)k * R2 + t];
-    st.S[(long long)mode * R2 + t] = s;
-    st.S32[t] = (float)s;
-  }
-}
-
 struct ResidualArgs {
   int N;
   long long dims[kMaxModes];
@@ -1672,28 +1924,36 @@ __global__ void k_explicit_residual(const float* __restrict__ X, ResidualArgs a,
 }
 
 __global__ void k_sum_pairs(const double* __restrict__ partials, int n, double* out) {
+  const double s = sum_blocks_warp(partials, 2, n), sx = sum_blocks_warp(partials + 1, 2, n);
   if (threadIdx.x == 0) {
-    double s = 0.0, sx = 0.0;
-    for (int i = 0; i < n; ++i) {
-      s += partials[2 * i];
-      sx += partials[2 * i + 1];
-    }
     out[0] = s;
     out[1] = sx;
   }
 }
 
-size_t hals_smem(int R) {
-  return (size_t)R * R * sizeof(float) + (size_t)kRowsPerBlock * (R + 1) * sizeof(float);
+int rows_rmax(int R) { return R <= 16 ? 16 : (R <= 32 ? 32 : (R <= 64 ? 64 : 128)); }
+
+size_t rows_smem(int R, bool sweep) {
+  const int rmax = rows_rmax(R);
+  return (size_t)(kRowsPerBlock * (rmax + 4) + (sweep ? R * rmax : 0)) * sizeof(float);
 }
 
 }  // namespace
 
 cudaError_t kernel_attributes_init() {
-  cudaError_t e = cudaFuncSetAttribute(k_hals_gram, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       200 * 1024);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_finalize, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  cudaError_t e = cudaSuccess;
+  const int rows = (int)rows_smem(kMaxRank, true);
+  auto opt_in = [&](auto k) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, rows);
+  };
+  opt_in(k_hals_gram<16>);
+  opt_in(k_hals_gram<32>);
+  opt_in(k_hals_gram<64>);
+  opt_in(k_hals_gram<128>);
+  opt_in(k_init_gram<16>);
+  opt_in(k_init_gram<32>);
+  opt_in(k_init_gram<64>);
+  opt_in(k_init_gram<128>);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_update_multi<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)multi_smem<16>());
@@ -1716,14 +1976,27 @@ cudaError_t kernel_attributes_init() {
   return e;
 }
 
-int hals_gram_blocks(int64_t In) { return (int)((In + kRowsPerBlock - 1) / kRowsPerBlock); }
+// row blocks of k_hals_gram: one per 64 rows, at most two per SM (of 152),
+// which then take several in turn
+int hals_gram_blocks(int64_t In) {
+  return (int)std::min<int64_t>((In + kRowsPerBlock - 1) / kRowsPerBlock, 304);
+}
+
+namespace {
+cudaError_t launch_rows(float* H, const float* M, int64_t In, int R, SolveState st, int do_hals,
+                        cudaStream_t stream) {
+  const int rmax = rows_rmax(R);
+  auto k = rmax == 16 ? k_hals_gram<16>
+                      : (rmax == 32 ? k_hals_gram<32> : (rmax == 64 ? k_hals_gram<64> : k_hals_gram<128>));
+  return launch_kernel(k, dim3(hals_gram_blocks(In)), dim3(kHalsThreads), rows_smem(R, do_hals == 1),
+                       stream, H, M, (long long)In, R, (const float*)st.S32, (const double*)st.lam,
+                       st.gram_part, (const int*)st.flags, do_hals);
+}
+}  // namespace
 
 cudaError_t launch_hals_gram(float* H, const float* M, int64_t In, int R, SolveState st,
                              cudaStream_t stream) {
-  size_t smem = hals_smem(R);
-  return launch_kernel(k_hals_gram, dim3(hals_gram_blocks(In)), dim3(kHalsThreads), smem, stream,
-                       H, M, (long long)In, R, st.S32, (const double*)st.lam,
-                       st.gram_part, (const int*)st.flags, 1);
+  return launch_rows(H, M, In, R, st, 1, stream);
 }
 
 cudaError_t launch_bpp_rows(float* H, const float* M, int64_t In, int R, SolveState st,
@@ -1740,9 +2013,7 @@ cudaError_t launch_bpp_update(float* H, const float* M, int64_t In, int R, Solve
   cudaError_t e = launch_bpp_rows(H, M, In, R, st, num_sms, stream);
   if (e != cudaSuccess) return e;
   // Gram partials and <M, W> of the new W (no sweep)
-  return launch_kernel(k_hals_gram, dim3(hals_gram_blocks(In)), dim3(kHalsThreads), hals_smem(R),
-                       stream, H, M, (long long)In, R, st.S32, (const double*)st.lam,
-                       st.gram_part, (const int*)st.flags, 2);
+  return launch_rows(H, M, In, R, st, 2, stream);
 }
 
 cudaError_t launch_admm_rows(float* H, float* U, const float* M, int64_t In, int R, int iters,
@@ -1759,9 +2030,7 @@ cudaError_t launch_admm_update(float* H, float* U, const float* M, int64_t In, i
                                SolveState st, cudaStream_t stream) {
   cudaError_t e = launch_admm_rows(H, U, M, In, R, iters, st, stream);
   if (e != cudaSuccess) return e;
-  return launch_kernel(k_hals_gram, dim3(hals_gram_blocks(In)), dim3(kHalsThreads), hals_smem(R),
-                       stream, H, M, (long long)In, R, st.S32, (const double*)st.lam,
-                       st.gram_part, (const int*)st.flags, 2);
+  return launch_rows(H, M, In, R, st, 2, stream);
 }
 
 cudaError_t launch_apg_rows(float* H, const float* M, int64_t In, int R, int iters,
@@ -1778,17 +2047,12 @@ cudaError_t launch_apg_update(float* H, const float* M, int64_t In, int R, int i
                               SolveState st, cudaStream_t stream) {
   cudaError_t e = launch_apg_rows(H, M, In, R, iters, st, stream);
   if (e != cudaSuccess) return e;
-  return launch_kernel(k_hals_gram, dim3(hals_gram_blocks(In)), dim3(kHalsThreads), hals_smem(R),
-                       stream, H, M, (long long)In, R, st.S32, (const double*)st.lam,
-                       st.gram_part, (const int*)st.flags, 2);
+  return launch_rows(H, M, In, R, st, 2, stream);
 }
 
 cudaError_t launch_gram_only(const float* H, int64_t In, int R, SolveState st,
                              cudaStream_t stream) {
-  size_t smem = hals_smem(R);
-  k_hals_gram<<<hals_gram_blocks(In), kHalsThreads, smem, stream>>>(
-      const_cast<float*>(H), nullptr, In, R, st.S32, st.lam, st.gram_part, st.flags, 0);
-  return cudaGetLastError();
+  return launch_rows(const_cast<float*>(H), nullptr, In, R, st, 0, stream);
 }
 
 // H(i, r) *= inv(r) for `rows` rows of R columns (row-major).
@@ -1808,7 +2072,13 @@ cudaError_t launch_scale_columns(float* H, int64_t rows, int R, const float* inv
   return cudaGetLastError();
 }
 
-bool multi_update_ok(int64_t In, int R) { return In <= kMultiMaxRows && R <= 64; }
+// k_update_multi's last CTA scales every row, k_finish's CTAs share them at the
+// price of a second launch: on a GB300 the two are level at about 131,072 factor
+// elements (4096 x 32: 80 us per outer iteration either way; 2048 x 16: 53
+// against 62, 16384 x 32: 125 against 84)
+bool multi_update_ok(int64_t In, int R) {
+  return In <= kMultiMaxRows && R <= 64 && In * R < 131072;
+}
 
 // partial scratch needed by the multi-CTA update (floats)
 size_t multi_update_scratch(int64_t In, int R) {
@@ -1858,22 +2128,65 @@ cudaError_t launch_update_cluster(float* H, const float* M, int64_t In, int R, i
   }
 }
 
-cudaError_t launch_finalize(float* H, int64_t In, int R, int N, int n, int next_mode,
-                            int nblocks, int is_last, int init, double tol, SolveState st,
-                            cudaStream_t stream, float* U) {
-  (void)tol;
-  size_t smem = ((size_t)R * R + R) * sizeof(double);
-  return launch_kernel(k_finalize, dim3(1), dim3(1024), smem, stream, H, (long long)In, R, N, n,
-                       next_mode, nblocks, is_last, init, st, U);
+cudaError_t launch_finish(float* H, int64_t In, int R, int N, int n, int next_mode, int is_last,
+                          SolveState st, double* gscr, cudaStream_t stream, float* U) {
+  // about 4096 row elements per CTA, and enough CTAs for the R x R outputs
+  const int64_t want = std::max<int64_t>(((int64_t)In * R + 4095) / 4096, ((int64_t)R * R + 511) / 512);
+  const int grid = (int)std::min<int64_t>(want, kFinishMax);
+  return launch_kernel(k_finish, dim3(grid), dim3(kFinishThreads), 0, stream, H, (long long)In, R, N,
+                       n, next_mode, hals_gram_blocks(In), is_last, st, U, gscr);
 }
 
-cudaError_t launch_solve_reset(SolveState st, int R, double tol, cudaStream_t stream) {
-  k_solve_reset<<<1, 128, 0, stream>>>(st, R, tol);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_compute_S(SolveState st, int N, int R, int mode, cudaStream_t stream) {
-  k_compute_S<<<1, 1024, 0, stream>>>(st, N, R, mode);
+cudaError_t launch_solve_init(int N, const int64_t* dims, int R, float* const* H, float* const* U,
+                              double tol, const double* alpha_part, int nalpha, SolveState st,
+                              float* scratch, size_t scratch_floats, cudaStream_t stream) {
+  InitArgs a;
+  memset(&a, 0, sizeof a);
+  a.N = N;
+  a.R = R;
+  int blocks[kMaxModes], total = 0, most = 1;
+  for (int n = 0; n < N; ++n) {
+    a.H[n] = H[n];
+    a.U[n] = U[n];
+    a.rows[n] = dims[n];
+    blocks[n] = std::min(hals_gram_blocks(dims[n]), 152);
+    most = std::max(most, hals_gram_blocks(dims[n]));
+    total += blocks[n];
+  }
+  // the partials go where there is room: the split-K scratch, else the partials
+  // of one mode update with the blocks cut to fit, else one block per mode, mode
+  // 1's there and the others' in their (later) S, which the last kernel of the
+  // initialisation writes for mode 1 alone
+  const size_t pitch = (size_t)R * R + 1;
+  double* base = reinterpret_cast<double*>(scratch);
+  bool spread = false;
+  if (total * pitch > scratch_floats / 2) {
+    base = st.gram_part;
+    int sum = 0;
+    for (int n = 0; n < N; ++n) {
+      blocks[n] = std::max(1, (int)((int64_t)blocks[n] * most / total));
+      sum += blocks[n];
+    }
+    if (sum > most) {
+      for (int n = 0; n < N; ++n) blocks[n] = 1;
+      spread = N > most;
+    }
+  }
+  for (int n = 0; n < N; ++n) {
+    a.part[n] = spread && n > 0 ? st.S + (size_t)n * R * R : base;
+    base += blocks[n] * pitch;
+  }
+  for (int n = 0; n < N; ++n) a.first[n + 1] = a.first[n] + blocks[n];
+  for (int n = N + 1; n <= kMaxModes; ++n) a.first[n] = a.first[N];
+  const int rmax = rows_rmax(R);
+  auto k = rmax == 16 ? k_init_gram<16>
+                      : (rmax == 32 ? k_init_gram<32> : (rmax == 64 ? k_init_gram<64> : k_init_gram<128>));
+  k<<<a.first[N], kHalsThreads, rows_smem(R, false), stream>>>(a);
+  int64_t elems = 0;
+  for (int n = 0; n < N; ++n) elems += dims[n] * R;
+  const int64_t want = std::max<int64_t>((elems + 4095) / 4096, ((int64_t)R * R + 511) / 512);
+  const int grid = (int)std::min<int64_t>(want, kFinishMax);
+  k_init_finish<<<grid, kFinishThreads, (size_t)N * R * 20, stream>>>(a, st, tol, alpha_part, nalpha);
   return cudaGetLastError();
 }
 
