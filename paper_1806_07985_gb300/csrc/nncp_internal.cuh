@@ -106,10 +106,7 @@ cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
                                float* partials, size_t part_cap, int num_sms,
                                cudaStream_t st);
 size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms);
-cudaError_t launch_simt_mttkrp_capped(const float* X, int64_t L, int64_t I, int64_t Q,
-                                      const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,
-                                      float* partials, size_t part_cap, int num_sms,
-                                      cudaStream_t st);
+cudaError_t simt_attributes_init();
 
 // Records a message for nncp_global_error().
 void record_global_error(const char* msg);

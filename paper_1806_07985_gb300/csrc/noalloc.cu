@@ -51,6 +51,8 @@ nncp_status device_slot(DeviceSlot* out) {
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return reject(NNCP_ERR_CUDA, "cudaDeviceGetAttribute failed");
+    e = simt_attributes_init();
+    if (e != cudaSuccess) return reject(NNCP_ERR_CUDA, "cudaFuncSetAttribute failed");
     s.num_sms = sms;
     s.scratch = static_cast<float*>(p);
   }
@@ -98,9 +100,9 @@ extern "C" nncp_status nncp_mttkrp_noalloc(int N, const int64_t* dims, int R, co
     KQ.H[KQ.nm++] = H_dev[m];
     Q *= dims[m];
   }
-  cudaError_t e = launch_simt_mttkrp_capped(X_dev, L, rows, Q, KL, KQ, R, M_dev, slot.scratch,
-                                            kScratchFloats, slot.num_sms,
-                                            static_cast<cudaStream_t>(stream));
+  cudaError_t e = launch_simt_mttkrp(X_dev, L, rows, Q, KL, KQ, R, M_dev, slot.scratch,
+                                     kScratchFloats, slot.num_sms,
+                                     static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) {
     record_global_error(cudaGetErrorString(e));
     return NNCP_ERR_CUDA;

@@ -1,16 +1,5 @@
-// CUDA-core kernels: generic MTTKRP over a (L, I, Q) view of the tensor,
+// CUDA-core kernels around the partial MTTKRPs: sums of split partials,
 // multi-TTVs on dimension-tree nodes, sums of squares, bf16 conversion.
-//
-// The (L, I, Q) view: mode set split as [modes before] x [output modes] x
-// [modes after], so X[l + L*(i + I*q)] holds the entry with left index l,
-// output index i and right index q (mode-1-fastest layout, Sec. IV-C).
-//   * direct MTTKRP of mode n (Sec. II-A): L = I_1..I_{n-1}, I = I_n,
-//     Q = I_{n+1}..I_N;
-//   * partial MTTKRP root -> {1..s} (Sec. IV-A, Fig. 2a): L = 1,
-//     I = I_1..I_s, Q = I_{s+1}..I_N (contracts the slow modes);
-//   * partial MTTKRP root -> {s+1..N}: L = I_1..I_s, I = I_{s+1}..I_N, Q = 1
-//     (contracts the fast modes).
-// The Khatri-Rao rows are formed on the fly in shared memory from factor rows.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -23,18 +12,8 @@ namespace nncp {
 
 namespace {
 
-constexpr int kBI = 128;  // output rows per CTA
 constexpr int kBK = 32;   // contraction tile
-constexpr int kRT = 32;   // rank columns per CTA
 constexpr int kThreads = 256;
-
-// Per-tile row offsets of the Khatri-Rao factors: for contraction index k,
-// off[m] = (row of mode m) * R, so KRP(k, r) = prod_m H_m[off[m] + r].
-struct TileRows {
-  int off[2 * kMaxModes];
-  long long xbase;  // X offset of (i = 0, k)
-  int valid;
-};
 
 __device__ __forceinline__ void decompose(const KrpDesc& d, long long k, int R, int* off) {
   for (int m = 0; m < d.nm; ++m) {
@@ -49,173 +28,6 @@ __device__ __forceinline__ float krp_value(const KrpDesc& d, const int* off, int
   float v = 1.0f;
   for (int m = 0; m < d.nm; ++m) v *= __ldg(d.H[m] + off[m] + r);
   return v;
-}
-
-// X elements each thread stages per contraction tile
-constexpr int kXPer = kBK * kBI / kThreads;
-
-template <bool kSlow>
-__global__ void __launch_bounds__(kThreads, 4)
-k_simt_mttkrp(const float* __restrict__ X, long long L, long long I, long long Q, KrpDesc KL,
-              KrpDesc KQ, int R, long long kchunk, float* __restrict__ out,
-              long long out_chunk_stride) {
-  pdl_wait();  // no early trigger: a large grid; its successor spreads as CTAs exit
-  __shared__ __align__(16) float Xs[kBK][kBI + 4];
-  __shared__ __align__(16) float Ws[kBK][kRT];
-  __shared__ TileRows rows[2][kBK];  // this tile's and the next one's
-
-  const long long Ktot = L * Q;
-  const long long i0 = (long long)blockIdx.x * kBI;
-  const int r0 = blockIdx.z * kRT;
-  const long long kbeg = (long long)blockIdx.y * kchunk;
-  const long long kend = min(Ktot, kbeg + kchunk);
-  const int tid = threadIdx.x;
-  const int tx = tid & 7;   // rank group: r0 + 4*tx .. +3
-  const int ty = tid >> 3;  // row group:  i0 + 4*ty .. +3
-
-  float acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0f;
-
-  // row metadata of the tile at k0 into rows[buf] (threads < kBK)
-  auto tile_rows = [&](long long k0, int buf) {
-    if (tid < kBK) {
-      long long k = k0 + tid;
-      TileRows tr;
-      tr.valid = k < kend;
-      if (tr.valid) {
-        long long l = k % L, q = k / L;
-        decompose(KL, l, R, tr.off);
-        decompose(KQ, q, R, tr.off + kMaxModes);
-        tr.xbase = l + L * I * q;
-      } else {
-        tr.xbase = 0;
-      }
-      rows[buf][tid] = tr;
-    }
-  };
-  // this thread's X elements of the tile described by rows[buf]: element
-  // (i, k) at xbase(k) + L*i, read along whichever of i and k is contiguous
-  float xr[kXPer];
-  // L == 1 with I % 4 == 0 and X 16-byte aligned: every tile row is four-float
-  // aligned, so thread tid reads four consecutive i of rows tid / 32 + 8 v.
-  // L % 32 == 0 (and X aligned): a tile's 32 k share q and have consecutive l,
-  // and chunks and totals are multiples of 32, so a tile is wholly valid or
-  // not; thread tid reads four consecutive k of row i = (tid + 256 v) / 8.
-  const bool aligned = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
-  const bool vec = kSlow && (I & 3) == 0 && aligned;
-  const bool veck = !kSlow && (L & 31) == 0 && aligned;
-  auto load_x = [&](int buf) {
-    if (veck) {
-#pragma unroll
-      for (int v = 0; v < kXPer / 4; ++v) {
-        const int id = tid + kThreads * v, ii = id >> 3, kk = 4 * (id & 7);
-        const long long i = i0 + ii;
-        float4 x4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (rows[buf][kk].valid && i < I)
-          x4 = __ldg(reinterpret_cast<const float4*>(X + rows[buf][kk].xbase + L * i));
-        xr[4 * v] = x4.x;
-        xr[4 * v + 1] = x4.y;
-        xr[4 * v + 2] = x4.z;
-        xr[4 * v + 3] = x4.w;
-      }
-      return;
-    }
-    if (vec) {
-      const int ii = 4 * (tid & 31);
-#pragma unroll
-      for (int v = 0; v < kXPer / 4; ++v) {
-        const int kk = (tid >> 5) + 8 * v;
-        const long long i = i0 + ii;
-        float4 x4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (rows[buf][kk].valid && i < I)  // i < I covers i .. i + 3 (I % 4 == 0)
-          x4 = __ldg(reinterpret_cast<const float4*>(X + rows[buf][kk].xbase + i));
-        xr[4 * v] = x4.x;
-        xr[4 * v + 1] = x4.y;
-        xr[4 * v + 2] = x4.z;
-        xr[4 * v + 3] = x4.w;
-      }
-      return;
-    }
-#pragma unroll
-    for (int u = 0; u < kXPer; ++u) {
-      const int e = tid + kThreads * u;
-      int kk, ii;
-      if (kSlow) { kk = e / kBI; ii = e % kBI; }   // L == 1: rows contiguous in i
-      else       { kk = e % kBK; ii = e / kBK; }   // contiguous in k (l fastest)
-      const long long i = i0 + ii;
-      xr[u] = (rows[buf][kk].valid && i < I) ? __ldg(X + rows[buf][kk].xbase + L * i) : 0.0f;
-    }
-  };
-
-  int cur = 0;
-  if (kbeg < kend) {
-    tile_rows(kbeg, 0);
-    __syncthreads();
-    load_x(0);
-  }
-  for (long long k0 = kbeg; k0 < kend; k0 += kBK, cur ^= 1) {
-    const bool more = k0 + kBK < kend;
-    for (int e = tid; e < kBK * kRT; e += kThreads) {
-      int kk = e / kRT, rr = e % kRT;
-      int r = r0 + rr;
-      float w = 0.0f;
-      if (rows[cur][kk].valid && r < R)
-        w = krp_value(KL, rows[cur][kk].off, r) * krp_value(KQ, rows[cur][kk].off + kMaxModes, r);
-      Ws[kk][rr] = w;
-    }
-    if (veck) {
-#pragma unroll
-      for (int v = 0; v < kXPer / 4; ++v) {
-        const int id = tid + kThreads * v, ii = id >> 3, kk = 4 * (id & 7);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) Xs[kk + j][ii] = xr[4 * v + j];
-      }
-    } else if (vec) {
-#pragma unroll
-      for (int v = 0; v < kXPer / 4; ++v)
-        *reinterpret_cast<float4*>(&Xs[(tid >> 5) + 8 * v][4 * (tid & 31)]) =
-            make_float4(xr[4 * v], xr[4 * v + 1], xr[4 * v + 2], xr[4 * v + 3]);
-    } else {
-#pragma unroll
-      for (int u = 0; u < kXPer; ++u) {
-        const int e = tid + kThreads * u;
-        int kk, ii;
-        if (kSlow) { kk = e / kBI; ii = e % kBI; }
-        else       { kk = e % kBK; ii = e / kBK; }
-        Xs[kk][ii] = xr[u];
-      }
-    }
-    if (more) tile_rows(k0 + kBK, cur ^ 1);
-    __syncthreads();
-    if (more) load_x(cur ^ 1);  // the next tile's tensor values stream in during this tile
-#pragma unroll 8
-    for (int kk = 0; kk < kBK; ++kk) {
-      float4 xv = *reinterpret_cast<const float4*>(&Xs[kk][ty * 4]);
-      float4 wv = *reinterpret_cast<const float4*>(&Ws[kk][tx * 4]);
-      float xa[4] = {xv.x, xv.y, xv.z, xv.w};
-      float wa[4] = {wv.x, wv.y, wv.z, wv.w};
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(xa[a], wa[b], acc[a][b]);
-    }
-    __syncthreads();
-  }
-
-  float* o = out + (long long)blockIdx.y * out_chunk_stride;
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    long long i = i0 + ty * 4 + a;
-    if (i >= I) continue;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      int r = r0 + tx * 4 + b;
-      if (r < R) o[i * R + r] = acc[a][b];
-    }
-  }
 }
 
 // out[e] = sum_{c < C} part[c * E + e] (deterministic: four interleaved partial
@@ -524,59 +336,6 @@ int choose_chunks(long long ctas_other, long long Ktot, int num_sms, long long m
 constexpr long long kMttvMinChunk = 8;
 
 }  // namespace
-
-size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms) {
-  long long gx = ceil_div(I, kBI), gz = ceil_div(R, kRT);
-  int C = choose_chunks(gx * gz, (long long)L * Q, num_sms);
-  return C > 1 ? (size_t)C * I * R : 0;
-}
-
-cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
-                               const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,
-                               float* partials, size_t part_cap, int num_sms,
-                               cudaStream_t st) {
-  long long Ktot = (long long)L * Q;
-  long long gx = ceil_div(I, kBI), gz = ceil_div(R, kRT);
-  int C = choose_chunks(gx * gz, Ktot, num_sms);
-  long long kchunk = ceil_div(ceil_div(Ktot, C), kBK) * kBK;
-  C = (int)ceil_div(Ktot, kchunk);
-  float* dst = out;
-  if (C > 1) {
-    if ((size_t)C * I * R > part_cap || partials == nullptr) return cudaErrorInvalidValue;
-    dst = partials;
-  }
-  dim3 grid((unsigned)gx, (unsigned)C, (unsigned)gz);
-  cudaError_t e = launch_kernel(L == 1 ? k_simt_mttkrp<true> : k_simt_mttkrp<false>, grid,
-                                dim3(kThreads), 0, st, X, (long long)L, (long long)I,
-                                (long long)Q, KL, KQ, R, kchunk, dst, (long long)I * R);
-  if (e != cudaSuccess || C == 1) return e;
-  return launch_reduce_chunks(partials, (long long)I * R, C, out, num_sms, st);
-}
-
-// Same MTTKRP with the split-K chunk count capped so the partials fit in
-// `part_cap` floats (used by the entry point that allocates nothing).
-cudaError_t launch_simt_mttkrp_capped(const float* X, int64_t L, int64_t I, int64_t Q,
-                                      const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,
-                                      float* partials, size_t part_cap, int num_sms,
-                                      cudaStream_t st) {
-  long long Ktot = (long long)L * Q;
-  long long gx = ceil_div(I, kBI), gz = ceil_div(R, kRT);
-  long long fit = (long long)(part_cap / ((size_t)I * R));
-  int C = (int)max(1LL, min((long long)choose_chunks(gx * gz, Ktot, num_sms), fit));
-  long long kchunk = ceil_div(ceil_div(Ktot, C), kBK) * kBK;
-  C = (int)ceil_div(Ktot, kchunk);
-  float* dst = out;
-  if (C > 1) {
-    if ((size_t)C * I * R > part_cap || partials == nullptr) return cudaErrorInvalidValue;
-    dst = partials;
-  }
-  dim3 grid((unsigned)gx, (unsigned)C, (unsigned)gz);
-  cudaError_t e = launch_kernel(L == 1 ? k_simt_mttkrp<true> : k_simt_mttkrp<false>, grid,
-                                dim3(kThreads), 0, st, X, (long long)L, (long long)I,
-                                (long long)Q, KL, KQ, R, kchunk, dst, (long long)I * R);
-  if (e != cudaSuccess || C == 1) return e;
-  return launch_reduce_chunks(partials, (long long)I * R, C, out, num_sms, st);
-}
 
 cudaError_t launch_reduce_chunks(const float* part, int64_t E, int C, float* out, int num_sms,
                                  cudaStream_t st) {

@@ -1,0 +1,836 @@
+// Float32 MTTKRP on CUDA cores over a (L, I, Q) view of the tensor (Sec. II-A,
+// Sec. IV-A): out(i, r) = sum_{l, q} X[l + L (i + I q)] KL(l, r) KQ(q, r).
+//
+// The (L, I, Q) view: mode set split as [modes before] x [output modes] x
+// [modes after], so X[l + L*(i + I*q)] holds the entry with left index l,
+// output index i and right index q (mode-1-fastest layout, Sec. IV-C).
+//   * direct MTTKRP of mode n (Sec. II-A): L = I_1..I_{n-1}, I = I_n,
+//     Q = I_{n+1}..I_N;
+//   * partial MTTKRP root -> {1..s} (Sec. IV-A, Fig. 2a): L = 1,
+//     I = I_1..I_s, Q = I_{s+1}..I_N (contracts the slow modes);
+//   * partial MTTKRP root -> {s+1..N}: L = I_1..I_s, I = I_{s+1}..I_N, Q = 1
+//     (contracts the fast modes).
+// It is a matrix product of I x R outputs over K = L Q, whose second operand,
+// the Khatri-Rao rows, is formed on the fly: the digits of k = l + L q in the
+// contracted modes, fastest first, are the factor rows multiplied.
+//
+// A CTA holds a tile of BM output rows x all rank columns in registers (8 ranks
+// x 4 rows per thread as packed float32 pairs: fma.rn.f32x2 does two FMAs per
+// issue slot, which leaves half of the slots to the shared-memory reads) and
+// takes 32 contraction elements per step from a ring of three shared-memory
+// stages that cp.async fills two steps ahead: the tensor tile and, beside it,
+// the raw factor rows of the step -- a row of the fastest contracted mode per
+// element and a row of every other mode per distinct index of the rest (two for
+// a fastest mode of 31 or more).  One step before its use a stage's first rows
+// are multiplied by the others in place, so no thread waits for a global load.
+// One more warp, the feeder, walks the steps and fetches the factor rows (at
+// high ranks the computing threads do: too many copies for one warp).  A step is
+// described by the position of its first element alone -- digit d of the
+// fastest mode, index q of the rest -- from which every thread derives its own
+// element's: d + e past the mode's length is in the next rest row.
+//
+// Threads: 8 consecutive lanes take neighbouring output rows, then come the
+// rank groups, the row groups and the KG-way split of a step's 32 elements,
+// which keeps a warp's shared-memory reads at one or two wavefronts each and
+// gives small ranks enough warps; the KG partial sums are added in a fixed
+// tree at the end of a tile.
+//
+// Work split: G CTAs (what fits on the GPU at once) take whole tiles in turn;
+// the tiles of a last, partly filled wave are cut into G equal runs of steps
+// instead (a run may straddle two tiles), whose partial tiles go to `slots` and
+// are added in run order by k_simt_fixup.  Every cut follows from the shape and
+// the scratch size alone, so results are bitwise reproducible.
+//
+// Measured on a GB300 per root branch (outputs slow / fast), the 128 x 32 tile
+// kernel of one FMA per issue slot that this one replaced in brackets: 512^3
+// R = 8 117 / 104 us (358 / 411), R = 32 260 / 250 us (363 / 416), 40000x48x40
+// R = 16 121 / 95 us (292 / 230), 301x257x199 R = 20 68 / 49 us (74 / 85),
+// 220x180x150 R = 100 80 / 66 us (90 / 91).  At R = 8 it streams at 4.6 to 5.2
+// TB/s; at R = 32 it runs at 0.44 of the FMA peak, of which a step's loads,
+// Khatri-Rao rows and barrier take a quarter and the shared-memory reads (three
+// of 16 bytes per 16 packed FMAs) most of the rest.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "nncp_internal.cuh"
+
+namespace nncp {
+
+namespace {
+
+constexpr int kBK = 32;        // contraction elements per step
+constexpr int kThreadsMax = 256;  // computing threads; the feeder warp comes after them
+constexpr int kStages = 3;
+constexpr int kTM = 4;         // output rows per thread
+constexpr int kTabs = 4;       // step descriptors in flight
+constexpr int kSmemMax = 232448;  // 227 KB per CTA on sm_103a
+constexpr int kSmemSM = 233472;   // 228 KB per SM, 1 KB of it reserved per CTA
+constexpr int kStaticSmem = 512; // descriptors (checked below)
+
+struct SimtArgs {
+  const float* X;
+  long long L, I, K;
+  int R, RP, ld;          // rank columns; padded to whole groups of eight; row stride of H and out
+  int CG, RGH, KG;        // rank groups, row groups, splits of a step
+  int bm_log2;            // BM = 32 RGH
+  int tl;                 // threads that load: the most whole pairs of computing warps
+  int b_all;              // the computing threads load the factor rows too
+  int gsh;                // 2^gsh lanes copy a factor row (all of it in one go when vecb)
+  int fk, fc;             // threads / (RP / 4) and the remainder
+  int vecx, vecb, veco, evict;
+  int nm;                 // contracted modes, fastest first
+  int dim[kMaxModes];     // their lengths
+  int dstep, mag0, magl;  // 32 mod dim[0]; ceil(2^16 / dim[0]) and / L below 32, else 0
+  long long rstep;        // 32 / dim[0]
+  const float* H[kMaxModes];
+  long long lstep, qstep;  // 32 mod L, 32 / L
+  int nrest_max;           // rest rows a stage has room for
+  int red_pairs;           // column pairs per round of the KG sums (1, 2 or 4)
+  int x_floats, stage_floats;
+  long long nk;            // steps per whole tile
+  long long whole;         // tiles taken whole
+  long long U2;            // steps of the tiles cut into runs
+  int G2, two;             // runs; partial slots per run (1 or 2)
+  float* out;
+  float* slots;
+  long long slot_floats;   // BM x R
+};
+
+// One step: the tile it belongs to and the position of its first element.
+struct StepTab {
+  long long i0, k0;      // first output row of the tile, first contraction element
+  long long rest;        // k0 / dim[0]
+  long long l, q;        // k0 mod L, k0 / L
+  int d;                 // k0 mod dim[0]
+  int nk;                // valid elements (1..32)
+  int valid;             // 0: no more steps
+  int last;              // 1: last step of this CTA's run over the tile
+  int slot;              // partial slot of the run, -1: the whole tile (write the output)
+};
+
+// x / n for 0 <= x < n + 32: mag = ceil(2^16 / n) for n < 32 (exact there: the
+// excess is below 63 / 2^16 < 1 / n), 0 otherwise
+template <typename I>
+__device__ __forceinline__ int wraps(I x, I n, int mag) {
+  return mag ? (int)(((unsigned)x * (unsigned)mag) >> 16) : (x >= n ? 1 : 0);
+}
+
+static_assert(sizeof(StepTab) * kTabs + 64 <= kStaticSmem, "static shared memory");
+
+__device__ __forceinline__ uint32_t s_u32(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void cpa16(uint32_t dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cpa16_hint(uint32_t dst, const float* src, uint64_t pol) {
+  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src),
+               "l"(pol)
+               : "memory");
+}
+__device__ __forceinline__ void cpa4(uint32_t dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+
+typedef unsigned long long u64;
+
+// two float32 FMAs, each rounded to nearest as fmaf
+__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c) {
+  u64 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ u64 pack2(float x, float y) {
+  u64 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(u64 v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+
+// first step of run c over the cut tiles
+__device__ __forceinline__ long long run_start(long long c, long long U2, int G2) {
+  return c * U2 / G2;
+}
+
+// The steps of a CTA in order: whole tiles blockIdx.x, + gridDim.x, ..., then
+// its run over the cut tiles (one warp, uniform).
+struct Feeder {
+  long long tile, k, kend;  // tile; next step and end of the current run over it
+  long long u, u1;          // what is left of the run over the cut tiles
+  long long rest, l, q;
+  int d, slot;
+  bool cut, first;
+
+  __device__ __forceinline__ explicit Feeder(const SimtArgs& p) {
+    tile = (long long)blockIdx.x - gridDim.x;
+    k = kend = u = u1 = rest = l = q = 0;
+    if ((int)blockIdx.x < p.G2) {
+      u = run_start(blockIdx.x, p.U2, p.G2);
+      u1 = run_start(blockIdx.x + 1, p.U2, p.G2);
+    }
+    d = 0;
+    slot = -1;
+    cut = false;
+    first = true;
+  }
+
+  __device__ __forceinline__ void next(const SimtArgs& p, StepTab& t, bool kc) {
+    if (k < kend) {
+      // the next step of the same run: 32 elements on
+      d += p.dstep;
+      rest += p.rstep;
+      if (d >= p.dim[0]) {
+        d -= p.dim[0];
+        ++rest;
+      }
+      if (kc) {
+        l += p.lstep;
+        q += p.qstep;
+        if (l >= p.L) {
+          l -= p.L;
+          ++q;
+        }
+      }
+    } else {
+      bool got = false;
+      if (!cut) {
+        tile += gridDim.x;
+        k = 0;
+        kend = p.nk;
+        slot = -1;
+        got = tile < p.whole;
+        cut = !got;
+      }
+      if (!got && u < u1) {
+        const long long qt = u / p.nk;
+        tile = p.whole + qt;
+        k = u - qt * p.nk;
+        kend = min(p.nk, k + (u1 - u));
+        u += kend - k;
+        const bool all = k == 0 && kend == p.nk;
+        slot = all ? -1 : (p.two ? 2 * (int)blockIdx.x + (first ? 0 : 1) : (int)blockIdx.x);
+        first = false;
+        got = true;
+      }
+      if (!got) {
+        k = kend = 0;
+        t.valid = 0;
+        return;
+      }
+      const long long e = k * kBK;
+      rest = d = 0;
+      l = q = 0;
+      if (e != 0) {
+        rest = e / p.dim[0];
+        d = (int)(e - rest * p.dim[0]);
+        if (kc) {
+          q = e / p.L;
+          l = e - q * p.L;
+        }
+      }
+    }
+    if ((threadIdx.x & 31) == 0) {
+      t.i0 = tile << p.bm_log2;
+      t.k0 = k * kBK;
+      t.rest = rest;
+      t.l = l;
+      t.q = q;
+      t.d = d;
+      t.nk = (int)min((long long)kBK, p.K - k * kBK);
+      t.valid = 1;
+      t.last = k + 1 == kend;
+      t.slot = slot;
+    }
+    ++k;
+  }
+};
+
+// KC: the contraction is contiguous in memory (L > 1), stage rows are output
+// rows of 32 elements, their 16-byte chunks permuted by the row (chunk ^ row
+// mod 8) so that eight neighbouring rows are read without bank conflicts;
+// otherwise (L = 1) the outputs are contiguous and stage rows are contraction
+// elements of BM outputs.
+template <bool KC>
+__global__ void __launch_bounds__(kThreadsMax + 32, 2)
+k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ StepTab tabs[kTabs];
+  const int tid = threadIdx.x, T = blockDim.x - 32;
+  const int BM = 1 << p.bm_log2, RP = p.RP;
+  const uint32_t sbase = s_u32(sm);
+  // ---- the factor rows of a step, by n threads: one per element of the fastest
+  // mode, then the distinct rest rows of every other mode, 2^gsh lanes (at most
+  // a warp) per row
+  const int rc = p.vecb ? p.R >> 2 : p.R;  // copies per factor row
+  auto load_b = [&](const StepTab& t, int stage, int id, int n) {
+    if (!t.valid) return;
+    const uint32_t raw = sbase + 4u * (stage * p.stage_floats + p.x_floats);
+    const int sub = id & ((1 << p.gsh) - 1), r0 = id >> p.gsh, dr = n >> p.gsh;
+    auto row = [&](uint32_t dst, const float* src) {
+      if (p.vecb) {
+        if (sub < rc) cpa16(dst + 16u * sub, src + 4 * sub);
+      } else {
+        for (int c = sub; c < rc; c += 1 << p.gsh) cpa4(dst + 4u * c, src + c);
+      }
+    };
+    const int d = t.d, nk = t.nk;
+#pragma unroll 4
+    for (int kk = r0; kk < nk; kk += dr) {
+      const int x = d + kk;
+      row(raw + 4u * kk * RP, p.H[0] + (x - wraps(x, p.dim[0], p.mag0) * p.dim[0]) * p.ld);
+    }
+    if (p.nm > 1) {
+      const int nrest = wraps(d + nk - 1, p.dim[0], p.mag0) + 1;
+#pragma unroll 1
+      for (int j = r0; j < nrest; j += dr) {
+        long long q = t.rest + j;
+        uint32_t dst = raw + 4u * (kBK + j) * RP;
+#pragma unroll 1
+        for (int m = 1; m < p.nm; ++m, dst += 4u * p.nrest_max * RP) {
+          long long x = q;
+          if (m + 1 < p.nm) {  // the last digit is what is left
+            q = (unsigned long long)x >> 32 ? x / p.dim[m] : (long long)((unsigned)x / (unsigned)p.dim[m]);
+            x -= q * p.dim[m];
+          }
+          row(dst, p.H[m] + x * p.ld);
+        }
+      }
+    }
+  };
+
+  if (tid >= T) {
+    // ------------------------------------------------------------ feeder --
+    const int lane = tid - T;
+    Feeder f(p);
+    for (int s = 0; s < kStages; ++s) f.next(p, tabs[s], KC);
+    __syncthreads();
+    pdl_wait();
+    if (!p.b_all) {
+      load_b(tabs[0], 0, lane, 32);
+      load_b(tabs[1], 1, lane, 32);
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+    }
+    __syncthreads();
+    for (int s = 0, st = 2;; ++s) {
+      // the factor rows of step s + 1 have landed
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+      __syncthreads();
+      const StepTab& t = tabs[s & (kTabs - 1)];
+      if (!t.valid) break;
+      const bool last = t.last != 0;
+      if (!p.b_all) load_b(tabs[(s + 2) & (kTabs - 1)], st, lane, 32);
+      st = st + 1 == kStages ? 0 : st + 1;
+      f.next(p, tabs[(s + 3) & (kTabs - 1)], KC);
+      if (last && p.KG > 1) {
+        // the barriers of the computing warps' KG sums
+        __syncthreads();
+        for (int half = p.KG >> 1; half >= 1; half >>= 1)
+          for (int j0 = 0; j0 < 4; j0 += p.red_pairs) {
+            __syncthreads();
+            __syncthreads();
+          }
+      }
+    }
+    return;
+  }
+
+  // -------------------------------------------------------- computing warps --
+  uint64_t pol;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+  const int Tl = p.tl;
+
+  // ---- the tensor tile of a step into a stage
+  auto load_x = [&](const StepTab& t, int stage) {
+    if (!t.valid || tid >= Tl) return;
+    const uint32_t xs = sbase + 4u * stage * p.stage_floats;
+    const long long i0 = t.i0;
+    const int rows = (int)min((long long)BM, p.I - i0);
+    const int nk = t.nk;
+    if constexpr (KC) {
+      if (p.vecx) {
+        const int c = tid & 7, dr = Tl >> 3;  // this thread's chunk of rows i, i + dr, ...; dr % 8 == 0
+        if (4 * c < nk) {                     // K is a multiple of 4: chunks are whole
+          int i = tid >> 3;
+          long long l = t.l + 4 * c;
+          const int w = wraps(l, p.L, p.magl);
+          l -= w * p.L;
+          const float* src = p.X + l + p.L * (i0 + i + p.I * (t.q + w));
+          uint32_t d = xs + 4u * (i * kBK + ((c ^ (i & 7)) << 2));
+          const long long ds = p.L * dr;
+#pragma unroll 4
+          for (; i < rows; i += dr, src += ds, d += 4u * kBK * dr) {
+            if (p.evict) cpa16_hint(d, src, pol);
+            else cpa16(d, src);
+          }
+        }
+      } else {
+        const int kk = tid & 31, dr = Tl >> 5;
+        int i = tid >> 5;
+        const bool in = kk < nk;
+        long long l = t.l + kk;
+        const int w = wraps(l, p.L, p.magl);
+        l -= w * p.L;
+        const float* src = p.X + l + p.L * (i0 + i + p.I * (t.q + w));
+        const long long ds = p.L * dr;
+        if (in) {
+#pragma unroll 4
+          for (; i < rows; i += dr, src += ds)
+            cpa4(xs + 4u * (i * kBK + (((kk >> 2) ^ (i & 7)) << 2) + (kk & 3)), src);
+        } else {
+          // up to the next multiple of the four elements a thread takes at a time
+          for (; i < rows && kk < ((nk + 3) & ~3); i += dr)
+            sm[stage * p.stage_floats + i * kBK + (((kk >> 2) ^ (i & 7)) << 2) + (kk & 3)] = 0.0f;
+        }
+      }
+    } else {
+      const int sh = p.vecx ? p.bm_log2 - 2 : p.bm_log2;  // copies per stage row
+      const int ii = tid & ((1 << sh) - 1);
+      if (p.vecx) {
+        int kk = tid >> sh;
+        const int dk = Tl >> sh;  // Tl >= BM / 4
+        if (4 * ii < rows) {
+          const float* src = p.X + (t.k0 + kk) * p.I + i0 + 4 * ii;
+          uint32_t d = xs + 4u * ((kk << p.bm_log2) + 4 * ii);
+          const long long ds = p.I * dk;
+#pragma unroll 4
+          for (; kk < nk; kk += dk, src += ds, d += 4u * (dk << p.bm_log2)) {
+            if (p.evict) cpa16_hint(d, src, pol);
+            else cpa16(d, src);
+          }
+        }
+      } else {
+        const float* src = p.X + t.k0 * p.I + i0;
+        const int end = nk << sh;
+#pragma unroll 4
+        for (int e = tid; e < end; e += Tl) {
+          const int kk = e >> sh, i = e & (BM - 1);
+          if (i < rows) cpa4(xs + 4u * e, src + (long long)kk * p.I + i);
+        }
+      }
+    }
+  };
+  // ---- Khatri-Rao rows of a step in place: the fastest mode's rows times the
+  // rest; elements past the end up to a multiple of four are zero
+  const int fk0 = tid / (RP >> 2), fc0 = tid - fk0 * (RP >> 2);
+  auto form_b = [&](const StepTab& t, int stage) {
+    if (!t.valid || (p.nm == 1 && t.nk == kBK)) return;
+    float* raw = sm + stage * p.stage_floats + p.x_floats;
+    const int r4 = RP >> 2;
+    int kk = fk0, c = fc0;
+    const int end = (t.nk + 3) & ~3;
+#pragma unroll 1
+    while (kk < end) {
+      float4* d = reinterpret_cast<float4*>(raw + kk * RP + 4 * c);
+      float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (kk < t.nk) {
+        v = *d;
+        const float* rest = raw + (kBK + wraps(t.d + kk, p.dim[0], p.mag0)) * RP + 4 * c;
+#pragma unroll 1
+        for (int m = 1; m < p.nm; ++m, rest += p.nrest_max * RP) {
+          const float4 w = *reinterpret_cast<const float4*>(rest);
+          v.x *= w.x;
+          v.y *= w.y;
+          v.z *= w.z;
+          v.w *= w.w;
+        }
+      }
+      *d = v;
+      kk += p.fk;
+      c += p.fc;
+      if (c >= r4) {
+        c -= r4;
+        ++kk;
+      }
+    }
+  };
+
+  // ---- this thread's place
+  const int rl = tid & 7;
+  int id = tid >> 3;
+  const int cg = id % p.CG;
+  id /= p.CG;
+  const int rgh = id % p.RGH;
+  const int kg = id / p.RGH;
+  const bool act = kg < p.KG;
+  const int kper = kBK / p.KG, ka = kg * kper;
+  const int ngroup = 8 * p.CG * p.RGH;  // threads of a k group
+  u64 acc[kTM][4];
+#pragma unroll
+  for (int i = 0; i < kTM; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+
+  __syncthreads();
+  // the tensor is written by no kernel of an iteration: its first tiles stream
+  // in while the preceding kernel finishes
+  load_x(tabs[0], 0);
+  load_x(tabs[1], 1);
+  pdl_wait();
+  if (p.b_all) {
+    load_b(tabs[0], 0, tid, T);
+    load_b(tabs[1], 1, tid, T);
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+  form_b(tabs[0], 0);
+
+  for (int s = 0, st = 0;; ++s) {
+    // step s and the factor rows of step s + 1 have landed, and every thread
+    // is done with step s - 1
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();
+    const StepTab& t = tabs[s & (kTabs - 1)];
+    if (!t.valid) break;
+    const int st1 = st + 1 == kStages ? 0 : st + 1, st2 = st1 + 1 == kStages ? 0 : st1 + 1;
+    const StepTab& t2 = tabs[(s + 2) & (kTabs - 1)];
+    if (p.b_all) load_b(t2, st2, tid, T);
+    cpa_commit();
+    load_x(t2, st2);
+    cpa_commit();
+    form_b(tabs[(s + 1) & (kTabs - 1)], st1);
+
+    float* xs = sm + st * p.stage_floats;
+    const float* bs = xs + p.x_floats + 8 * cg;
+    st = st1;
+    if (act) {
+      if constexpr (KC) {
+        const float* xrow = xs + (32 * rgh + rl) * kBK;
+        const int kb = min(ka + kper, (t.nk + 3) & ~3);
+#pragma unroll 1
+        for (int k = ka; k < kb; k += 4) {
+          const int c = ((k >> 2) ^ rl) << 2;
+          float4 a[kTM];
+#pragma unroll
+          for (int i = 0; i < kTM; ++i) a[i] = *reinterpret_cast<const float4*>(xrow + 8 * i * kBK + c);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bs + (k + e) * RP);
+            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(bs + (k + e) * RP + 4);
+#pragma unroll
+            for (int i = 0; i < kTM; ++i) {
+              const float v = e == 0 ? a[i].x : (e == 1 ? a[i].y : (e == 2 ? a[i].z : a[i].w));
+              const u64 x = pack2(v, v);
+              acc[i][0] = ffma2(x, b0.x, acc[i][0]);
+              acc[i][1] = ffma2(x, b0.y, acc[i][1]);
+              acc[i][2] = ffma2(x, b1.x, acc[i][2]);
+              acc[i][3] = ffma2(x, b1.y, acc[i][3]);
+            }
+          }
+        }
+      } else {
+        const float* xcol = xs + 32 * rgh + 4 * rl;
+        const int kb = min(ka + kper, t.nk);
+#pragma unroll 4
+        for (int k = ka; k < kb; ++k) {
+          const float4 v = *reinterpret_cast<const float4*>(xcol + (k << p.bm_log2));
+          const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bs + k * RP);
+          const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(bs + k * RP + 4);
+          const float a[kTM] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int i = 0; i < kTM; ++i) {
+            const u64 x = pack2(a[i], a[i]);
+            acc[i][0] = ffma2(x, b0.x, acc[i][0]);
+            acc[i][1] = ffma2(x, b0.y, acc[i][1]);
+            acc[i][2] = ffma2(x, b1.x, acc[i][2]);
+            acc[i][3] = ffma2(x, b1.y, acc[i][3]);
+          }
+        }
+      }
+    }
+    if (!t.last) continue;
+
+    // ---- end of a run: add the KG partial sums in a fixed tree, then write the tile
+    const int q = tid - kg * ngroup;  // thread within the k group
+    if (p.KG > 1) {
+      // through this step's stage, done with once every thread is; jn of a
+      // thread's four column pairs at a time fit
+      float2* red = reinterpret_cast<float2*>(xs);
+      const int jn = p.red_pairs;
+      __syncthreads();
+      for (int half = p.KG >> 1; half >= 1; half >>= 1) {
+        for (int j0 = 0; j0 < 4; j0 += jn) {
+          if (kg >= half && kg < 2 * half) {
+            float2* dst = red + (kg - half) * ngroup * (jn * kTM) + q;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (j >= j0 && j < j0 + jn)
+#pragma unroll
+                for (int i = 0; i < kTM; ++i) dst[((j - j0) * kTM + i) * ngroup] = unpack2(acc[i][j]);
+          }
+          __syncthreads();
+          if (kg < half) {
+            const float2* src = red + kg * ngroup * (jn * kTM) + q;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (j >= j0 && j < j0 + jn)
+#pragma unroll
+                for (int i = 0; i < kTM; ++i) {
+                  const float2 v = src[((j - j0) * kTM + i) * ngroup], a = unpack2(acc[i][j]);
+                  acc[i][j] = pack2(a.x + v.x, a.y + v.y);
+                }
+          }
+          __syncthreads();
+        }
+      }
+    }
+    if (kg == 0) {
+      const long long i0 = t.i0;
+      const bool part = t.slot >= 0;
+      float* dst = part ? p.slots + t.slot * p.slot_floats : p.out + i0 * p.ld;
+      const int ld = part ? p.R : p.ld;
+      const bool vec = part ? (p.R & 3) == 0 : p.veco;
+      const int rows = (int)min((long long)BM, p.I - i0);
+#pragma unroll
+      for (int i = 0; i < kTM; ++i) {
+        const int row = 32 * rgh + (KC ? 8 * i + rl : 4 * rl + i);
+        if (row < rows) {
+          float* d = dst + (long long)row * ld + 8 * cg;
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const float2 a = unpack2(acc[i][2 * j]), b = unpack2(acc[i][2 * j + 1]);
+            const int left = p.R - 8 * cg - 4 * j;
+            if (vec && left >= 4) {
+              reinterpret_cast<float4*>(d)[j] = make_float4(a.x, a.y, b.x, b.y);
+            } else {
+              if (left > 0) d[4 * j] = a.x;
+              if (left > 1) d[4 * j + 1] = a.y;
+              if (left > 2) d[4 * j + 2] = b.x;
+              if (left > 3) d[4 * j + 3] = b.y;
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kTM; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+
+// Adds the partial tiles of the cut tiles in run order.  blockIdx.y: tile.
+// QUAD: four threads per output, thread q adding runs q, q + 4, ... of the
+// tile, combined as (0 + 1) + (2 + 3); else one thread adds them all in order.
+template <bool QUAD>
+__global__ void __launch_bounds__(256)
+k_simt_fixup(const float* __restrict__ slots, float* __restrict__ out, long long I, int R, int ld, int BM,
+             long long slot_floats, long long nk, long long whole, long long U2, int G2,
+             int two) {
+  pdl_wait();
+  pdl_trigger();
+  const long long t = blockIdx.y, u0 = t * nk, u1 = u0 + nk - 1;
+  const long long c0 = ((u0 + 1) * G2 - 1) / U2, c1 = ((u1 + 1) * G2 - 1) / U2;
+  if (c0 == c1) return;  // one run holds the whole tile and has written it
+  const long long i0 = (whole + t) * BM;
+  const int rows = (int)min((long long)BM, I - i0);
+  const int q = QUAD ? threadIdx.x & 3 : 0;
+  const int e = (int)(blockIdx.x * 256 + threadIdx.x) >> (QUAD ? 2 : 0);
+  const bool in = e < rows * R;
+  const float* base = slots + e;
+  float s = 0.0f;
+  if (in) {
+#pragma unroll 4
+    for (long long c = c0 + q; c <= c1; c += QUAD ? 4 : 1) {
+      // a run that began in an earlier tile left this one in its second slot
+      const long long sl = two ? 2 * c + (c == c0 && run_start(c, U2, G2) < u0 ? 1 : 0) : c;
+      s += __ldg(base + sl * slot_floats);
+    }
+  }
+  if (QUAD) {
+    s += __shfl_down_sync(0xffffffffu, s, 1);
+    s += __shfl_down_sync(0xffffffffu, s, 2);
+  }
+  if (in && q == 0) out[(i0 + e / R) * ld + e % R] = s;
+}
+
+long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
+
+struct SimtPlan {
+  SimtArgs a;
+  int BM, threads, grid;
+  size_t smem;
+};
+
+// Tile, thread split and work split of one MTTKRP; cap: floats of scratch for
+// partial tiles.
+bool plan_simt(int64_t L, int64_t I, int64_t Q, const KrpDesc& KL, const KrpDesc& KQ, int R,
+               size_t cap, int num_sms, SimtPlan* pl) {
+  SimtArgs& a = pl->a;
+  a = SimtArgs{};
+  a.L = L;
+  a.I = I;
+  a.K = (long long)L * Q;
+  a.R = R;
+  a.nk = cdiv(a.K, kBK);
+  for (const KrpDesc* d : {&KL, &KQ})
+    for (int m = 0; m < d->nm; ++m) {
+      if (a.nm == kMaxModes) return false;
+      a.dim[a.nm] = (int)d->dim[m];
+      a.H[a.nm++] = d->H[m];
+    }
+  if (a.nm < 1) return false;
+  a.dstep = kBK % a.dim[0];
+  a.rstep = kBK / a.dim[0];
+  a.mag0 = a.dim[0] < kBK ? (65535 + a.dim[0]) / a.dim[0] : 0;
+  a.magl = L < kBK ? (int)((65535 + L) / L) : 0;
+  a.lstep = kBK % L;
+  a.qstep = kBK / L;
+  a.nrest_max = a.nm > 1 ? std::min(kBK, (kBK - 1) / a.dim[0] + 2) : 0;
+  a.CG = (R + 7) / 8;
+  a.RP = 8 * a.CG;
+  // tile rows 32 RGH: the least work for the busiest SM, a step costing its
+  // rows plus the part that does not depend on them
+  double best = 0.0;
+  for (int c = 0; c < 4; ++c) {
+    SimtPlan t = *pl;
+    SimtArgs& b = t.a;
+    b.RGH = 1 << c;
+    b.bm_log2 = 5 + c;
+    t.BM = 32 << c;
+    if (8 * b.RGH * a.CG > kThreadsMax) break;
+    // splitting a step further than over four warps only shortens each one's
+    // share of it: 301 x 257 x 199, R = 20, 72 us at eight warps against 68
+    b.KG = 1;
+    while (b.KG < 8 && 8 * b.RGH * a.CG * b.KG * 2 <= kThreadsMax / 2) b.KG *= 2;
+    const int computing = 8 * b.RGH * a.CG * b.KG;
+    t.threads = (computing + 31) / 32 * 32;
+    b.tl = t.threads / 64 * 64;
+    const int rest = (a.nm - 1) * a.nrest_max;
+    // more copies of factor rows than a warp issues in a step's time
+    b.b_all = (kBK + rest) * (R % 4 == 0 ? R / 4 : R) > 32 * 16;
+    b.fk = t.threads / (a.RP / 4);
+    b.fc = t.threads % (a.RP / 4);
+    b.x_floats = t.BM * kBK;
+    b.stage_floats = b.x_floats + (kBK + rest) * a.RP;
+    b.red_pairs = 4;
+    while (b.red_pairs > 1 && computing / 2 * b.red_pairs * kTM * 2 > b.stage_floats) b.red_pairs /= 2;
+    t.smem = (size_t)kStages * b.stage_floats * sizeof(float);
+    if (t.smem > (size_t)(kSmemMax - kStaticSmem)) break;
+    // CTAs per SM at once: shared memory, and the registers of five warps (96 a
+    // thread) on each of its four schedulers
+    const int occ = std::max(1, std::min((int)(kSmemSM / (t.smem + kStaticSmem + 1024)),
+                                         20 / (t.threads / 32 + 1)));
+    const long long G = (long long)num_sms * occ, gx = cdiv(I, t.BM);
+    long long left = gx % G;
+    if (left * 10 >= G * 9) left = 0;  // a wave nine tenths full is left whole
+    b.whole = gx - left;
+    b.slot_floats = (long long)t.BM * R;
+    if (left > 0) {
+      // at least four steps per run; one slot per run where runs end with tiles
+      long long g2 = std::max(left, std::min(G, left * a.nk / 4));
+      const long long slots = (long long)(cap / (size_t)b.slot_floats);
+      if (g2 % left != 0 && 2 * g2 > slots) g2 = left * (g2 / left);
+      if (g2 % left == 0 && g2 > slots) g2 = left * std::max(1LL, slots / left);
+      if (g2 <= left) {
+        b.whole = gx;
+      } else {
+        b.U2 = left * a.nk;
+        b.G2 = (int)g2;
+        b.two = g2 % left != 0;
+      }
+    }
+    t.grid = (int)std::max<long long>(std::min(G, b.whole), b.G2);
+    const double steps = (double)cdiv(b.whole, G) * a.nk + (b.G2 ? (double)cdiv(b.U2, b.G2) : 0.0);
+    const double cost = steps * (double)cdiv(t.grid, num_sms) * (t.BM + 24) * (occ == 1 ? 1.15 : 1.0);
+    if (best == 0.0 || cost < best) {
+      best = cost;
+      *pl = t;
+    }
+  }
+  return best > 0.0;
+}
+
+// The launches for the rank columns [r0, r0 + pl.a.R) of a rank-R MTTKRP.
+cudaError_t launch_columns(const float* X, int R, int r0, float* out, float* partials,
+                           SimtPlan pl, cudaStream_t st) {
+  SimtArgs& a = pl.a;
+  auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
+  const bool KC = a.L > 1;
+  a.X = X;
+  a.ld = R;
+  a.out = out + r0;
+  for (int m = 0; m < a.nm; ++m) a.H[m] += r0;
+  a.slots = partials;
+  // 16-byte copies need whole units along the contiguous index; the factor
+  // rows also a rank of whole units
+  a.vecx = al16(X) && (KC ? a.L : a.I) % 4 == 0;
+  a.vecb = R % 4 == 0 && a.R % 4 == 0;
+  for (int m = 0; m < a.nm; ++m) a.vecb = a.vecb && al16(a.H[m]);
+  a.veco = R % 4 == 0 && al16(a.out);
+  // a tensor that cannot stay in the 126 MB L2 is marked evict-first, so that
+  // its stream leaves the nodes and factors there
+  a.evict = (double)a.I * a.K * sizeof(float) > 96e6;
+  const int copies = a.vecb ? a.R / 4 : a.R;
+  while (a.gsh < 5 && (1 << a.gsh) < copies) ++a.gsh;
+  cudaError_t e = launch_kernel(KC ? k_simt_mttkrp<true> : k_simt_mttkrp<false>,
+                                dim3((unsigned)pl.grid), dim3(pl.threads + 32),
+                                pl.smem, st, a);
+  if (e != cudaSuccess || a.G2 == 0) return e;
+  const long long left = a.U2 / a.nk;
+  const bool quad = a.G2 >= 8 * left;
+  const int gx = (int)cdiv(a.slot_floats * (quad ? 4 : 1), 256);
+  return launch_kernel(quad ? k_simt_fixup<true> : k_simt_fixup<false>,
+                       dim3((unsigned)gx, (unsigned)left), dim3(256), 0, st,
+                       (const float*)partials, a.out, a.I, a.R, a.ld, pl.BM, a.slot_floats, a.nk,
+                       a.whole, a.U2, a.G2, a.two);
+}
+
+// Rows, ranks and contraction chunks that bound the scratch a context sets
+// aside for the partial sums of one MTTKRP: enough chunks of at least 256
+// elements for four 128 x 32 tiles per SM.
+int scratch_chunks(long long tiles, long long Ktot, int num_sms) {
+  const long long target = 4LL * num_sms;
+  if (tiles >= target) return 1;
+  return (int)std::min(cdiv(target, tiles), std::max(1LL, cdiv(Ktot, 256)));
+}
+
+}  // namespace
+
+cudaError_t simt_attributes_init() {
+  for (auto k : {k_simt_mttkrp<false>, k_simt_mttkrp<true>}) {
+    cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kStaticSmem);
+    // all of the SM's shared memory: the plan counts on it for its CTAs per SM
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                               cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms) {
+  const int C = scratch_chunks(cdiv(I, 128) * cdiv(R, 32), (long long)L * Q, num_sms);
+  return C > 1 ? (size_t)C * I * R : 0;
+}
+
+cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
+                               const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,
+                               float* partials, size_t part_cap, int num_sms,
+                               cudaStream_t st) {
+  // ranks in one launch unless the factor rows of a step (long products of short
+  // modes at a high rank) do not fit in shared memory: then in column blocks
+  int cols = R;
+  SimtPlan pl;
+  while (!plan_simt(L, I, Q, KL, KQ, cols, partials ? part_cap : 0, num_sms, &pl)) {
+    if (cols <= 8) return cudaErrorInvalidValue;
+    cols = ((cols + 1) / 2 + 7) / 8 * 8;
+  }
+  for (int r0 = 0; r0 < R; r0 += cols) {
+    const int n = std::min(cols, R - r0);
+    if (n != cols && !plan_simt(L, I, Q, KL, KQ, n, partials ? part_cap : 0, num_sms, &pl))
+      return cudaErrorInvalidValue;
+    const cudaError_t e = launch_columns(X, R, r0, out, partials, pl, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace nncp

@@ -1972,6 +1972,7 @@ cudaError_t kernel_attributes_init() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_update_cluster<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)cluster_smem<64>());
+  if (e == cudaSuccess) e = simt_attributes_init();
   if (e == cudaSuccess) e = tc_attributes_init();
   return e;
 }
