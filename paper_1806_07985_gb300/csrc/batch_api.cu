@@ -106,6 +106,17 @@ size_t b_tensor_layout(int N, const int64_t* dm, int R, int fit_cap, BTensor* d,
   return off;
 }
 
+void b_plan_sizes(const BTensor* ts, int count, BPlan* p) {
+  p->max_rows = p->max_factor = p->max_order = 1;
+  for (int t = 0; t < count; ++t) {
+    p->max_order = std::max(p->max_order, ts[t].N);
+    for (int n = 0; n < ts[t].N; ++n) {
+      p->max_rows = std::max(p->max_rows, (int)ts[t].dims[n]);
+      p->max_factor = std::max(p->max_factor, (int)ts[t].dims[n] * ts[t].R);
+    }
+  }
+}
+
 void b_build_plan(const BTensor* ts, int C, int N, BPlan* p) {
   p->count = C;
   p->N = N;
@@ -115,11 +126,10 @@ void b_build_plan(const BTensor* ts, int C, int N, BPlan* p) {
   p->lam_total = 0;
   int rmax = 1;
   p->hs_floats = 0;
-  p->max_rows = 1;
+  b_plan_sizes(ts, C, p);
   for (int t = 0; t < C; ++t) {
     rmax = std::max(rmax, ts[t].R);
     p->hs_floats = std::max(p->hs_floats, (int)ts[t].dims[0] * b_rank_pad(ts[t].R));
-    for (int n = 0; n < N; ++n) p->max_rows = std::max(p->max_rows, (int)ts[t].dims[n]);
     p->lam_off[t] = (int)p->lam_total;
     p->lam_total += ts[t].R;
   }

@@ -10,6 +10,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "batch_kernels.cuh"
 
@@ -21,8 +22,30 @@ __device__ __forceinline__ bool tensor_done(const BTensor& t) { return t.flags[0
 
 // ---------------------------------------------------------------- init --
 
+// Float-float accumulator: TwoSum keeps what a float32 addition rounds off, so
+// the pair carries about 48 bits at a few float32 operations per term (a float64
+// addition issues at about a sixtieth of their rate here).
+struct SumFF {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float v) {
+    const float s = hi + v, t = s - hi;
+    lo += (hi - (s - t)) + (v - t);
+    hi = s;
+  }
+  // a * b exactly: the rounded product and its error
+  __device__ __forceinline__ void add_product(float a, float b) {
+    const float p = a * b;
+    lo += fmaf(a, b, -p);
+    add(p);
+  }
+  __device__ __forceinline__ double value() const {
+    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+  }
+};
+
 // alpha partials: item (tensor, chunk of kAlphaChunk elements) -> alpha_part[item];
-// squares summed four at a time in FP32, the rest in FP64 (fixed order)
+// squares summed four at a time in FP32, those sums as float-float pairs, the
+// threads' totals in FP64 (fixed order)
 __global__ void __launch_bounds__(256) k_b_sumsq(const BTensor* __restrict__ ts,
                                                  const int4* __restrict__ items,
                                                  double* __restrict__ alpha_part) {
@@ -32,11 +55,20 @@ __global__ void __launch_bounds__(256) k_b_sumsq(const BTensor* __restrict__ ts,
   const int n = (int)min(kAlphaChunk, t.I - e0);
   const float* x = t.X + e0;
   const int n4 = n >> 2;
+  const float4* x4 = reinterpret_cast<const float4*>(x);
   double acc = 0.0;
-#pragma unroll 4
-  for (int v = threadIdx.x; v < n4; v += blockDim.x) {
-    const float4 a = __ldcs(reinterpret_cast<const float4*>(x) + v);
-    acc += (double)(a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w);
+  for (int v0 = threadIdx.x; v0 < n4; v0 += 8 * 256) {
+    // eight loads in flight; into float64 after each eight, which keeps
+    // float32's range out of the sum
+    float4 a[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      a[q] = v0 + 256 * q < n4 ? __ldcs(x4 + v0 + 256 * q) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    SumFF s;
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      s.add(a[q].x * a[q].x + a[q].y * a[q].y + a[q].z * a[q].z + a[q].w * a[q].w);
+    acc += s.value();
   }
   if ((int)threadIdx.x < n - 4 * n4) {
     const float v = x[4 * n4 + threadIdx.x];
@@ -55,14 +87,59 @@ __global__ void __launch_bounds__(256) k_b_sumsq(const BTensor* __restrict__ ts,
 
 // per tensor: alpha = sum of its partials (in order), normalise every factor
 // (lambda = product of the column norms), G_n = H_n^T H_n, S for mode 1,
-// flags and fit history cleared (Alg. 3 initialisation).
-__global__ void k_b_init(BTensor* __restrict__ ts, const double* __restrict__ alpha_part,
-                         const int* __restrict__ alpha_first) {
+// flags and fit history cleared (Alg. 3 initialisation).  CTA (tensor, mode)
+// for the factors, then CTA per tensor for what joins the modes.  The column
+// sums and Grams are float-float sums of exact products; in float64, with a
+// float64 division per factor element, one CTA per tensor took 257 us for 1024
+// tensors on a GB300.
+__global__ void __launch_bounds__(256) k_b_init_mode(BTensor* __restrict__ ts) {
+  BTensor& t = ts[blockIdx.x];
+  const int n = blockIdx.y;
+  if (n >= t.N) return;  // the tensors may be of different orders
+  const int R = t.R, R2 = R * R;
+  const int In = (int)t.dims[n];
+  float* Hn = t.H[n];
+  extern __shared__ __align__(16) float hs[];  // In x R
+  __shared__ double inv[kBatchMaxRank];
+  __shared__ double part[256];
+  const int tid = threadIdx.x;
+  for (int e = tid; e < In * R; e += 256) hs[e] = Hn[e];
+  __syncthreads();
+  // column sums of squares: the rows of a column over 256 / R threads, their
+  // sums added in order
+  const int P = 256 / R, r0 = tid % R, p0 = tid / R;
+  if (p0 < P) {
+    SumFF s;
+    for (int i = p0; i < In; i += P) s.add_product(hs[i * R + r0], hs[i * R + r0]);
+    part[tid] = s.value();
+  }
+  __syncthreads();
+  if (tid < R) {
+    double s = 0.0;
+    for (int p = 0; p < P; ++p) s += part[p * R + tid];
+    if (!(s > 1e-30 && s < 1e36)) {  // squares near the ends of float32's range: in float64
+      s = 0.0;
+      for (int i = 0; i < In; ++i) s += (double)hs[i * R + tid] * hs[i * R + tid];
+    }
+    const double c = sqrt(s);
+    inv[tid] = c > 0.0 ? 1.0 / c : 0.0;
+    // the norms wait in this mode's Gram row for k_b_init
+    t.G[(long long)n * R2 + tid] = c;
+  }
+  __syncthreads();
+  for (int e = tid; e < In * R; e += 256) {
+    const float h = (float)((double)hs[e] * inv[e % R]);
+    hs[e] = h;
+    Hn[e] = h;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_b_init(BTensor* __restrict__ ts, const double* __restrict__ alpha_part,
+                                                const int* __restrict__ alpha_first) {
   BTensor& t = ts[blockIdx.x];
   const int R = t.R, N = t.N, R2 = R * R;
-  __shared__ double lam[kBatchMaxRank];
-  __shared__ double cn[kBatchMaxRank];
-  if (threadIdx.x == 0) {
+  const int tid = threadIdx.x;
+  if (tid == 0) {
     double a = 0.0;
     for (int c = alpha_first[blockIdx.x]; c < alpha_first[blockIdx.x + 1]; ++c) a += alpha_part[c];
     t.scal[0] = a;
@@ -71,38 +148,42 @@ __global__ void k_b_init(BTensor* __restrict__ ts, const double* __restrict__ al
     t.flags[1] = 0;
     t.flags[2] = 0;
   }
-  for (int r = threadIdx.x; r < R; r += blockDim.x) lam[r] = 1.0;
+  if (tid < R) {
+    double l = 1.0;
+    for (int n = 0; n < N; ++n) l *= t.G[(long long)n * R2 + tid];
+    t.lam[tid] = l;
+  }
+  extern __shared__ __align__(16) float hs[];  // one factor
   __syncthreads();
+  double S[(kBatchMaxRank * kBatchMaxRank + 255) / 256];
+#pragma unroll
+  for (int q = 0; q < (int)(sizeof S / sizeof S[0]); ++q) S[q] = 1.0;
   for (int n = 0; n < N; ++n) {
-    float* Hn = t.H[n];
     const int In = (int)t.dims[n];
-    for (int r = threadIdx.x; r < R; r += blockDim.x) {
-      double s = 0.0;
-      for (int i = 0; i < In; ++i) s += (double)Hn[i * R + r] * Hn[i * R + r];
-      cn[r] = sqrt(s);
-      lam[r] *= cn[r];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < In * R; e += blockDim.x) {
-      const double c = cn[e % R];
-      Hn[e] = c > 0.0 ? (float)((double)Hn[e] / c) : 0.0f;
-    }
+    for (int e = tid; e < In * R; e += 256) hs[e] = t.H[n][e];
     __syncthreads();
     double* Gn = t.G + (long long)n * R2;
-    for (int e = threadIdx.x; e < R2; e += blockDim.x) {
-      const int a = e / R, b = e % R;
-      double s = 0.0;
-      for (int i = 0; i < In; ++i) s += (double)Hn[i * R + a] * Hn[i * R + b];
-      Gn[e] = s;
+#pragma unroll
+    for (int q = 0; q < (int)(sizeof S / sizeof S[0]); ++q) {
+      const int e = tid + 256 * q;
+      if (e < R2) {
+        const int a = e / R, b = e - a * R;
+        SumFF s;
+        for (int i = 0; i < In; ++i) s.add_product(hs[i * R + a], hs[i * R + b]);
+        const double g = s.value();
+        Gn[e] = g;
+        if (n > 0) S[q] *= g;
+      }
     }
     __syncthreads();
   }
-  for (int r = threadIdx.x; r < R; r += blockDim.x) t.lam[r] = lam[r];
-  for (int e = threadIdx.x; e < R2; e += blockDim.x) {
-    double s = 1.0;
-    for (int k = 1; k < N; ++k) s *= t.G[(long long)k * R2 + e];
-    t.S[e] = s;
-    t.S32[e] = (float)s;
+#pragma unroll
+  for (int q = 0; q < (int)(sizeof S / sizeof S[0]); ++q) {
+    const int e = tid + 256 * q;
+    if (e < R2) {
+      t.S[e] = S[q];
+      t.S32[e] = (float)S[q];
+    }
   }
 }
 
@@ -1347,57 +1428,87 @@ __global__ void __launch_bounds__(256) k_b_mttv_leaf(const BTensor* __restrict__
 
 // child node {a+1..N} from node {a..N}: out(j, r) = sum_i T[(i + I_a j) R + r] H_a(i, r)
 // with the updated H_a; the output is M when the child is a leaf.  Item
-// (tensor, block of first_jb[a] rows j); warp per row j (two rows at a time,
-// for more loads in flight): lanes = (i phase, rank) read the row's I_a x R
-// block coalesced, then add their i phases in a fixed shuffle tree.
+// (tensor, block of first_jb[a] rows j); warp per row j, four rows at a time.
+// Lanes = (i phase, group of V ranks, V = 4 when R % 4 == 0): they read the
+// row's I_a x R block coalesced, V floats per load, and their i phases are added
+// in a fixed shuffle tree.  Bound by the latency of the node's loads: with one
+// rank per lane and two rows in flight it took 107 us for 1024 tensors on a
+// GB300 (11 % of the issue slots).
+template <int V>
+__device__ __forceinline__ void first_rows(const float* __restrict__ T, const float* __restrict__ Ha,
+                                           float* __restrict__ out, int R, int Ia, int j0, int j1) {
+  constexpr int NR = 4;  // rows in flight
+  using VT = typename std::conditional<V == 4, float4, float>::type;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+  const int RV = R / V, E = Ia * R;
+  for (int rb = 0; rb < RV; rb += 32) {
+    const int Rb = min(32, RV - rb), S = 32 / Rb;
+    const int sub = lane / Rb, r = (rb + lane - sub * Rb) * V;
+    const bool act = sub < S;
+    for (int j = j0 + warp; j < j1; j += NR * nwarp) {
+      float acc[NR][V];
+      const float* Tj[NR];
+#pragma unroll
+      for (int q = 0; q < NR; ++q) {
+        const int jq = j + q * nwarp;
+        Tj[q] = T + (long long)(jq < j1 ? jq : j) * E + r;
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[q][v] = 0.0f;
+      }
+      if (act) {
+#pragma unroll 4
+        for (int i = sub; i < Ia; i += S) {
+          const VT hv = __ldg(reinterpret_cast<const VT*>(Ha + i * R + r));
+          const float* h = reinterpret_cast<const float*>(&hv);
+          VT x[NR];
+#pragma unroll
+          for (int q = 0; q < NR; ++q) x[q] = *reinterpret_cast<const VT*>(Tj[q] + i * R);
+#pragma unroll
+          for (int q = 0; q < NR; ++q) {
+            const float* xf = reinterpret_cast<const float*>(&x[q]);
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[q][v] = fmaf(xf[v], h[v], acc[q][v]);
+          }
+        }
+      }
+      for (int o = 1; o < S; o <<= 1) {
+        const bool add = act && (sub & (2 * o - 1)) == 0 && sub + o < S;
+#pragma unroll
+        for (int q = 0; q < NR; ++q)
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            const float w = __shfl_down_sync(0xffffffffu, acc[q][v], o * Rb);
+            if (add) acc[q][v] += w;
+          }
+      }
+      if (act && sub == 0) {
+#pragma unroll
+        for (int q = 0; q < NR; ++q) {
+          const int jq = j + q * nwarp;
+          if (jq < j1) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) out[(long long)jq * R + r + v] = acc[q][v];
+          }
+        }
+      }
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256) k_b_mttv_first(const BTensor* __restrict__ ts,
                                                       const int4* __restrict__ items, int a) {
   const int4 it = items[blockIdx.x];
   const BTensor& t = ts[it.x];
   if (tensor_done(t)) return;
   const int R = t.R, N = t.N;
-  const int Ia = (int)t.dims[a];
-  const int E = Ia * R;
   int K = 1;
   for (int m = a + 1; m < N; ++m) K *= (int)t.dims[m];
   const int jb = t.first_jb[a];
   const int j0 = it.y * jb, j1 = min(K, j0 + jb);
-  const float* T = t.node[a];
   float* out = (a + 1 == N - 1) ? t.M : t.node[a + 1];
-  const float* Ha = t.H[a];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-  for (int rb = 0; rb < R; rb += 32) {
-    const int Rb = min(32, R - rb), S = 32 / Rb;
-    const int sub = lane / Rb, r = rb + lane - sub * Rb;
-    const bool act = sub < S;
-    for (int j = j0 + warp; j < j1; j += 2 * nwarp) {
-      const int j2 = j + nwarp;
-      const bool two = j2 < j1;
-      const float* Tj = T + (long long)j * E;
-      const float* Tk = T + (long long)(two ? j2 : j) * E;
-      float acc = 0.0f, acc2 = 0.0f;
-      if (act) {
-#pragma unroll 8
-        for (int i = sub; i < Ia; i += S) {
-          const float h = __ldg(Ha + i * R + r);
-          acc = fmaf(Tj[i * R + r], h, acc);
-          acc2 = fmaf(Tk[i * R + r], h, acc2);
-        }
-      }
-      for (int o = 1; o < S; o <<= 1) {
-        const float v = __shfl_down_sync(0xffffffffu, acc, o * Rb);
-        const float v2 = __shfl_down_sync(0xffffffffu, acc2, o * Rb);
-        if (act && (sub & (2 * o - 1)) == 0 && sub + o < S) {
-          acc += v;
-          acc2 += v2;
-        }
-      }
-      if (act && sub == 0) {
-        out[(long long)j * R + r] = acc;
-        if (two) out[(long long)j2 * R + r] = acc2;
-      }
-    }
-  }
+  // nodes and factors start on 16-byte boundaries
+  if ((R & 3) == 0) first_rows<4>(t.node[a], t.H[a], out, R, (int)t.dims[a], j0, j1);
+  else first_rows<1>(t.node[a], t.H[a], out, R, (int)t.dims[a], j0, j1);
 }
 
 // ---------------------------------------------------------- mode update --
@@ -1566,6 +1677,9 @@ cudaError_t batch_attributes_init() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_b_update<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)update_smem<64>());
+  const int fac = kBatchMaxI * kBatchMaxRank * (int)sizeof(float);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_init_mode, cudaFuncAttributeMaxDynamicSharedMemorySize, fac);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_init, cudaFuncAttributeMaxDynamicSharedMemorySize, fac);
   const int right = (2 * kTileFloats + kWsFloats) * (int)sizeof(float);
   const int left = (left_fixed_floats() + kBatchMaxI * kBatchMaxRank) * (int)sizeof(float);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_right<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, right);
@@ -1735,7 +1849,10 @@ cudaError_t b_launch_init(const BPlan& p, BTensor* ts, const int4* items, double
   if (p.count == 0) return cudaSuccess;
   if (p.alpha.count > 0)
     k_b_sumsq<<<p.alpha.count, 256, 0, st>>>(ts, items + p.alpha.off, alpha_part);
-  k_b_init<<<p.count, 256, 0, st>>>(ts, alpha_part, alpha_first);
+  if (p.max_factor < 1 || p.max_order < 1) return cudaErrorInvalidValue;  // b_plan_sizes not called
+  const size_t fac = (size_t)p.max_factor * sizeof(float);
+  k_b_init_mode<<<dim3((unsigned)p.count, (unsigned)p.max_order), 256, fac, st>>>(ts);
+  k_b_init<<<p.count, 256, fac, st>>>(ts, alpha_part, alpha_first);
   return cudaGetLastError();
 }
 

@@ -94,6 +94,8 @@ struct BPhase {
 struct BPlan {
   int count = 0, N = 0, rmax = 16, hs_floats = 0;
   int max_rows = 1;  // longest mode of any tensor of the batch
+  // elements of its largest factor and its highest order (0: not set yet)
+  int max_factor = 0, max_order = 0;
   std::vector<int4> items;
   BPhase alpha, pmr, pmr_red, pml;
   BPhase leaf[kMaxModes], leaf_red[kMaxModes], first[kMaxModes];
@@ -106,6 +108,9 @@ struct BPlan {
 // (sizes only when base is NULL) and fills the shape-derived fields of *d.
 size_t b_tensor_layout(int N, const int64_t* dims, int R, int fit_cap, BTensor* d, char* base);
 void b_build_plan(const BTensor* ts, int count, int N, BPlan* p);
+// p->max_rows, max_factor and max_order alone (b_build_plan calls it): what
+// b_launch_init needs of tensors of any orders beside its alpha items
+void b_plan_sizes(const BTensor* ts, int count, BPlan* p);
 
 cudaError_t batch_attributes_init();
 // alpha, normalisation, Grams and S of every tensor of the plan

@@ -317,6 +317,7 @@ cudaError_t init_new(nncp_server* s, const std::vector<Request*>& fresh) {
   }
   p.alpha.count = (int)p.items.size();
   p.alpha_first[fresh.size()] = p.alpha.count;
+  b_plan_sizes(ts.data(), (int)ts.size(), &p);
   cudaError_t e = ensure(&s->d_init_ts, &s->cap_init_ts, ts.size());
   if (e == cudaSuccess) e = ensure(&s->d_init_items, &s->cap_init_items, p.items.size());
   if (e == cudaSuccess) e = ensure(&s->d_alpha_part, &s->cap_alpha, p.items.size());
