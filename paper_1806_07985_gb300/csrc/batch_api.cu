@@ -523,15 +523,18 @@ nncp_status nncp_batch_run(nncp_batch* b, int max_iters, double tol, int* iters_
       return bfail(b, NNCP_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
     }
   }
-  int launched = 0, every = 4;
+  // with tol <= 0 only a non-finite fit stops a tensor before max_iters: no
+  // count is read back before the end of a long run
+  int launched = 0, every = tol > 0.0 ? 4 : 64;
   while (launched < max_iters) {
     const int n = std::min(every, max_iters - launched);
     for (int k = 0; k < n; ++k) BCK(cudaGraphLaunch(b->graph, b->work));
     launched += n;
+    if (launched >= max_iters) break;
     BCK(cudaMemcpyAsync(b->host_done, done, sizeof(int), cudaMemcpyDeviceToHost, b->work));
     BCK(cudaStreamSynchronize(b->work));
     if (b->host_done[0] >= b->count) break;
-    every = std::min(every * 2, 16);
+    every = tol > 0.0 ? std::min(every * 2, 16) : 64;
   }
   int* d_iters = at<int>(b, b->off_out_iters);
   double* d_fits = at<double>(b, b->off_out_fits);

@@ -73,6 +73,7 @@ struct nncp_ctx {
   int graph_kernels = 0;
   int* host_flags = nullptr;  // pinned
   double* host_dbl = nullptr; // pinned
+  double* host_lam = nullptr; // pinned, kMaxRank entries after host_dbl's 16
   bool initialised = false;   // nncp_solve_begin ran on the current state
   // nncp_mttkrp_cached: versions of the factors (bumped by nncp_factor_changed)
   // and, per tree node [half][depth], whether it holds a result and the
@@ -574,7 +575,8 @@ nncp_status nncp_create(int N, const int64_t* dims, int R, nncp_ctx** out) {
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMallocHost(&c->host_flags, 16 * sizeof(int));
-  if (e == cudaSuccess) e = cudaMallocHost(&c->host_dbl, 16 * sizeof(double));
+  if (e == cudaSuccess) e = cudaMallocHost(&c->host_dbl, (16 + kMaxRank) * sizeof(double));
+  if (e == cudaSuccess) c->host_lam = c->host_dbl + 16;
   if (e == cudaSuccess) e = kernel_attributes_init();
   if (e != cudaSuccess) {
     nncp_status s = cuda_fail(nullptr, e, "nncp_create");
@@ -834,34 +836,38 @@ nncp_status nncp_solve_bound(nncp_ctx* c, int max_iters, double tol, double* lam
   if ((s = begin_on_work(c)) != NNCP_OK) return s;
   if ((s = solve_init(c, tol)) != NNCP_OK) return s;
   if ((s = ensure_graph(c)) != NNCP_OK) return s;
-  int launched = 0, check_every = 4;
+  // with tol <= 0 only a non-finite fit stops a solve early, and what follows
+  // it changes nothing: no flag is read back before the end of a long run
+  int launched = 0, check_every = tol > 0.0 ? 4 : 64;
   while (launched < max_iters) {
     int batch = std::min(check_every, max_iters - launched);
     CK(launch_iterations(c, batch));
     launched += batch;
+    if (launched >= max_iters) break;
     CK(cudaMemcpyAsync(c->host_flags, c->st.flags, 4 * sizeof(int), cudaMemcpyDeviceToHost,
                        c->work));
     CK(cudaStreamSynchronize(c->work));
     if (c->host_flags[0]) break;
-    check_every = std::min(check_every * 2, 32);
+    check_every = tol > 0.0 ? std::min(check_every * 2, 32) : 64;
   }
+  // everything the call returns, in one round trip: the flags, the last fit
+  // (scalars[5]), lambda and the tensor-core error word
+  c->host_flags[12] = 0;
   CK(cudaMemcpyAsync(c->host_flags, c->st.flags, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->work));
+  CK(cudaMemcpyAsync(c->host_dbl, c->st.scalars + 5, sizeof(double), cudaMemcpyDeviceToHost, c->work));
+  if (lambda_out)
+    CK(cudaMemcpyAsync(c->host_lam, c->st.lam, c->R * sizeof(double), cudaMemcpyDeviceToHost, c->work));
+  if (c->tc.bytes)
+    CK(cudaMemcpyAsync(c->host_flags + 12, tc_error_word(c->tc), sizeof(int), cudaMemcpyDeviceToHost,
+                       c->work));
   CK(cudaStreamSynchronize(c->work));
   const int iters = c->host_flags[2];
-  if (lambda_out)
-    CK(cudaMemcpy(lambda_out, c->st.lam, c->R * sizeof(double), cudaMemcpyDeviceToHost));
-  double fit = 0.0;
-  if (iters > 0)
-    CK(cudaMemcpy(&fit, c->st.fits + (iters - 1), sizeof(double), cudaMemcpyDeviceToHost));
+  if (lambda_out) memcpy(lambda_out, c->host_lam, c->R * sizeof(double));
   if (iters_out) *iters_out = iters;
-  if (fit_out) *fit_out = fit;
+  if (fit_out) *fit_out = iters > 0 ? c->host_dbl[0] : 0.0;
   if ((s = end_on_work(c)) != NNCP_OK) return s;
-  if (c->tc.bytes) {
-    int tc_err = 0;
-    CK(cudaMemcpy(&tc_err, tc_error_word(c->tc), sizeof(int), cudaMemcpyDeviceToHost));
-    if (tc_err)
-      return fail(c, NNCP_ERR_TIMEOUT, "a tensor-core kernel gave up waiting (error word set)");
-  }
+  if (c->host_flags[12])
+    return fail(c, NNCP_ERR_TIMEOUT, "a tensor-core kernel gave up waiting (error word set)");
   if (c->host_flags[3]) return fail(c, NNCP_ERR_NUMERIC, "non-finite fit at iteration %d", iters);
   return NNCP_OK;
 }
