@@ -94,9 +94,15 @@ __device__ __forceinline__ void rows_block(float* __restrict__ H, const float* _
                    ((reinterpret_cast<uintptr_t>(H) | reinterpret_cast<uintptr_t>(M)) & 15) == 0;
   if (do_hals == 1) {
     // columns past R are zero; S is symmetric, so row r serves as column r
+#pragma unroll 4
     for (int e = tid; e < R * (RMAX / 4); e += kHalsThreads) {
       const int r = e / (RMAX / 4), c = 4 * (e - r * (RMAX / 4));
-      float4 v;
+      float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if ((R & 3) == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0) {
+        if (c < R) v = __ldg(reinterpret_cast<const float4*>(S + r * R + c));
+        *reinterpret_cast<float4*>(Ss + r * RMAX + c) = v;
+        continue;
+      }
       v.x = c < R ? __ldg(S + r * R + c) : 0.0f;
       v.y = c + 1 < R ? __ldg(S + r * R + c + 1) : 0.0f;
       v.z = c + 2 < R ? __ldg(S + r * R + c + 2) : 0.0f;
@@ -303,6 +309,21 @@ __device__ void record_fit(SolveState st, double beta, double gamma) {
 }
 
 
+// sqrt(g) and its reciprocal (0 for g = 0) in float64, refined from a float32
+// estimate as above where float32's range allows, by the plain functions elsewhere
+__device__ __forceinline__ void norm_f64(double g, double* root, double* rinv) {
+  if (g > 1e-30 && g < 1e30) {
+    double r = (double)rsqrtf((float)g);
+    r = r * (1.5 - 0.5 * g * r * r);
+    r = r * (1.5 - 0.5 * g * r * r);
+    *rinv = r;
+    *root = g * r;
+  } else {
+    *root = sqrt(g);
+    *rinv = *root > 0.0 ? 1.0 / *root : 0.0;
+  }
+}
+
 // Column sums over the row blocks' partials: part(b) = W^T W of block b, pitch
 // doubles apart.  A warp per output over many blocks (fixed butterfly), a
 // thread per output over few.
@@ -318,6 +339,36 @@ __device__ __forceinline__ double sum_blocks_warp(const double* p, long long pit
 #pragma unroll 4
   for (int b = threadIdx.x & 31; b < nblocks; b += 32) s += p[b * pitch];
   return warp_sum_d(s);
+}
+
+// This CTA's share of H(i, r) /= c(r) (0 where c = 0), and of U when given: 32-bit
+// indices, the column kept by addition (a 64-bit remainder per element cost more
+// than the row it scaled).
+template <typename F>
+__device__ __forceinline__ void rows_share(int tot, int R, F f) {
+  const unsigned stride = gridDim.x * blockDim.x;
+  const int dr = (int)(stride % (unsigned)R);
+  unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  int r = (int)(t % (unsigned)R);
+#pragma unroll 4
+  for (; t < (unsigned)tot; t += stride) {
+    f(t, r);
+    r += dr;
+    if (r >= R) r -= R;
+  }
+}
+__device__ __forceinline__ void scale_rows(float* H, float* U, int tot, int R, const float* cf) {
+  if (U)
+    rows_share(tot, R, [&](unsigned t, int r) {
+      const float c = cf[r];
+      H[t] = c > 0.0f ? H[t] / c : 0.0f;
+      U[t] = c > 0.0f ? U[t] / c : 0.0f;
+    });
+  else
+    rows_share(tot, R, [&](unsigned t, int r) {
+      const float c = cf[r];
+      H[t] = c > 0.0f ? H[t] / c : 0.0f;
+    });
 }
 
 // The rest of a mode update after k_hals_gram, over gridDim.x CTAs: every CTA
@@ -345,8 +396,9 @@ k_finish(float* __restrict__ H, long long In, int R, int N, int n, int next_mode
   const long long pitch = R2 + 1;
   const bool few = nblocks <= kFewBlocks;
   auto column = [&](int r, double g) {
-    const double v = sqrt(g);
-    cinv[r] = v > 0.0 ? 1.0 / v : 0.0;
+    double v, vi;
+    norm_f64(g, &v, &vi);
+    cinv[r] = vi;
     cf[r] = (float)v;
     if (blockIdx.x == 0) st.lam[r] = v;
   };
@@ -385,12 +437,8 @@ k_finish(float* __restrict__ H, long long In, int R, int N, int n, int next_mode
     }
   }
   // this CTA's share of H = W / lambda
-  const long long tot = In * R, stride = (long long)gridDim.x * T;
-  for (long long t = (long long)blockIdx.x * T + tid; t < tot; t += stride) {
-    const float c = cf[t % R];
-    H[t] = c > 0.0f ? H[t] / c : 0.0f;
-    if (U) U[t] = c > 0.0f ? U[t] / c : 0.0f;  // ADMM dual, same frame as H
-  }
+  // (I_n R < 2^31; the ADMM dual in the same frame as H)
+  scale_rows(H, U, (int)(In * R), R, cf);
   if (is_last) {
     gamma = warp_sum_d(gamma);
     if (lane == 0) red[warp] = gamma;
@@ -451,9 +499,10 @@ k_init_finish(const __grid_constant__ InitArgs a, SolveState st, double tol,
   bool few = true;
   for (int n = 0; n < N; ++n) few = few && a.first[n + 1] - a.first[n] <= kFewBlocks;
   auto column = [&](int x, double g) {
-    const double v = sqrt(g);
+    double v, vi;
+    norm_f64(g, &v, &vi);
     cn[x] = v;
-    cinv[x] = v > 0.0 ? 1.0 / v : 0.0;
+    cinv[x] = vi;
     cf[x] = (float)v;
   };
   if (few) {
@@ -505,17 +554,15 @@ k_init_finish(const __grid_constant__ InitArgs a, SolveState st, double tol,
     }
   }
   // rows of every factor; the ADMM duals start at zero
-  const long long stride = (long long)gridDim.x * T;
   for (int n = 0; n < N; ++n) {
-    const long long tot = a.rows[n] * R;
     float* H = a.H[n];
     float* U = a.U[n];
     const float* c = cf + n * R;
-    for (long long t = (long long)blockIdx.x * T + tid; t < tot; t += stride) {
-      const float v = c[t % R];
+    rows_share((int)(a.rows[n] * R), R, [&](unsigned t, int r) {
+      const float v = c[r];
       H[t] = v > 0.0f ? H[t] / v : 0.0f;
       U[t] = 0.0f;
-    }
+    });
   }
 }
 
@@ -2131,8 +2178,8 @@ cudaError_t launch_update_cluster(float* H, const float* M, int64_t In, int R, i
 
 cudaError_t launch_finish(float* H, int64_t In, int R, int N, int n, int next_mode, int is_last,
                           SolveState st, double* gscr, cudaStream_t stream, float* U) {
-  // about 4096 row elements per CTA, and enough CTAs for the R x R outputs
-  const int64_t want = std::max<int64_t>(((int64_t)In * R + 4095) / 4096, ((int64_t)R * R + 511) / 512);
+  // about 1024 row elements per CTA, and enough CTAs for the R x R outputs
+  const int64_t want = std::max<int64_t>(((int64_t)In * R + 1023) / 1024, ((int64_t)R * R + 255) / 256);
   const int grid = (int)std::min<int64_t>(want, kFinishMax);
   return launch_kernel(k_finish, dim3(grid), dim3(kFinishThreads), 0, stream, H, (long long)In, R, N,
                        n, next_mode, hals_gram_blocks(In), is_last, st, U, gscr);
@@ -2185,7 +2232,7 @@ cudaError_t launch_solve_init(int N, const int64_t* dims, int R, float* const* H
   k<<<a.first[N], kHalsThreads, rows_smem(R, false), stream>>>(a);
   int64_t elems = 0;
   for (int n = 0; n < N; ++n) elems += dims[n] * R;
-  const int64_t want = std::max<int64_t>((elems + 4095) / 4096, ((int64_t)R * R + 511) / 512);
+  const int64_t want = std::max<int64_t>((elems + 1023) / 1024, ((int64_t)R * R + 255) / 256);
   const int grid = (int)std::min<int64_t>(want, kFinishMax);
   k_init_finish<<<grid, kFinishThreads, (size_t)N * R * 20, stream>>>(a, st, tol, alpha_part, nalpha);
   return cudaGetLastError();
