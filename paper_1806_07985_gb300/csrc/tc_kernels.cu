@@ -9,15 +9,17 @@
 //   contract_slow: out(i, r) = sum_j X[i + IL*j] K(j, r)   (M = IL rows, K = IR)
 // contract_fast tiles (128 output rows x 64 contraction elements per stage)
 // arrive K-major from TMA with the 128-byte swizzle; contract_slow tiles arrive
-// MN-major (no swizzle).  SPLIT_BF16X3 converter threads read one row of A each
-// and write its bf16 hi and lo parts into a ring of A stages in tensor memory
-// (tcgen05.st, one TMEM lane per row), from which the MMA takes A; the TMA stage
-// is released as soon as it has been read.  The other modes hand A to the MMA
-// from shared memory, K-major with the 128-byte swizzle: TF32 K-major tiles
-// directly, everything else converted in place (the converted tile has the size
-// of its source, so each converter thread reads its share into registers, a
-// named barrier separates the reads from the writes, and the result overwrites
-// the TMA stage).  Precision modes:
+// MN-major (bf16: two of 64 outputs with the 128-byte swizzle; float32: no
+// swizzle).  SPLIT_BF16X3 converter threads read one row of A each and write its
+// bf16 hi and lo parts into a ring of A stages in tensor memory (tcgen05.st, one
+// TMEM lane per row), from which the MMA takes A; the TMA stage is released as
+// soon as it has been read.  The other modes hand A to the MMA
+// from shared memory with the 128-byte swizzle: TF32 K-major tiles and bf16
+// tiles of either kind directly (the MMA takes bf16 A MN-major too; transposing
+// it by 2-byte shared-memory reads had held contract_slow of a 600 x 404 x 330
+// bf16 tensor at R = 40 to 116 us on a GB300); TF32 MN-major tiles transposed in
+// place (each converter thread reads its share into registers, a named barrier
+// separates the reads from the writes).  Precision modes:
 //   TF32         kind::tf32 on the float32 tensor (direct when K-major);
 //   SPLIT_BF16X3 x = hi + lo in bf16, K = Khi + Klo: D = [hi*Khi | hi*Klo +
 //                lo*Khi] (three products in two float32 TMEM accumulators,
@@ -100,6 +102,7 @@ struct TcParams {
   int mode;
   int contract_fast;
   int direct;  // MMA reads the TMA stage (no converter)
+  int a_mn;    // ... MN-major (bf16 tensor, contract_slow)
   int bf16x;   // tensor stored as bf16
   int b_resident;  // every unit spans the whole contraction: B formed once per CTA
   // Stages accumulated in one tensor-memory accumulator before it is added into
@@ -233,6 +236,20 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t addr) {
   return d;
 }
 
+// The same swizzle, MN-major: rows of 64 bf16 outputs (128 bytes) per contraction
+// element, eight elements 1024 bytes apart (SBO), the tile's second 64 outputs
+// 8192 bytes on (LBO).
+__device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr >> 4) & 0x3FFFu);
+  d |= (uint64_t)(8192 >> 4) << 16;       // LBO
+  d |= (uint64_t)(1024 >> 4) << 32;       // SBO
+  d |= (uint64_t)1 << 46;                 // descriptor version
+  d |= (uint64_t)2 << 61;                 // 128-byte swizzle
+  return d;
+}
+constexpr uint32_t kIdescAMn = 1u << 15;  // A is MN-major
+
 // Instruction descriptor: D float32, A/B type `ab` (1 = bf16 under kind::f16,
 // 2 = tf32 under kind::tf32), both K-major, M = 128, N = n.
 __host__ __device__ constexpr uint32_t make_idesc(uint32_t ab, uint32_t n) {
@@ -343,12 +360,6 @@ __device__ __forceinline__ float4 lds128(uint32_t addr) {
 __device__ __forceinline__ float lds32(uint32_t addr) {
   float v;
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ uint32_t lds16(uint32_t addr) {
-  uint16_t v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
   return v;
 }
 
@@ -516,6 +527,9 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
               tma_load_2d(dst, &tmap, k0, m0, raw_full(sf), pol);
               tma_load_2d(dst + 16384, &tmap, k0 + 32, m0, raw_full(sf), pol);
             }
+          } else if (p.a_mn) {
+            tma_load_2d(dst, &tmap, m0, k0, raw_full(sf), pol);
+            tma_load_2d(dst + 8192, &tmap, m0 + 64, k0, raw_full(sf), pol);
           } else {
             tma_load_2d(dst, &tmap, m0, k0, raw_full(sf), pol);
           }
@@ -539,9 +553,8 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
       uint32_t pha = 0, phb = 0;
       const int nA = kSF;
       bool ok = true;
-      const bool split = p.mode == NNCP_SPLIT_BF16X3;
       const bool tf32 = p.mode == NNCP_TF32;
-      const uint32_t idesc_full = tf32 ? make_idesc(2, Rp) : make_idesc(1, 2 * Rp);
+      const uint32_t idesc_full = tf32 ? make_idesc(2, Rp) : make_idesc(1, 2 * Rp) | (p.a_mn ? kIdescAMn : 0u);
       const uint32_t idesc_hi = make_idesc(1, Rp);
       if (p.b_resident && n_units > blockIdx.x && !mbar_wait(b_full(0), 0, abort_flag, p.err))
         ok = false;
@@ -604,10 +617,10 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
             } else {
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk) {
-                const uint32_t o = kk * 32;
-                mma_f16(d, sw128_desc(a + o), sw128_desc(b + o), idesc_full,
-                        (sp > 0 || kk > 0) ? 1u : 0u);
-                if (split) mma_f16(d, sw128_desc(a + 16384 + o), sw128_desc(b + o), idesc_hi, 1u);
+                // 16 contraction elements: 32 bytes of a K-major row, 16 rows of an
+                // MN-major tile
+                const uint64_t ad = p.a_mn ? sw128_mn_desc(a + kk * 2048) : sw128_desc(a + kk * 32);
+                mma_f16(d, ad, sw128_desc(b + kk * 32), idesc_full, (sp > 0 || kk > 0) ? 1u : 0u);
               }
             }
             mma_commit(aempty);
@@ -859,14 +872,12 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
   } else {
     // ---------------------------------------- converters + epilogue --
     const int ct = threadIdx.x - kWarpConv * 32;  // 0..255
-    // row m and contraction half kh (elements 32 kh .. 32 kh + 31).  K-major
-    // sources: the two halves of a row in lanes l and l + 16 of one warp, eight
-    // consecutive rows per quarter-warp (conflict-free 16-byte reads).  MN-major
-    // sources: 32 consecutive rows per warp (conflict-free 4-byte reads).
-    // (split-BF16x3 writes A to tensor memory: row m must sit in this warp's lane
-    // quarter, so 32 consecutive rows per warp for both sources)
-    const int m = (p.contract_fast && !a_tmem) ? ((ct >> 5) * 16 + (ct & 15)) : (ct & 127);
-    const int kh = (p.contract_fast && !a_tmem) ? ((ct >> 4) & 1) : (ct >> 7);
+    // row m and contraction half kh (elements 32 kh .. 32 kh + 31): 32
+    // consecutive rows per warp, for conflict-free reads of an MN-major source
+    // and because split-BF16x3 writes row m of A into this warp's lane quarter of
+    // tensor memory
+    const int m = ct & 127;
+    const int kh = ct >> 7;
     const int q = warp & 3;                       // TMEM lane quarter of this warp
     const bool two = p.mode != NNCP_TF32;
     int sf = 0;
@@ -996,70 +1007,28 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
         }
       }
       for (int s = 0; s < w.nk && !p.direct && !SPLIT; ++s) {
+        // TF32, contract_slow: transpose the MN-major stage in place
         const bool got = mbar_wait(raw_full(sf), phf, abort_flag, p.err);
         const uint32_t st = raw0 + sf * kRawBytes;
-        // read phase: this thread's 32 source elements of row m, half kh
+        // read phase: this thread's 32 source elements of row m, half kh (row j
+        // of the stage holds 128 consecutive i, 512 B)
         float x[32];
         if (got) {
-          if (p.mode == NNCP_BF16_STORED) {
-            // MN-major bf16 source: row j holds 128 consecutive i (256 B)
 #pragma unroll
-            for (int e = 0; e < 32; ++e)
-              x[e] = __uint_as_float(lds16(st + (32 * kh + e) * 256 + m * 2));
-          } else if (p.contract_fast) {
-            // K-major fp32 source: sub-tile kh, row m, its 8 chunks
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const float4 a = lds128(sw128_chunk(st + kh * 16384, m, c));
-              x[4 * c] = a.x; x[4 * c + 1] = a.y; x[4 * c + 2] = a.z; x[4 * c + 3] = a.w;
-            }
-          } else {
-            // MN-major fp32 source: row j holds 128 consecutive i (512 B)
-#pragma unroll
-            for (int e = 0; e < 32; ++e) x[e] = lds32(st + (32 * kh + e) * 512 + m * 4);
-          }
+          for (int e = 0; e < 32; ++e) x[e] = lds32(st + (32 * kh + e) * 512 + m * 4);
         }
-        // In place: every element is read before any is overwritten.  A K-major
-        // source row m is overwritten only by row m's own output, whose two halves
-        // sit in this warp; an MN-major source row is spread over all output rows,
-        // so the whole converter group must have read first.
-        if (p.contract_fast) {
-          if (!__all_sync(0xffffffffu, got)) {
-            ok = false;
-            break;
-          }
-        } else if (bar_red_or(2, kConvThreads, !got)) {
+        // a source row is spread over all output rows, so the whole converter
+        // group must have read before any of it is overwritten
+        if (bar_red_or(2, kConvThreads, !got)) {
           ok = false;
           break;
         }
-        if (p.mode == NNCP_SPLIT_BF16X3) {
-          // hi tile at +0, lo tile at +16 KB; chunks 4 kh .. 4 kh + 3 of row m
+        // K-major fp32: sub-tile kh, chunks 0..7 of row m
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            uint32_t hi[4], lo[4];
-            split8(x + 8 * g, hi, lo);
-            sts128(sw128_chunk(st, m, 4 * kh + g), hi[0], hi[1], hi[2], hi[3]);
-            sts128(sw128_chunk(st + 16384, m, 4 * kh + g), lo[0], lo[1], lo[2], lo[3]);
-          }
-        } else if (p.mode == NNCP_TF32) {
-          // K-major fp32: sub-tile kh, chunks 0..7 of row m
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            sts128(sw128_chunk(st + kh * 16384, m, c), __float_as_uint(x[4 * c]),
-                   __float_as_uint(x[4 * c + 1]), __float_as_uint(x[4 * c + 2]),
-                   __float_as_uint(x[4 * c + 3]));
-        } else {
-          // K-major bf16: chunks 4 kh .. 4 kh + 3 of row m
-#pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            uint32_t w4[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              w4[e] = (__float_as_uint(x[8 * g + 2 * e]) & 0xFFFFu) |
-                      (__float_as_uint(x[8 * g + 2 * e + 1]) << 16);
-            sts128(sw128_chunk(st, m, 4 * kh + g), w4[0], w4[1], w4[2], w4[3]);
-          }
-        }
+        for (int c = 0; c < 8; ++c)
+          sts128(sw128_chunk(st + kh * 16384, m, c), __float_as_uint(x[4 * c]),
+                 __float_as_uint(x[4 * c + 1]), __float_as_uint(x[4 * c + 2]),
+                 __float_as_uint(x[4 * c + 3]));
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) mbar_arrive(conv_full(sf));
@@ -1251,9 +1220,9 @@ cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, i
     box[1] = 128;              // output rows
     swz = CU_TENSOR_MAP_SWIZZLE_128B;
   } else {
-    box[0] = 128;              // output rows (contiguous)
-    box[1] = kKC;              // contraction elements
-    swz = CU_TENSOR_MAP_SWIZZLE_NONE;
+    box[0] = bf16x ? 64 : 128;  // output rows (contiguous)
+    box[1] = kKC;               // contraction elements
+    swz = bf16x ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE;
   }
   cuuint32_t estride[2] = {1, 1};
   CUresult r = g_encode(&map, bf16x ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
@@ -1267,7 +1236,8 @@ cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, i
   p.mode = precision;
   p.contract_fast = contract_fast;
   p.bf16x = bf16x;
-  p.direct = contract_fast && precision != NNCP_SPLIT_BF16X3;
+  p.a_mn = bf16x && !contract_fast;
+  p.direct = (contract_fast && precision != NNCP_SPLIT_BF16X3) || p.a_mn;
   p.seg = precision == NNCP_SPLIT_BF16X3 ? kSegStages : (1 << 30);
   p.M = pl.M;
   p.K = pl.K;
