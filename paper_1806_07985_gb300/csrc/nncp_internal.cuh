@@ -24,6 +24,25 @@ __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// ---- packed float32 pairs ----------------------------------------------------------
+typedef unsigned long long u64;
+// two float32 FMAs, each rounded to nearest as fmaf
+__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c) {
+  u64 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ u64 pack2(float x, float y) {
+  u64 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(u64 v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+
 // Launches k(args...) on st: with programmatic stream serialization while st is
 // being captured into a graph, as an ordinary launch otherwise.  Only kernels
 // that follow the pdl_wait() rule above are launched through this.

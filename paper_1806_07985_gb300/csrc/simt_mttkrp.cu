@@ -134,24 +134,6 @@ __device__ __forceinline__ void cpa4(uint32_t dst, const float* src) {
 }
 __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 
-typedef unsigned long long u64;
-
-// two float32 FMAs, each rounded to nearest as fmaf
-__device__ __forceinline__ u64 ffma2(u64 a, u64 b, u64 c) {
-  u64 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ u64 pack2(float x, float y) {
-  u64 d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
-  return d;
-}
-__device__ __forceinline__ float2 unpack2(u64 v) {
-  float2 f;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
-  return f;
-}
 
 // first step of run c over the cut tiles
 __device__ __forceinline__ long long run_start(long long c, long long U2, int G2) {

@@ -1316,15 +1316,7 @@ k_probe_ffma(int reps, float seed, float* sink) {
   if (s == 12345.678f) sink[0] = s;  // keeps the chains live
 }
 
-// The same with packed pairs: fma.rn.f32x2 performs two float32 FMAs (each
-// rounded to nearest, as fmaf) per instruction.
-__device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b,
-                                                    unsigned long long c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-
+// The same with packed pairs: fma.rn.f32x2 performs two float32 FMAs per instruction.
 __global__ void __launch_bounds__(kProbeThreads)
 k_probe_ffma2(int reps, float seed, float* sink) {
   unsigned long long a[kProbeChains];

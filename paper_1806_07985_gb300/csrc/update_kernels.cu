@@ -69,166 +69,327 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // a row per quad gives four times the threads that a row per thread would, and
 // one of S's rows is read for eight matrix rows at once.  (A warp per row with a
 // five-step shuffle sum per column took 285 us for 220 rows at R = 100 on a GB300.)
+// Past 64 ranks shared memory bounds that form: every thread reads R / 4 floats of
+// S per column and row, at 128 bytes per cycle and SM.  There sixteen lanes share
+// four rows, keep the residuals m - S w of their eight columns of each, and a
+// column step adds the change of w_r times their part of S's row r, read once for
+// the four rows (220 rows at R = 100: quads and dot products 48 us, residuals with
+// one row per eight lanes 44 us, this 38 us, and with S and H on their way before
+// the wait for the predecessor 32 us).
 template <int RMAX>
 struct RowsCfg {
-  static constexpr int NJ = RMAX / 16;       // chunks of four columns per lane
+  static constexpr int LANES = RMAX > 64 ? 16 : 4;         // lanes per row ...
+  static constexpr int ROWS = LANES * kRowsPerBlock / kHalsThreads;  // ... and rows per thread
+  static constexpr int CH = 4 * LANES;       // columns of a chunk, four per lane
+  static constexpr int NJ = RMAX / CH;       // chunks
   static constexpr int RP = RMAX + 4;        // padded row stride in shared memory
   static constexpr int TB = RMAX <= 32 ? 2 : 4;  // W^T W tile of a thread
 };
+
+__device__ __forceinline__ void cp_async16(float* smem_dst, const float* gmem_src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
+}
+// up to four of the n floats at p (zero past them)
+__device__ __forceinline__ float4 load_rank4(const float* p, int n, bool vec) {
+  if (vec) return *reinterpret_cast<const float4*>(p);
+  float4 v;
+  v.x = p[0];
+  v.y = n > 1 ? p[1] : 0.0f;
+  v.z = n > 2 ? p[2] : 0.0f;
+  v.w = n > 3 ? p[3] : 0.0f;
+  return v;
+}
+
+// One row's HALS sweep over the lanes of a quad (lane q): column r = dot product,
+// update; columns in order.
+template <int RMAX>
+__device__ __forceinline__ void sweep_quads(float (&w)[RMAX / 16][4], const float (&m)[RMAX / 16][4],
+                                            const float* Ss, const float* srr, const float* sinv,
+                                            int R, int q) {
+  constexpr int NJ = RMAX / 16;
+  const int nb4 = (R + 3) >> 2;
+#pragma unroll 1
+  for (int r4 = 0; r4 < nb4; ++r4) {
+    const int jr = r4 >> 2;
+    const bool own = (r4 & 3) == q;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int r = 4 * r4 + t;
+      if (r >= R) break;
+      const float4* srow = reinterpret_cast<const float4*>(Ss + r * RMAX) + q;
+      float d0 = 0.0f, d1 = 0.0f, d2 = 0.0f, d3 = 0.0f;
+      float wr = 0.0f, mr = 0.0f;
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const float4 sv = srow[4 * j];
+        d0 = fmaf(w[j][0], sv.x, d0);
+        d1 = fmaf(w[j][1], sv.y, d1);
+        d2 = fmaf(w[j][2], sv.z, d2);
+        d3 = fmaf(w[j][3], sv.w, d3);
+        if (j == jr) {
+          wr = w[j][t];
+          mr = m[j][t];
+        }
+      }
+      float dot = (d0 + d1) + (d2 + d3);
+      dot += __shfl_xor_sync(0xffffffffu, dot, 1);
+      dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+      // (m - dot) / s_rr: the product with the reciprocal, corrected once
+      const float num = mr - dot, si = sinv[r];
+      float step = num * si;
+      step = fmaf(fmaf(-srr[r], step, num), si, step);
+      const float upd = fmaxf(0.0f, wr + step);
+      if (own && si != 0.0f) {  // S_rr = 0: column left as it is
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+          if (j == jr) w[j][t] = upd;
+      }
+    }
+  }
+}
+
+// The same sweep with residuals for the ROWS rows of a group of LANES lanes: res =
+// S w - m of the lane's columns is kept up to date, so a column step is the update
+// by its owner, a shuffle of the change and packed FMAs.  Wrow: ROWS padded rows of
+// shared memory for these lanes.
+template <int RMAX>
+__device__ __forceinline__ void sweep_residuals(
+    float (&w)[RowsCfg<RMAX>::ROWS][RowsCfg<RMAX>::NJ][4],
+    const float (&m)[RowsCfg<RMAX>::ROWS][RowsCfg<RMAX>::NJ][4], const float* Ss, float* Wrow,
+    const float* srr, const float* sinv, int R, int q) {
+  using C = RowsCfg<RMAX>;
+  constexpr int NJ = C::NJ, RP = C::RP, LANES = C::LANES, ROWS = C::ROWS, CH = C::CH;
+  u64 res[ROWS][2 * NJ];
+#pragma unroll
+  for (int k = 0; k < ROWS; ++k)
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      *reinterpret_cast<float4*>(Wrow + k * RP + CH * j + 4 * q) =
+          make_float4(w[k][j][0], w[k][j][1], w[k][j][2], w[k][j][3]);
+      res[k][2 * j] = pack2(-m[k][j][0], -m[k][j][1]);
+      res[k][2 * j + 1] = pack2(-m[k][j][2], -m[k][j][3]);
+    }
+  __syncwarp();
+  // sixteen columns of w at a time, so that no chain of roundings is longer than
+  // 16 + R / 16 (columns past R are zero)
+  const float* scol = Ss + 4 * q;
+  const u64 one = pack2(1.0f, 1.0f);
+#pragma unroll 1
+  for (int r0 = 0; r0 < R; r0 += 16) {
+    u64 run[ROWS][2 * NJ];
+#pragma unroll
+    for (int k = 0; k < ROWS; ++k)
+#pragma unroll
+      for (int j = 0; j < 2 * NJ; ++j) run[k][j] = 0;
+    const int r1 = min(R, r0 + 16);
+#pragma unroll 1
+    for (int r = r0; r < r1; r += 4) {
+      float wv[ROWS][4];
+#pragma unroll
+      for (int k = 0; k < ROWS; ++k)
+        *reinterpret_cast<float4*>(wv[k]) = *reinterpret_cast<const float4*>(Wrow + k * RP + r);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        if (r + t >= r1) break;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          const ulonglong2 sv = *reinterpret_cast<const ulonglong2*>(scol + (r + t) * RMAX + CH * j);
+#pragma unroll
+          for (int k = 0; k < ROWS; ++k) {
+            const u64 w2 = pack2(wv[k][t], wv[k][t]);
+            run[k][2 * j] = ffma2(w2, sv.x, run[k][2 * j]);
+            run[k][2 * j + 1] = ffma2(w2, sv.y, run[k][2 * j + 1]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < ROWS; ++k)
+#pragma unroll
+      for (int j = 0; j < 2 * NJ; ++j) res[k][j] = ffma2(run[k][j], one, res[k][j]);
+  }
+  __syncwarp();
+  // column r = CH jr + 4 own + t
+#pragma unroll
+  for (int jr = 0; jr < NJ; ++jr) {
+#pragma unroll 1
+    for (int own = 0; own < LANES; ++own) {
+      if (CH * jr + 4 * own >= R) break;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int r = CH * jr + 4 * own + t;
+        if (r >= R) break;
+        const float si = sinv[r], sd = srr[r];
+        ulonglong2 sv[NJ];
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+          sv[j] = *reinterpret_cast<const ulonglong2*>(scol + r * RMAX + CH * j);
+#pragma unroll
+        for (int k = 0; k < ROWS; ++k) {
+          const float2 rr = unpack2(res[k][2 * jr + (t >> 1)]);
+          const float num = -((t & 1) ? rr.y : rr.x), wr = w[k][jr][t];
+          // (m - S w) / s_rr: the product with the reciprocal, corrected once
+          float step = num * si;
+          step = fmaf(fmaf(-sd, step, num), si, step);
+          const float upd = si != 0.0f ? fmaxf(0.0f, wr + step) : wr;  // S_rr = 0: left as it is
+          const float d = __shfl_sync(0xffffffffu, upd - wr, own, LANES);
+          if (q == own) w[k][jr][t] = upd;
+          const u64 d2 = pack2(d, d);
+#pragma unroll
+          for (int j = 0; j < NJ; ++j) {
+            res[k][2 * j] = ffma2(d2, sv[j].x, res[k][2 * j]);
+            res[k][2 * j + 1] = ffma2(d2, sv[j].y, res[k][2 * j + 1]);
+          }
+        }
+      }
+    }
+  }
+}
 
 template <int RMAX>
 __device__ __forceinline__ void rows_block(float* __restrict__ H, const float* __restrict__ M,
                                            long long In, int R, const float* __restrict__ S,
                                            const double* __restrict__ lam, double* __restrict__ gp,
-                                           int do_hals, int block, int nblocks, float* sm,
-                                           bool write_beta = true) {
+                                           const int* flags, int do_hals, int block, int nblocks,
+                                           float* sm, bool write_beta = true) {
   using C = RowsCfg<RMAX>;
-  constexpr int NJ = C::NJ, RP = C::RP;
+  constexpr int NJ = C::NJ, RP = C::RP, LANES = C::LANES, ROWS = C::ROWS, CH = C::CH;
   float* Ws = sm;                               // kRowsPerBlock x RP
   float* Ss = Ws + kRowsPerBlock * RP;          // R x RMAX (sweeps only)
   __shared__ double wbeta[kHalsThreads / 32];
   __shared__ float lamf[RMAX], srr_s[RMAX], sinv[RMAX];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int q = tid & 3, row = tid >> 2;
+  const int q = tid % LANES, rowt = ROWS * (tid / LANES);  // first of the thread's rows
   const bool vec = (R & 3) == 0 &&
                    ((reinterpret_cast<uintptr_t>(H) | reinterpret_cast<uintptr_t>(M)) & 15) == 0;
-  if (do_hals == 1) {
+  // Everything but M is written two or more kernels earlier when W comes from H here
+  // (see k_update_cluster), so it is on its way before the wait for the predecessor.
+  if (do_hals != 1) {
+    pdl_wait();
+    pdl_trigger();
+    if (flags && flags[0]) return;
+  } else {
     // columns past R are zero; S is symmetric, so row r serves as column r
+    const bool svec = (R & 3) == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0;
 #pragma unroll 4
     for (int e = tid; e < R * (RMAX / 4); e += kHalsThreads) {
       const int r = e / (RMAX / 4), c = 4 * (e - r * (RMAX / 4));
-      float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if ((R & 3) == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0) {
-        if (c < R) v = __ldg(reinterpret_cast<const float4*>(S + r * R + c));
-        *reinterpret_cast<float4*>(Ss + r * RMAX + c) = v;
+      float* d = Ss + r * RMAX + c;
+      if (svec && c < R) {
+        cp_async16(d, S + r * R + c);
         continue;
       }
+      float4 v;
       v.x = c < R ? __ldg(S + r * R + c) : 0.0f;
       v.y = c + 1 < R ? __ldg(S + r * R + c + 1) : 0.0f;
       v.z = c + 2 < R ? __ldg(S + r * R + c + 2) : 0.0f;
       v.w = c + 3 < R ? __ldg(S + r * R + c + 3) : 0.0f;
-      *reinterpret_cast<float4*>(Ss + r * RMAX + c) = v;
+      *reinterpret_cast<float4*>(d) = v;
     }
-    for (int r = tid; r < R; r += kHalsThreads) {
-      const float d = __ldg(S + r * R + r);
-      srr_s[r] = d;
-      sinv[r] = d != 0.0f ? 1.0f / d : 0.0f;
-      lamf[r] = (float)lam[r];
-    }
-    __syncthreads();
   }
   constexpr int TB = C::TB;
-  const int nb4 = (R + 3) >> 2, nt = (R + TB - 1) / TB, tiles = nt * nt;
+  const int nt = (R + TB - 1) / TB;
+  // past 64 ranks the tiles on and above the diagonal only (the rest are mirrored):
+  // row f of them and row nt - 1 - f together are nt + 1 tiles
+  constexpr bool kHalf = RMAX > 64;
+  const int tiles = kHalf ? (nt + 1) / 2 * (nt + 1) : nt * nt;
   double beta = 0.0;
   bool first = true;
   for (long long row0 = (long long)block * kRowsPerBlock; row0 < In;
        row0 += (long long)nblocks * kRowsPerBlock) {
     const int nrows = (int)min((long long)kRowsPerBlock, In - row0);
-    const long long i = row0 + row;
-    const bool in = row < nrows;
-    float w[NJ][4], m[NJ][4];
+    float w[ROWS][NJ][4], m[ROWS][NJ][4];
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const int c = 16 * j + 4 * q;
-      float4 h = make_float4(0.0f, 0.0f, 0.0f, 0.0f), mm = h;
-      if (in && c < R) {
-        const float* hp = H + i * R + c;
-        const float* mp = M + i * R + c;
-        if (vec) {
-          h = *reinterpret_cast<const float4*>(hp);
-          if (do_hals) mm = *reinterpret_cast<const float4*>(mp);
-        } else {
-          h.x = hp[0];
-          if (c + 1 < R) h.y = hp[1];
-          if (c + 2 < R) h.z = hp[2];
-          if (c + 3 < R) h.w = hp[3];
-          if (do_hals) {
-            mm.x = mp[0];
-            if (c + 1 < R) mm.y = mp[1];
-            if (c + 2 < R) mm.z = mp[2];
-            if (c + 3 < R) mm.w = mp[3];
-          }
-        }
-      }
-      w[j][0] = h.x; w[j][1] = h.y; w[j][2] = h.z; w[j][3] = h.w;
-      m[j][0] = mm.x; m[j][1] = mm.y; m[j][2] = mm.z; m[j][3] = mm.w;
+    for (int kj = 0; kj < ROWS * NJ; ++kj) {
+      const int k = kj / NJ, j = kj % NJ;
+      const long long i = row0 + rowt + k;
+      const bool in = rowt + k < nrows;
+      const int c = CH * j + 4 * q;
+      const float4 h = in && c < R ? load_rank4(H + i * R + c, R - c, vec) : float4{};
+      w[k][j][0] = h.x; w[k][j][1] = h.y; w[k][j][2] = h.z; w[k][j][3] = h.w;
     }
+    if (first && do_hals == 1) {
+      for (int r = tid; r < R; r += kHalsThreads) {
+        const float d = __ldg(S + r * R + r);
+        srr_s[r] = d;
+        sinv[r] = d != 0.0f ? 1.0f / d : 0.0f;
+        lamf[r] = (float)lam[r];
+      }
+      pdl_wait();
+      pdl_trigger();
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+      if (flags && flags[0]) return;
+    }
+#pragma unroll
+    for (int kj = 0; kj < ROWS * NJ; ++kj) {
+      const int k = kj / NJ, j = kj % NJ;
+      const long long i = row0 + rowt + k;
+      const int c = CH * j + 4 * q;
+      const float4 v =
+          do_hals && rowt + k < nrows && c < R ? load_rank4(M + i * R + c, R - c, vec) : float4{};
+      m[k][j][0] = v.x; m[k][j][1] = v.y; m[k][j][2] = v.z; m[k][j][3] = v.w;
+    }
+    if (first && do_hals == 1) __syncthreads();
     if (do_hals == 1) {
 #pragma unroll
       for (int j = 0; j < NJ; ++j)
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-          const int c = 16 * j + 4 * q + t;
-          w[j][t] = c < R ? w[j][t] * lamf[c] : 0.0f;
+          const int c = CH * j + 4 * q + t;
+#pragma unroll
+          for (int k = 0; k < ROWS; ++k) w[k][j][t] = c < R ? w[k][j][t] * lamf[c] : 0.0f;
         }
-#pragma unroll 1
-      for (int r4 = 0; r4 < nb4; ++r4) {
-        const int jr = r4 >> 2;
-        const bool own = (r4 & 3) == q;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const int r = 4 * r4 + t;
-          if (r >= R) break;
-          const float4* srow = reinterpret_cast<const float4*>(Ss + r * RMAX) + q;
-          float d0 = 0.0f, d1 = 0.0f, d2 = 0.0f, d3 = 0.0f;
-          float wr = 0.0f, mr = 0.0f;
-#pragma unroll
-          for (int j = 0; j < NJ; ++j) {
-            const float4 sv = srow[4 * j];
-            d0 = fmaf(w[j][0], sv.x, d0);
-            d1 = fmaf(w[j][1], sv.y, d1);
-            d2 = fmaf(w[j][2], sv.z, d2);
-            d3 = fmaf(w[j][3], sv.w, d3);
-            if (j == jr) {
-              wr = w[j][t];
-              mr = m[j][t];
-            }
-          }
-          float dot = (d0 + d1) + (d2 + d3);
-          dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-          dot += __shfl_xor_sync(0xffffffffu, dot, 2);
-          // (m - dot) / s_rr: the product with the reciprocal, corrected once
-          const float num = mr - dot, si = sinv[r];
-          float step = num * si;
-          step = fmaf(fmaf(-srr_s[r], step, num), si, step);
-          const float upd = fmaxf(0.0f, wr + step);
-          if (own && si != 0.0f) {  // S_rr = 0: column left as it is
-#pragma unroll
-            for (int j = 0; j < NJ; ++j)
-              if (j == jr) w[j][t] = upd;
-          }
-        }
-      }
+      if constexpr (ROWS == 1)
+        sweep_quads<RMAX>(w[0], m[0], Ss, srr_s, sinv, R, q);
+      else
+        sweep_residuals<RMAX>(w, m, Ss, Ws + rowt * RP, srr_s, sinv, R, q);
     }
-    float b = 0.0f;
+    float b[ROWS] = {};  // <m, w> of each row
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      const int c = 16 * j + 4 * q;
+    for (int kj = 0; kj < ROWS * NJ; ++kj) {
+      const int k = kj / NJ, j = kj % NJ;
+      const bool in = rowt + k < nrows;
+      const int c = CH * j + 4 * q;
+      const float4 v = make_float4(w[k][j][0], w[k][j][1], w[k][j][2], w[k][j][3]);
 #pragma unroll
-      for (int t = 0; t < 4; ++t) b = fmaf(m[j][t], w[j][t], b);
-      *reinterpret_cast<float4*>(Ws + row * RP + c) = make_float4(w[j][0], w[j][1], w[j][2], w[j][3]);
+      for (int t = 0; t < 4; ++t) b[k] = fmaf(m[k][j][t], w[k][j][t], b[k]);
+      *reinterpret_cast<float4*>(Ws + (rowt + k) * RP + c) = v;
       if (do_hals == 1 && in && c < R) {
-        float* hp = H + i * R + c;
+        float* hp = H + (row0 + rowt + k) * R + c;
         if (vec) {
-          *reinterpret_cast<float4*>(hp) = make_float4(w[j][0], w[j][1], w[j][2], w[j][3]);
+          *reinterpret_cast<float4*>(hp) = v;
         } else {
 #pragma unroll
           for (int t = 0; t < 4; ++t)
-            if (c + t < R) hp[t] = w[j][t];
+            if (c + t < R) hp[t] = w[k][j][t];
         }
       }
     }
     if (do_hals) {
-      b += __shfl_xor_sync(0xffffffffu, b, 1);
-      b += __shfl_xor_sync(0xffffffffu, b, 2);
-      beta += q == 0 ? (double)b : 0.0;
+#pragma unroll
+      for (int k = 0; k < ROWS; ++k) {
+#pragma unroll
+        for (int o = 1; o < LANES; o *= 2) b[k] += __shfl_xor_sync(0xffffffffu, b[k], o);
+        beta += q == 0 ? (double)b[k] : 0.0;
+      }
     }
     __syncthreads();
     // W^T W of these rows, every output over the rows in order: a thread per
     // TB x TB tile
 #pragma unroll 1
     for (int tile = tid; tile < tiles; tile += kHalsThreads) {
-      const int a0 = (tile / nt) * TB, b0 = (tile % nt) * TB;
+      int ta, tb;
+      if (kHalf) {
+        const int f = tile / (nt + 1), p = tile % (nt + 1);
+        ta = p < nt - f ? f : nt - 1 - f;
+        tb = p < nt - f ? f + p : p - 1;
+        if (p >= nt - f && ta == f) continue;  // the middle row of an odd nt, once
+      } else {
+        ta = tile / nt;
+        tb = tile % nt;
+      }
+      const int a0 = ta * TB, b0 = tb * TB;
       float acc[TB][TB];
 #pragma unroll
       for (int x = 0; x < TB; ++x)
@@ -252,7 +413,9 @@ __device__ __forceinline__ void rows_block(float* __restrict__ H, const float* _
         for (int y = 0; y < TB; ++y)
           if (a0 + x < R && b0 + y < R) {
             double* o = gp + (a0 + x) * R + b0 + y;
-            *o = first ? (double)acc[x][y] : *o + (double)acc[x][y];
+            const double g = first ? (double)acc[x][y] : *o + (double)acc[x][y];
+            *o = g;
+            if (kHalf && ta != tb) gp[(b0 + y) * R + a0 + x] = g;
           }
     }
     __syncthreads();
@@ -277,11 +440,8 @@ __global__ void __launch_bounds__(kHalsThreads)
 k_hals_gram(float* __restrict__ H, const float* __restrict__ M, long long In, int R,
             const float* __restrict__ S, const double* __restrict__ lam,
             double* __restrict__ gram_part, const int* __restrict__ flags, int do_hals) {
-  pdl_wait();
-  pdl_trigger();
-  if (flags && flags[0]) return;
   extern __shared__ __align__(16) float sm[];
-  rows_block<RMAX>(H, M, In, R, S, lam, gram_part + (long long)blockIdx.x * (R * R + 1), do_hals,
+  rows_block<RMAX>(H, M, In, R, S, lam, gram_part + (long long)blockIdx.x * (R * R + 1), flags, do_hals,
                    blockIdx.x, gridDim.x, sm);
 }
 
@@ -484,7 +644,7 @@ __global__ void __launch_bounds__(kHalsThreads) k_init_gram(const __grid_constan
   while ((int)blockIdx.x >= a.first[n + 1]) ++n;
   const int b = blockIdx.x - a.first[n], nb = a.first[n + 1] - a.first[n];
   rows_block<RMAX>(a.H[n], nullptr, a.rows[n], a.R, nullptr, nullptr,
-                   a.part[n] + (long long)b * (a.R * a.R + 1), 0, b, nb, sm, false);
+                   a.part[n] + (long long)b * (a.R * a.R + 1), nullptr, 0, b, nb, sm, false);
 }
 
 __global__ void __launch_bounds__(kFinishThreads)
@@ -566,10 +726,6 @@ k_init_finish(const __grid_constant__ InitArgs a, SolveState st, double tol,
   }
 }
 
-__device__ __forceinline__ void cp_async16(float* smem_dst, const float* gmem_src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
-}
 __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gmem_src) : "memory");

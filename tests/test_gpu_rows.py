@@ -13,11 +13,11 @@ from paper_1806_07985_gb300 import nncp, synth
 pytestmark = pytest.mark.gpu
 
 # rows per block 64, blocks at most 304 (19,456 rows in one pass); four columns per lane and
-# 16 per register chunk, so ranks at the edges of both
+# 16 (past rank 64: 64) per register chunk, so ranks at the edges of both
 SHAPES = [((20001, 6, 5), 7, 0), ((19457, 5, 4), 16, 1), ((5, 17000, 4), 33, 0),
           ((65, 9, 8), 65, 0), ((64, 63, 3), 128, 0), ((3, 130, 7), 100, 2),
           ((1100, 4, 3), 81, 1), ((2, 2, 2, 2), 3, 0), ((2, 3), 90, 0),
-          ((2048, 5, 3), 64, 0), ((2047, 5, 3), 64, 1)]
+          ((2048, 5, 3), 64, 0), ((2047, 5, 3), 64, 1), ((19460, 3, 2), 70, 0)]
 
 
 @pytest.mark.parametrize("nls", ["hals", "bpp", "admm"])
