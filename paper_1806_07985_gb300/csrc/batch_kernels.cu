@@ -497,6 +497,20 @@ __device__ __forceinline__ bool mb_test(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// the same without suspending the thread
+__device__ __forceinline__ bool mb_poll(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// A try_wait may suspend a thread for longer than a limit below this many cycles.
+constexpr long long kBriefWaitCycles = 1000000;
 // Bounded wait of a whole warp (all 32 lanes call it, converged): every lane
 // polls (and so acquires the phase), the warp decides together, so a warp
 // never splits over an expired wait (the lanes read one clock).  On expiry
@@ -504,9 +518,10 @@ __device__ __forceinline__ bool mb_test(uint32_t bar, uint32_t parity) {
 // clock64 cycles (kWsWaitCycles unless a test shortens it).
 __device__ __forceinline__ bool mb_wait(uint32_t bar, uint32_t parity, long long limit, int* err,
                                         int site) {
-  if (__all_sync(0xffffffffu, mb_test(bar, parity))) return true;
+  const bool brief = limit < kBriefWaitCycles;
+  if (__all_sync(0xffffffffu, brief ? mb_poll(bar, parity) : mb_test(bar, parity))) return true;
   const long long t0 = clock64();
-  while (!__all_sync(0xffffffffu, mb_test(bar, parity))) {
+  while (!__all_sync(0xffffffffu, brief ? mb_poll(bar, parity) : mb_test(bar, parity))) {
     if (clock64() - t0 > limit) {
       if ((threadIdx.x & 31) == 0) atomicCAS(err, 0, 1 + site);
       return false;
