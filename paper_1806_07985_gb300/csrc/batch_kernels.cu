@@ -905,129 +905,199 @@ __global__ void __launch_bounds__(kReduceBlock) k_b_reduce(const BTensor* __rest
 constexpr int kLeftRedFloats = 4 * kThreads;
 constexpr int kLeftStageFloats = kTileFloats + kLeftMaxRows;  // rows at odd stride
 
-__host__ __device__ constexpr int left_fixed_floats() {
-  return 2 * kLeftStageFloats + kLeftRedFloats;
+// groups that split the i range of a tile's (row, rank group) pairs
+__device__ __forceinline__ int left_groups(int I1, int R) {
+  const int P = b_rows_left(I1) * (b_rq(R) / b_rqb_left(I1, R));
+  return P >= kGroupThreads ? 1 : kGroupThreads / P;
 }
 
 // root -> node {2..N}: T(j, r) = sum_i X[i + I1 j] H_1(i, r).  Item (tensor,
 // kLeftItemTiles tiles of rows j); H_1 (rank padded to b_rank_pad(R) with
-// zeros) sits in shared memory.  Thread = (row j, block of RQB rank groups);
-// when a tile has fewer than 256 such pairs (then RQB = 1) the i range is
-// split over groups added in group order.
-template <int RQB>
+// zeros) sits in shared memory.  The sums' order: where a tile has fewer than 256
+// (row, rank group) pairs the i range is split over G groups added in group order.
+//
+// Shared memory returns 128 bytes per cycle and SM however few of them differ, so
+// the kernel is bound by what its threads read: a thread with one row and one rank
+// group reads five floats for four FMAs.  Here it holds four rows x four ranks in
+// registers, eight floats for sixteen FMAs.  128 threads take two tiles at a time,
+// single-buffered: five CTAs per SM hide each other's copies, where double buffering
+// left two warps each.  Rows are read one, two or four floats at a time, whichever
+// divides I_1, so that dense 16-byte copies leave no bank conflicts (a row of 8 k
+// floats is padded by four).  (1024 tensors of 16 to 128 per mode at ranks 4, 8 and
+// 16, 629 MB: one row per thread behind 4-byte copies to an odd stride 350 us, four
+// rows double-buffered 259 us, this 175 us.)
+constexpr int kLeftThreads = 128;
+constexpr int kLeftTiles = 2;  // tiles in shared memory
+// H_1 with an entry more per rank group
+__host__ __device__ constexpr int left_h_floats(int hs_floats) { return hs_floats + kBatchMaxRank; }
+
+// floats from row to row of a tile in shared memory
+__device__ __forceinline__ int left_stride(int I1, int nj) {
+  return (I1 & 7) == 0 && nj * (I1 + 4) <= kLeftTiles * kLeftStageFloats ? I1 + 4 : I1;
+}
+
+// hp: this rank group's entries of H_1, one per i; xp: the first of four rows, ST apart
+template <int V>
+__device__ __forceinline__ void left_rows(const float* xp, int ST, const float4* hp, int ia, int ib,
+                                          float (&a)[4][4]) {
+  const float* x0 = xp;
+  const float* x1 = x0 + ST;
+  const float* x2 = x1 + ST;
+  const float* x3 = x2 + ST;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) a[t][0] = a[t][1] = a[t][2] = a[t][3] = 0.0f;
+  auto one = [&](int i) {
+    const float4 h = hp[i];
+    fma4(a[0], x0[i], h);
+    fma4(a[1], x1[i], h);
+    fma4(a[2], x2[i], h);
+    fma4(a[3], x3[i], h);
+  };
+  int i = ia;
+  if (V > 1) {
+#pragma unroll 1
+    for (; i < ib && (i & (V - 1)); ++i) one(i);
+    using W = typename std::conditional<V == 4, float4, float2>::type;
+#pragma unroll (V == 2 ? 4 : 2)
+    for (; i + V <= ib; i += V) {
+      W w[4];
+      w[0] = *reinterpret_cast<const W*>(x0 + i);
+      w[1] = *reinterpret_cast<const W*>(x1 + i);
+      w[2] = *reinterpret_cast<const W*>(x2 + i);
+      w[3] = *reinterpret_cast<const W*>(x3 + i);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const float4 h = hp[i + v];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) fma4(a[t], reinterpret_cast<const float*>(&w[t])[v], h);
+      }
+    }
+#pragma unroll 1
+    for (; i < ib; ++i) one(i);
+  } else {
+#pragma unroll 4
+    for (; i < ib; ++i) one(i);
+  }
+}
+
+// ranks 4 q .. 4 q + 3 of row j of T
+__device__ __forceinline__ void left_store(float* T, long long j, int q, int R, const float (&v)[4]) {
+  float* o = T + j * R + 4 * q;
+  if ((R & 3) == 0) {
+    if (4 * q < R) *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+    return;
+  }
+#pragma unroll
+  for (int b = 0; b < 4; ++b)
+    if (4 * q + b < R) o[b] = v[b];
+}
+
+__device__ __forceinline__ void left_copy(float* Xs, const float* __restrict__ src, int rows, int I1, int S) {
+  const int L = rows * I1, L4 = L & ~3;
+  if (S == I1) {
+#pragma unroll 4
+    for (int e = 4 * (int)threadIdx.x; e < L4; e += 4 * kLeftThreads) cp_async16(Xs + e, src + e);
+    const int tail = L4 + (int)threadIdx.x;
+    if (tail < L) cp_async4(Xs + tail, src + tail);
+    return;
+  }
+  const int n4 = I1 >> 2;  // chunks per row
+  const int drow = kLeftThreads / n4, dc = kLeftThreads - drow * n4;
+  int row = threadIdx.x / n4, c = threadIdx.x - row * n4;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < L4 >> 2; e += kLeftThreads) {
+    cp_async16(Xs + row * S + 4 * c, src + 4 * e);
+    row += drow;
+    c += dc;
+    if (c >= n4) {
+      c -= n4;
+      ++row;
+    }
+  }
+}
+
 __device__ __forceinline__ void pm_left_item(const BTensor& t, int item, float* smem) {
-  float* Xbuf[2] = {smem, smem + kLeftStageFloats};
-  float* red = smem + 2 * kLeftStageFloats;  // kLeftRedFloats
-  float* Hs = red + kLeftRedFloats;          // I1 x padded rank
+  float* Xs = smem;
+  float* Hs = smem + kLeftTiles * kLeftStageFloats;  // padded rank x I1
   const int tid = threadIdx.x;
   const int R = t.R, Rq = b_rq(R), Rp = 4 * Rq;
-  const int I1 = (int)t.dims[0], S = I1 | 1;
-  const int nj = t.rows_l;
+  const int I1 = (int)t.dims[0];
+  const int nj = kLeftTiles * t.rows_l, Jq = nj >> 2;
+  const int S = left_stride(I1, nj);
   const int J = (int)(t.I / I1);
-  const int jb0 = item * nj * kLeftItemTiles;
-  const int jb1 = min(J, jb0 + nj * kLeftItemTiles);
-  const int NB = Rq / RQB;  // rank blocks per row
-  const int P = nj * NB;
-  const int G = P >= kGroupThreads ? 1 : kGroupThreads / P;
-  const int npass = (P + kThreads - 1) / kThreads;
-  const int g = G > 1 ? tid / P : 0;
-  const int ia = g * I1 / G, ib = (g + 1) * I1 / G;
-  tile_copy_rows(Xbuf[0], t.X + (long long)jb0 * I1, min(nj, jb1 - jb0) * I1, I1, S);
-  cp_async_commit();
+  const int jb0 = item * t.rows_l * kLeftItemTiles;
+  const int jb1 = min(J, jb0 + t.rows_l * kLeftItemTiles);
+  const int G = left_groups(I1, R);
+  const int P = nj * Rq;
+  // thread = (rows jl + x Jq, rank group qb, group g); a pass covers 128 / Rq rows jl
+  // of G = 1, everything when G > 1 (then P G <= 512)
+  const int lg = __ffs(Rq) - 1, qb = tid & (Rq - 1);
+  const int g = G > 1 ? (tid >> lg) / Jq : 0;
+  const int jl0 = (tid >> lg) - g * Jq;
+  const int ia = g * I1 / G, ib = min(g + 1, G) * I1 / G;
+  const int HT = I1 | 1;  // entries from rank group to rank group (no bank conflicts)
+  const float4* hp = reinterpret_cast<const float4*>(Hs) + qb * HT;
   {
     const float* H1 = t.H[0];
     if (R == Rp) {
-      const int n4 = I1 * Rq;
-      for (int v0 = tid; v0 < n4; v0 += 4 * kThreads) {
-        float4 h[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int v = v0 + u * kThreads;
-          if (v < n4) h[u] = __ldg(reinterpret_cast<const float4*>(H1) + v);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int v = v0 + u * kThreads;
-          if (v < n4) reinterpret_cast<float4*>(Hs)[v] = h[u];
-        }
-      }
+      for (int v = tid; v < I1 * Rq; v += kLeftThreads)
+        cp_async16(Hs + 4 * ((v & (Rq - 1)) * HT + (v >> lg)), H1 + 4 * v);
     } else {
-      for (int e = tid; e < I1 * Rp; e += kThreads) {
-        const int i = e / Rp, r = e - i * Rp;
-        Hs[e] = r < R ? __ldg(H1 + i * R + r) : 0.0f;
+      for (int e = tid; e < I1 * Rp; e += kLeftThreads) {
+        const int i = e >> (lg + 2), r = e & (Rp - 1);
+        Hs[4 * ((r >> 2) * HT + i) + (r & 3)] = r < R ? __ldg(H1 + i * R + r) : 0.0f;
       }
     }
   }
-  const float4* H4 = reinterpret_cast<const float4*>(Hs);
   float* T = t.node[1];
   const int ntile = (jb1 - jb0 + nj - 1) / nj;
   for (int k = 0; k < ntile; ++k) {
     const int jt = jb0 + k * nj, njk = min(nj, jb1 - jt);
-    if (k + 1 < ntile) {
-      const int jn = jt + nj;
-      tile_copy_rows(Xbuf[(k + 1) & 1], t.X + (long long)jn * I1, min(nj, jb1 - jn) * I1, I1, S);
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
+    left_copy(Xs, t.X + (long long)jt * I1, njk, I1, S);
+    cp_async_wait_all();
     __syncthreads();
-    const float* Xs = Xbuf[k & 1];
-    for (int p = 0; p < npass; ++p) {
-      const int pair = G > 1 ? tid - g * P : tid + kThreads * p;
-      const int jl = pair / NB, qb = pair - jl * NB;
-      const bool v = g < G && pair < P && jl < njk;
-      float a[RQB][4];
+    float a[4][4];
+    for (int jl = jl0; jl < Jq && g < G; jl += kLeftThreads >> lg) {
+      const float* xp = Xs + jl * S;
+      if ((I1 & 3) == 0)
+        left_rows<4>(xp, Jq * S, hp, ia, ib, a);
+      else if ((I1 & 1) == 0)
+        left_rows<2>(xp, Jq * S, hp, ia, ib, a);
+      else
+        left_rows<1>(xp, Jq * S, hp, ia, ib, a);
+      if (G > 1) break;
 #pragma unroll
-      for (int u = 0; u < RQB; ++u)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) a[u][b] = 0.0f;
-      if (v) {
-        const float* xp = Xs + jl * S;
-        const float4* hp = H4 + qb * RQB;
-#pragma unroll 4
-        for (int i = ia; i < ib; ++i) {
-          const float x = xp[i];
-#pragma unroll
-          for (int u = 0; u < RQB; ++u) fma4(a[u], x, hp[i * Rq + u]);
-        }
-      }
-      if (G > 1) {  // RQB == 1 here
-        if (g < G) reinterpret_cast<float4*>(red)[tid] = make_float4(a[0][0], a[0][1], a[0][2], a[0][3]);
-        __syncthreads();
-        if (tid < P) {
-          const int jl0 = tid / NB, q0 = tid - jl0 * NB;
-          if (jl0 < njk) {
-            float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            for (int gg = 0; gg < G; ++gg) {
-              const float4 w = reinterpret_cast<const float4*>(red)[gg * P + tid];
-              s4[0] += w.x;
-              s4[1] += w.y;
-              s4[2] += w.z;
-              s4[3] += w.w;
-            }
-#pragma unroll
-            for (int b = 0; b < 4; ++b)
-              if (4 * q0 + b < R) T[(long long)(jt + jl0) * R + 4 * q0 + b] = s4[b];
-          }
-        }
-        __syncthreads();
-      } else if (v) {
-#pragma unroll
-        for (int u = 0; u < RQB; ++u)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int r = 4 * (qb * RQB + u) + b;
-            if (r < R) T[(long long)(jt + jl) * R + r] = a[u][b];
-          }
+      for (int x = 0; x < 4; ++x) {
+        if (jl + x * Jq < njk) left_store(T, jt + jl + x * Jq, qb, R, a[x]);
       }
     }
     __syncthreads();
+    if (G > 1) {  // the groups' sums through the tile's own space
+      float4* red = reinterpret_cast<float4*>(Xs);
+      if (g < G) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          red[g * P + (jl0 + x * Jq) * Rq + qb] = make_float4(a[x][0], a[x][1], a[x][2], a[x][3]);
+        }
+      }
+      __syncthreads();
+      for (int e = tid; e < njk * Rq; e += kLeftThreads) {
+        float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int gg = 0; gg < G; ++gg) {
+          const float4 w = red[gg * P + e];
+          s4[0] += w.x;
+          s4[1] += w.y;
+          s4[2] += w.z;
+          s4[3] += w.w;
+        }
+        left_store(T, jt + (e >> lg), e & (Rq - 1), R, s4);
+      }
+      __syncthreads();
+    }
   }
 }
 
-template <int RMAX>
-__global__ void __launch_bounds__(kThreads, RMAX <= 16 ? 4 : 2)
+__global__ void __launch_bounds__(kLeftThreads)
 k_b_pm_left(const BTensor* __restrict__ ts, const int4* __restrict__ items, int n_items,
             int* queue) {
   extern __shared__ __align__(16) float smem[];
@@ -1037,13 +1107,7 @@ k_b_pm_left(const BTensor* __restrict__ ts, const int4* __restrict__ items, int 
     const int4 it = items[w];
     const BTensor& t = ts[it.x];
     if (tensor_done(t)) continue;
-    switch (b_rqb_left((int)t.dims[0], t.R)) {
-      case 1: pm_left_item<1>(t, it.y, smem); break;
-      case 2: pm_left_item<2>(t, it.y, smem); break;
-      case 4: pm_left_item<4>(t, it.y, smem); break;
-      case 8: if constexpr (RMAX >= 32) pm_left_item<8>(t, it.y, smem); break;
-      default: if constexpr (RMAX >= 64) pm_left_item<16>(t, it.y, smem); break;
-    }
+    pm_left_item(t, it.y, smem);
   }
 }
 
@@ -1060,7 +1124,7 @@ k_b_pm_left(const BTensor* __restrict__ ts, const int4* __restrict__ items, int 
 //                      H slots; copy the tile to the odd row stride S = I_1 | 1
 //                      (conflict-free column reads) into a ring of SO stages,
 //                      with the header; free the dense stage;
-//   warps 5-12, consumers (the 256 threads of pm_left_item): the (row, rank
+//   warps 5-12, consumers (256 threads): the (row, rank
 //                      block) passes over each odd-stride tile, group sums
 //                      through a small buffer, rows of T written out; an odd
 //                      stage is freed after its tile, an H slot after its item.
@@ -1696,7 +1760,7 @@ cudaError_t batch_attributes_init() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_init_mode, cudaFuncAttributeMaxDynamicSharedMemorySize, fac);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_init, cudaFuncAttributeMaxDynamicSharedMemorySize, fac);
   const int right = (2 * kTileFloats + kWsFloats) * (int)sizeof(float);
-  const int left = (left_fixed_floats() + kBatchMaxI * kBatchMaxRank) * (int)sizeof(float);
+  const int left = (kLeftTiles * kLeftStageFloats + left_h_floats(kBatchMaxI * kBatchMaxRank)) * (int)sizeof(float);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_right<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, right);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_right<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, right);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_right<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, right);
@@ -1709,9 +1773,7 @@ cudaError_t batch_attributes_init() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_left_ws<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_left_ws<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_left_ws<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_left<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, left);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_left<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, left);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_left<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, left);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_left, cudaFuncAttributeMaxDynamicSharedMemorySize, left);
   return e;
 }
 
@@ -1721,12 +1783,12 @@ namespace {
 // persistent CTAs (every CTA that fits at once at this shared-memory size)
 // taking items from the counter `queue`.
 template <typename K>
-int phase_grid(K kernel, size_t smem, int n_items, const int* queue) {
+int phase_grid(K kernel, int threads, size_t smem, int n_items, const int* queue) {
   if (!queue) return n_items;
   int dev = 0, sms = 1, per_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess ||
       per_sm < 1)
     per_sm = 1;
   return std::max(1, std::min(n_items, sms * per_sm));
@@ -1813,11 +1875,11 @@ cudaError_t launch_pm_right(const BPlan& p, const BTensor* ts, const int4* items
     if (e != cudaSuccess) return e;
   } else if (n > 0) {
     if (p.rmax <= 16)
-      k_b_pm_right<16><<<phase_grid(k_b_pm_right<16>, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
+      k_b_pm_right<16><<<phase_grid(k_b_pm_right<16>, kThreads, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
     else if (p.rmax <= 32)
-      k_b_pm_right<32><<<phase_grid(k_b_pm_right<32>, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
+      k_b_pm_right<32><<<phase_grid(k_b_pm_right<32>, kThreads, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
     else
-      k_b_pm_right<64><<<phase_grid(k_b_pm_right<64>, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
+      k_b_pm_right<64><<<phase_grid(k_b_pm_right<64>, kThreads, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
   }
   if (p.pmr_red.count > 0)
     k_b_reduce<<<p.pmr_red.count, kReduceBlock, 0, st>>>(ts, items + p.pmr_red.off);
@@ -1834,13 +1896,8 @@ cudaError_t launch_pm_left(const BPlan& p, const BTensor* ts, const int4* items,
     return p.rmax <= 16   ? launch_pm_left_ws<16>(ts, it, n, queue, p.hs_floats, err, wait_cycles, st)
            : p.rmax <= 32 ? launch_pm_left_ws<32>(ts, it, n, queue, p.hs_floats, err, wait_cycles, st)
                           : launch_pm_left_ws<64>(ts, it, n, queue, p.hs_floats, err, wait_cycles, st);
-  const size_t sm = (size_t)(left_fixed_floats() + p.hs_floats) * sizeof(float);
-  if (p.rmax <= 16)
-    k_b_pm_left<16><<<phase_grid(k_b_pm_left<16>, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
-  else if (p.rmax <= 32)
-    k_b_pm_left<32><<<phase_grid(k_b_pm_left<32>, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
-  else
-    k_b_pm_left<64><<<phase_grid(k_b_pm_left<64>, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
+  const size_t sm = (size_t)(kLeftTiles * kLeftStageFloats + left_h_floats(p.hs_floats)) * sizeof(float);
+  k_b_pm_left<<<phase_grid(k_b_pm_left, kLeftThreads, sm, n, queue), kLeftThreads, sm, st>>>(ts, it, n, queue);
   return cudaGetLastError();
 }
 
