@@ -190,12 +190,10 @@ __global__ void __launch_bounds__(256) k_b_init(BTensor* __restrict__ ts, const 
 // ------------------------------------------------ partial MTTKRPs (root) --
 //
 // Both root contractions stream X_(1)^T (rows j of I_1 contiguous floats) in
-// tiles of whole rows.  A tile is fetched into registers (eight float4 per
-// thread, every load issued before any is used) one tile ahead of the
-// compute, then stored to shared memory; the thread mapping is sized from
-// the tensor's own rank, and when one tile holds too few (row, rank-group)
-// pairs for 256 threads the contraction range is split over thread groups
-// whose partial sums are added in group order.
+// tiles of whole rows; the thread mapping is sized from the tensor's own rank, and
+// when one tile holds too few (row, rank-group) pairs for 256 threads the
+// contraction range is split over groups whose partial sums are added in group
+// order.
 
 constexpr int kThreads = 256;
 // Split groups are sized for kGroupThreads whatever the block size, so the
@@ -203,8 +201,7 @@ constexpr int kThreads = 256;
 constexpr int kGroupThreads = 256;
 
 // Tiles are copied global -> shared with cp.async (no registers held while
-// in flight) into a two-stage ring, so tile k+1 streams in while tile k is
-// formed and contracted; X is read once per pass.
+// in flight); the CTAs of an SM hide each other's copies.  X is read once per pass.
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -214,42 +211,7 @@ __device__ __forceinline__ void cp_async16(float* dst, const float* src) {
 __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int NPENDING>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(NPENDING) : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// floats [0, L) of src (16-byte aligned) to Xs[0, L)
-__device__ __forceinline__ void tile_copy_dense(float* Xs, const float* __restrict__ src, int L) {
-  const int L4 = L & ~3;
-  for (int e = 4 * (int)threadIdx.x; e < L4; e += 4 * kThreads) cp_async16(Xs + e, src + e);
-  const int tail = L4 + (int)threadIdx.x;
-  if (tail < L) cp_async4(Xs + tail, src + tail);
-}
-
-// rows of I1 floats to an odd stride S (threads reading one column of
-// consecutive rows hit distinct banks): Xs[row * S + col] = src[row * I1 + col]
-__device__ __forceinline__ void tile_copy_rows(float* Xs, const float* __restrict__ src, int L,
-                                               int I1, int S) {
-  if (S == I1) {
-    tile_copy_dense(Xs, src, L);
-    return;
-  }
-  int e = threadIdx.x;
-  int row = e / I1, col = e - row * I1;
-  const int drow = kThreads / I1, dcol = kThreads - drow * I1;
-  for (; e < L; e += kThreads) {
-    cp_async4(Xs + row * S + col, src + e);
-    row += drow;
-    col += dcol;
-    if (col >= I1) {
-      col -= I1;
-      ++row;
-    }
-  }
-}
 
 // ranks r0 .. r0 + 3 of a factor row (zero beyond R); vector load when R % 4 == 0
 __device__ __forceinline__ float4 ld_rank4(const float* __restrict__ row, int r0, int R) {
@@ -265,125 +227,23 @@ __device__ __forceinline__ float4 ld_rank4(const float* __restrict__ row, int r0
   return h;
 }
 
+// ranks 4 q .. 4 q + 3 of an output row (16-byte aligned when R % 4 == 0)
+__device__ __forceinline__ void store_rank4(float* row, int q, int R, const float (&v)[4]) {
+  float* o = row + 4 * q;
+  if ((R & 3) == 0) {
+    if (4 * q < R) *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+    return;
+  }
+#pragma unroll
+  for (int b = 0; b < 4; ++b)
+    if (4 * q + b < R) o[b] = v[b];
+}
+
 __device__ __forceinline__ void fma4(float (&a)[4], float x, const float4& w) {
   a[0] = fmaf(x, w.x, a[0]);
   a[1] = fmaf(x, w.y, a[1]);
   a[2] = fmaf(x, w.z, a[2]);
   a[3] = fmaf(x, w.w, a[3]);
-}
-
-// root -> node {1}: part[c](i, r) = sum_{j in chunk c} X[i + I1 j] K(j, r),
-// K = H_N (.) ... (.) H_2 (rows formed per tile, never stored whole).
-// Item (tensor, chunk).  Thread = row i with all RQB = b_rq(R) rank groups;
-// 256 / I1 column groups split each tile's rows (j = g, g + G, ...) and are
-// added in group order at the end of the chunk.
-template <int RQB>
-__device__ __forceinline__ void pm_right_item(const BTensor& t, int chunk, float* smem) {
-  constexpr int WU = kWsFloats / 4 / kThreads;
-  float* Xbuf[2] = {smem, smem + kTileFloats};
-  float* Ws = smem + 2 * kTileFloats;  // kWsFloats: rows x padded rank
-  const int tid = threadIdx.x;
-  const int R = t.R, N = t.N;
-  const int I1 = (int)t.dims[0];
-  const int nj = t.rows_r;
-  const int J = (int)(t.I / I1);
-  const int j0 = chunk * (int)t.jchunk;
-  const int j1 = min(J, j0 + (int)t.jchunk);
-  const int G = kGroupThreads / I1;
-  const int g = tid / I1, i = tid - g * I1;
-  const bool act = g < G;
-  float acc[RQB][4];
-#pragma unroll
-  for (int u = 0; u < RQB; ++u)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[u][b] = 0.0f;
-  const int ntile = (j1 - j0 + nj - 1) / nj;
-  const float4* W4 = reinterpret_cast<const float4*>(Ws);
-  tile_copy_dense(Xbuf[0], t.X + (long long)j0 * I1, min(nj, j1 - j0) * I1);
-  cp_async_commit();
-  for (int k = 0; k < ntile; ++k) {
-    const int jt = j0 + k * nj, njk = min(nj, j1 - jt);
-    if (k + 1 < ntile) {
-      const int jn = jt + nj;
-      tile_copy_dense(Xbuf[(k + 1) & 1], t.X + (long long)jn * I1, min(nj, j1 - jn) * I1);
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    // Khatri-Rao rows of the tile: float4 entries (row, rank group), nj * RQB <= kWsFloats / 4
-    {
-      float4 w[WU];
-      int rem[WU];
-#pragma unroll
-      for (int u = 0; u < WU; ++u) {
-        rem[u] = jt + (tid + kThreads * u) / RQB;
-        w[u] = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
-      }
-      for (int m = 1; m < N; ++m) {
-        const int dm = (int)t.dims[m];
-        const float* Hm = t.H[m];
-#pragma unroll
-        for (int u = 0; u < WU; ++u) {
-          const int e = tid + kThreads * u;
-          if (e / RQB < njk) {
-            const int jm = rem[u] % dm;
-            rem[u] /= dm;
-            const float4 h = ld_rank4(Hm + jm * R, 4 * (e % RQB), R);
-            w[u].x *= h.x;
-            w[u].y *= h.y;
-            w[u].z *= h.z;
-            w[u].w *= h.w;
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < WU; ++u) {
-        const int e = tid + kThreads * u;
-        if (e / RQB < njk) reinterpret_cast<float4*>(Ws)[e] = w[u];
-      }
-    }
-    __syncthreads();
-    if (act) {
-      const float* xp = Xbuf[k & 1] + i;
-#pragma unroll 2
-      for (int jj = g; jj < njk; jj += G) {
-        const float x = xp[jj * I1];
-#pragma unroll
-        for (int u = 0; u < RQB; ++u) fma4(acc[u], x, W4[jj * RQB + u]);
-      }
-    }
-    __syncthreads();
-  }
-  float* out = t.part + (long long)chunk * I1 * R;
-  if (G > 1) {
-    float4* red = reinterpret_cast<float4*>(Xbuf[0]);  // G * I1 <= 256 float4
-#pragma unroll
-    for (int u = 0; u < RQB; ++u) {
-      if (act) red[tid] = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-      __syncthreads();
-      if (tid < I1) {
-        float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        for (int gg = 0; gg < G; ++gg) {
-          const float4 v = red[gg * I1 + tid];
-          s4[0] += v.x;
-          s4[1] += v.y;
-          s4[2] += v.z;
-          s4[3] += v.w;
-        }
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-          if (4 * u + b < R) out[tid * R + 4 * u + b] = s4[b];
-      }
-      __syncthreads();
-    }
-  } else if (act) {
-#pragma unroll
-    for (int u = 0; u < RQB; ++u)
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-        if (4 * u + b < R) out[i * R + 4 * u + b] = acc[u][b];
-  }
 }
 
 // Work item w of a phase for this CTA: with queue == NULL the CTA's own
@@ -398,10 +258,215 @@ __device__ __forceinline__ int next_item(int* queue, int n_items, int* slot, boo
   return *slot < n_items ? *slot : -1;
 }
 
+// root -> node {1}: part[c](i, r) = sum_{j in chunk c} X[i + I1 j] K(j, r),
+// K = H_N (.) ... (.) H_2 (rows formed per tile, never stored whole).  Item (tensor,
+// chunk).  The sums' order: G = 256 / I1 column groups split each tile's rows
+// (j = g, g + G, ...) and are added in group order at the end of the chunk.
+//
+// What bounds it is shared memory, which returns 128 bytes per cycle and SM however
+// few of them differ: a thread with one row reads 1 + R floats for R FMAs.  Here it
+// holds four rows of one column group (rows ii + x ceil(I1 / 4)) x one, two or four
+// rank groups; tiles are single-buffered, CTAs small and several per SM, and the
+// Khatri-Rao rows are formed while a tile's copies are in flight.  (1024 tensors of 16
+// to 128 per mode at ranks 4, 8 and 16, 629 MB: one row per thread 275 us, this 202 us.)
 template <int RMAX>
-__global__ void __launch_bounds__(kThreads, RMAX <= 16 ? 4 : (RMAX <= 32 ? 3 : 2))
-k_b_pm_right(const BTensor* __restrict__ ts, const int4* __restrict__ items, int n_items,
-             int* queue) {
+struct RightCfg {
+  static constexpr int T = RMAX <= 32 ? 128 : 256;  // threads
+  static constexpr int NA = RMAX <= 16 ? 8 : 16;    // accumulators of four ranks per thread
+  static constexpr int CTAS = RMAX <= 16 ? 5 : (RMAX <= 32 ? 4 : 2);
+};
+
+// A thread's Khatri-Rao rows: their digit in mode 2 and the rest, kept by addition
+// from tile to tile (a division per row and mode cost more than the products).
+struct KrDigits {
+  int a, rest;     // of this thread's first row of the tile
+  int ta, trest;   // a tile's rows
+  int sa, srest;   // the rows from one of the thread's entries to its next
+};
+__device__ __forceinline__ void kr_step(int& a, int& rest, int da, int drest, int d) {
+  a += da;
+  rest += drest;
+  if (a >= d) {
+    a -= d;
+    ++rest;
+  }
+}
+
+// Khatri-Rao rows of a tile of njk: entry (row, rank group)
+template <int T>
+__device__ __forceinline__ void right_krp(const BTensor& t, int njk, int lg, KrDigits& k, float* Ws) {
+  const int N = t.N, R = t.R, r0 = 4 * ((int)threadIdx.x & ((1 << lg) - 1)), d = (int)t.dims[1];
+  const float* H1 = t.H[1];
+  const float* H2 = N > 2 ? t.H[2] : nullptr;
+  int a = k.a, rest = k.rest;
+#pragma unroll 2
+  for (int e = threadIdx.x; e < njk << lg; e += T) {
+    float4 w = ld_rank4(H1 + a * R, r0, R);
+    if (N == 3) {
+      const float4 h = ld_rank4(H2 + rest * R, r0, R);
+      w.x *= h.x;
+      w.y *= h.y;
+      w.z *= h.z;
+      w.w *= h.w;
+    } else {
+      unsigned rem = (unsigned)rest;
+      for (int m = 2; m < N; ++m) {
+        const unsigned dm = (unsigned)t.dims[m];
+        const float4 h = ld_rank4(t.H[m] + (int)(rem % dm) * R, r0, R);
+        rem /= dm;
+        w.x *= h.x;
+        w.y *= h.y;
+        w.z *= h.z;
+        w.w *= h.w;
+      }
+    }
+    reinterpret_cast<float4*>(Ws)[e] = w;
+    kr_step(a, rest, k.sa, k.srest, d);
+  }
+  kr_step(k.a, k.rest, k.ta, k.trest, d);
+}
+
+// One item, in one of two forms with the same copies, Khatri-Rao rows and group sums
+// (one body: the CTAs of an SM run different forms, and a body each overflowed the
+// instruction cache): four rows x rqt rank groups, rqt the fewest with which T threads
+// suffice, or, where ceil(I_1 / 4) rounds up too far for any, 256 / T (column group,
+// row) pairs with all rank groups.
+template <int RQT, int NA>
+__device__ __forceinline__ void right_quads(const float* xp, const float4* wp, int Iq, int first, int njk,
+                                            int G, int xs, int ws, float (&acc)[NA][4]) {
+#pragma unroll 2
+  for (int jj = first; jj < njk; jj += G, xp += xs, wp += ws) {
+    float xv[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) xv[x] = xp[x * Iq];  // past the last row: not used
+#pragma unroll
+    for (int u = 0; u < RQT; ++u) {
+      const float4 w = wp[u];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) fma4(acc[4 * u + x], xv[x], w);
+    }
+  }
+}
+
+template <int RMAX>
+__device__ __forceinline__ void pm_right_item(const BTensor& t, int chunk, float* smem) {
+  constexpr int T = RightCfg<RMAX>::T, NA = RightCfg<RMAX>::NA;
+  constexpr int NP = kGroupThreads / T;  // pairs per thread, NA / NP rank groups each
+  float* Xs = smem;
+  float* Ws = smem + kTileFloats;
+  const int tid = threadIdx.x;
+  const int R = t.R, Rq = b_rq(R), lg = __ffs(Rq) - 1;
+  const int I1 = (int)t.dims[0];
+  const int nj = t.rows_r;
+  const int J = (int)(t.I / I1);
+  const int j0 = chunk * (int)t.jchunk;
+  const int j1 = min(J, j0 + (int)t.jchunk);
+  const int G = kGroupThreads / I1;
+  const int Iq = (I1 + 3) >> 2;
+  const int units = Iq * G;  // threads for four rows and every rank group, about 64
+  int rqt = 1;
+  while (rqt < Rq && units * (Rq / rqt) > T) rqt *= 2;
+  const bool pairs = units * (Rq / rqt) > T || 4 * rqt > NA;
+  if (pairs) rqt = Rq;
+  // thread = (row ii, block ub of rank groups, column group g), ii fastest; pairs:
+  // (g, ii) and, with two, (g1, i1)
+  const int nub = Rq / rqt, w1 = pairs ? I1 : Iq;
+  const int v = tid / w1, ii = tid - v * w1;
+  const int ub = v & (nub - 1), g = v / nub;
+  const int g1 = (tid + T) / I1, i1 = tid + T - g1 * I1;
+  float acc[NA][4];
+#pragma unroll
+  for (int x = 0; x < NA; ++x)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[x][b] = 0.0f;
+  const float4* W4 = reinterpret_cast<const float4*>(Ws) + ub * rqt;
+  KrDigits kd;
+  {
+    const int d = (int)t.dims[1], row = j0 + (tid >> lg), step = T >> lg;
+    kd.rest = row / d;
+    kd.a = row - kd.rest * d;
+    kd.trest = nj / d;
+    kd.ta = nj - kd.trest * d;
+    kd.srest = step / d;
+    kd.sa = step - kd.srest * d;
+  }
+  for (int jt = j0; jt < j1; jt += nj) {
+    const int njk = min(nj, j1 - jt);
+    {
+      const float* src = t.X + (long long)jt * I1;
+      const int L = njk * I1, L4 = L & ~3;
+#pragma unroll 4
+      for (int e = 4 * tid; e < L4; e += 4 * T) cp_async16(Xs + e, src + e);
+      if (L4 + tid < L) cp_async4(Xs + L4 + tid, src + L4 + tid);
+    }
+    right_krp<T>(t, njk, lg, kd, Ws);
+    cp_async_wait_all();
+    __syncthreads();
+    const float* xp = Xs + ii + g * I1;
+    const float4* wp = W4 + (g << lg);
+    const int first = g < G ? g : njk;
+    if (pairs) {
+#pragma unroll
+      for (int x = 0; x < NP; ++x) {
+        const int gx = x ? g1 : g, ix = x ? i1 : ii;
+#pragma unroll 1
+        for (int jj = gx < G ? gx : njk; jj < njk; jj += G) {
+          const float xv = Xs[jj * I1 + ix];
+#pragma unroll
+          for (int u = 0; u < NA / NP; ++u)
+            if (u < Rq) fma4(acc[NA / NP * x + u], xv, W4[(jj << lg) + u]);
+        }
+      }
+    } else if (rqt == 1) {
+      right_quads<1>(xp, wp, Iq, first, njk, G, G * I1, G << lg, acc);
+    } else if (NA == 8 || rqt == 2) {
+      right_quads<2>(xp, wp, Iq, first, njk, G, G * I1, G << lg, acc);
+    } else {
+      right_quads<NA / 4>(xp, wp, Iq, first, njk, G, G * I1, G << lg, acc);
+    }
+    __syncthreads();
+  }
+  // the column groups' sums, added in group order, four rank groups at a time:
+  // (rank group, column group, row)
+  float4* red = reinterpret_cast<float4*>(Xs);
+  float* out = t.part + (long long)chunk * I1 * R;
+#pragma unroll 1
+  for (int q0 = 0; q0 < Rq; q0 += 4) {
+    const int nq = min(4, Rq - q0);
+#pragma unroll
+    for (int x = 0; x < NA; ++x) {
+      const int px = x / (NA / NP);  // pair of the accumulator
+      const int u = (pairs ? x % (NA / NP) : ub * rqt + (x >> 2)) - q0;
+      const int gx = pairs && px ? g1 : g;
+      const int ix = pairs ? (px ? i1 : ii) : ii + (x & 3) * Iq;
+      if ((pairs || (x >> 2) < rqt) && u >= 0 && u < nq && gx < G && ix < I1)
+        red[u * kGroupThreads + gx * I1 + ix] = make_float4(acc[x][0], acc[x][1], acc[x][2], acc[x][3]);
+    }
+    __syncthreads();
+    for (int e = tid; e < I1 * nq; e += T) {
+      const int q = e & (nq - 1), i = e / nq;
+      const float4* rp = red + q * kGroupThreads + i;
+      float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      if (G == 1) {
+        s4[0] = rp->x; s4[1] = rp->y; s4[2] = rp->z; s4[3] = rp->w;
+      }
+#pragma unroll 1
+      for (int gg = 0; gg < (G > 1 ? G : 0); ++gg) {
+        const float4 w = rp[gg * I1];
+        s4[0] += w.x;
+        s4[1] += w.y;
+        s4[2] += w.z;
+        s4[3] += w.w;
+      }
+      store_rank4(out + i * R, q0 + q, R, s4);
+    }
+    __syncthreads();
+  }
+}
+
+template <int RMAX>
+__global__ void __launch_bounds__(RightCfg<RMAX>::T, RightCfg<RMAX>::CTAS)
+k_b_pm_right(const BTensor* __restrict__ ts, const int4* __restrict__ items, int n_items, int* queue) {
   extern __shared__ __align__(16) float smem[];
   __shared__ int slot;
   for (int w = next_item(queue, n_items, &slot, true); w >= 0;
@@ -409,13 +474,7 @@ k_b_pm_right(const BTensor* __restrict__ ts, const int4* __restrict__ items, int
     const int4 it = items[w];
     const BTensor& t = ts[it.x];
     if (tensor_done(t)) continue;
-    switch (b_rq(t.R)) {
-      case 1: pm_right_item<1>(t, it.y, smem); break;
-      case 2: pm_right_item<2>(t, it.y, smem); break;
-      case 4: pm_right_item<4>(t, it.y, smem); break;
-      case 8: if constexpr (RMAX >= 32) pm_right_item<8>(t, it.y, smem); break;
-      default: if constexpr (RMAX >= 64) pm_right_item<16>(t, it.y, smem); break;
-    }
+    pm_right_item<RMAX>(t, it.y, smem);
   }
 }
 
@@ -433,7 +492,7 @@ k_b_pm_right(const BTensor* __restrict__ ts, const int4* __restrict__ items, int
 //                      stage's full barrier as the copies land;
 //   warps 2-4, builders: take stages in turn and form a stage's Khatri-Rao
 //                      rows;
-//   warps 5-12, consumers (the 256 threads of pm_right_item): contract each
+//   warps 5-12, consumers (256 threads, a row each): contract each
 //                      tile and free its stage; at the end of an item they
 //                      add the column groups in group order through the last
 //                      stage's tile area, then free it.
@@ -902,7 +961,6 @@ __global__ void __launch_bounds__(kReduceBlock) k_b_reduce(const BTensor* __rest
   }
 }
 
-constexpr int kLeftRedFloats = 4 * kThreads;
 constexpr int kLeftStageFloats = kTileFloats + kLeftMaxRows;  // rows at odd stride
 
 // groups that split the i range of a tile's (row, rank group) pairs
@@ -978,18 +1036,6 @@ __device__ __forceinline__ void left_rows(const float* xp, int ST, const float4*
 #pragma unroll 4
     for (; i < ib; ++i) one(i);
   }
-}
-
-// ranks 4 q .. 4 q + 3 of row j of T
-__device__ __forceinline__ void left_store(float* T, long long j, int q, int R, const float (&v)[4]) {
-  float* o = T + j * R + 4 * q;
-  if ((R & 3) == 0) {
-    if (4 * q < R) *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
-    return;
-  }
-#pragma unroll
-  for (int b = 0; b < 4; ++b)
-    if (4 * q + b < R) o[b] = v[b];
 }
 
 __device__ __forceinline__ void left_copy(float* Xs, const float* __restrict__ src, int rows, int I1, int S) {
@@ -1068,7 +1114,7 @@ __device__ __forceinline__ void pm_left_item(const BTensor& t, int item, float* 
       if (G > 1) break;
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
-        if (jl + x * Jq < njk) left_store(T, jt + jl + x * Jq, qb, R, a[x]);
+        if (jl + x * Jq < njk) store_rank4(T + (long long)(jt + jl + x * Jq) * R, qb, R, a[x]);
       }
     }
     __syncthreads();
@@ -1090,7 +1136,7 @@ __device__ __forceinline__ void pm_left_item(const BTensor& t, int item, float* 
           s4[2] += w.z;
           s4[3] += w.w;
         }
-        left_store(T, jt + (e >> lg), e & (Rq - 1), R, s4);
+        store_rank4(T + (long long)(jt + (e >> lg)) * R, e & (Rq - 1), R, s4);
       }
       __syncthreads();
     }
@@ -1759,11 +1805,7 @@ cudaError_t batch_attributes_init() {
   const int fac = kBatchMaxI * kBatchMaxRank * (int)sizeof(float);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_init_mode, cudaFuncAttributeMaxDynamicSharedMemorySize, fac);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_init, cudaFuncAttributeMaxDynamicSharedMemorySize, fac);
-  const int right = (2 * kTileFloats + kWsFloats) * (int)sizeof(float);
   const int left = (kLeftTiles * kLeftStageFloats + left_h_floats(kBatchMaxI * kBatchMaxRank)) * (int)sizeof(float);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_right<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, right);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_right<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, right);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_b_pm_right<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, right);
   int dev = 0, optin = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -1864,7 +1906,7 @@ cudaError_t launch_pm_left_ws(const BTensor* ts, const int4* it, int n, int* que
 
 cudaError_t launch_pm_right(const BPlan& p, const BTensor* ts, const int4* items, int mode,
                             int* queue, int* err, cudaStream_t st, long long wait_cycles) {
-  const size_t sm = (size_t)(2 * kTileFloats + kWsFloats) * sizeof(float);
+  const size_t sm = (size_t)(kTileFloats + kWsFloats) * sizeof(float);
   const int n = p.pmr.count;
   const int4* it = items + p.pmr.off;
   if (mode == 0 || !queue) queue = nullptr;
@@ -1874,12 +1916,15 @@ cudaError_t launch_pm_right(const BPlan& p, const BTensor* ts, const int4* items
                                    : launch_pm_right_ws<64>(ts, it, n, queue, err, wait_cycles, st);
     if (e != cudaSuccess) return e;
   } else if (n > 0) {
+    auto run = [&](auto k, int threads) {
+      k<<<phase_grid(k, threads, sm, n, queue), threads, sm, st>>>(ts, it, n, queue);
+    };
     if (p.rmax <= 16)
-      k_b_pm_right<16><<<phase_grid(k_b_pm_right<16>, kThreads, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
+      run(k_b_pm_right<16>, RightCfg<16>::T);
     else if (p.rmax <= 32)
-      k_b_pm_right<32><<<phase_grid(k_b_pm_right<32>, kThreads, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
+      run(k_b_pm_right<32>, RightCfg<32>::T);
     else
-      k_b_pm_right<64><<<phase_grid(k_b_pm_right<64>, kThreads, sm, n, queue), kThreads, sm, st>>>(ts, it, n, queue);
+      run(k_b_pm_right<64>, RightCfg<64>::T);
   }
   if (p.pmr_red.count > 0)
     k_b_reduce<<<p.pmr_red.count, kReduceBlock, 0, st>>>(ts, items + p.pmr_red.off);
