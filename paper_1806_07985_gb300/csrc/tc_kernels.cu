@@ -407,7 +407,7 @@ __device__ __forceinline__ Unit get_unit(const TcParams& p, long long u) {
 // instantiation so that the plain kernel carries none of its code.  SPLIT:
 // the split-BF16x3 precision (A in tensor memory, segmented accumulation),
 // separate so that neither form carries the other's registers.
-template <bool LEAF, bool SPLIT>
+template <bool LEAF, bool SPLIT, bool WRAP>
 __global__ void __launch_bounds__(kThreads, 1)
 k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
   // Launched in a graph with programmatic serialization, the kernel may start
@@ -652,8 +652,12 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
     int* so = offs + bw * kKC * (kMaxModes + 1);  // this slot's offsets [kKC][kMaxModes + 1]
     uint32_t bt_base = b0 + bw * kBBytes;
     // the first Khatri-Rao mode spans whole 64-element stages: the other modes'
-    // rows are the same for every element of a stage
-    const bool lead_aligned = (kdim[0] % kKC) == 0;
+    // rows are the same for every element of a stage.  WRAP: it does not, but is long;
+    // it wraps at most once within the 32 elements that a warp forms, so the other
+    // modes' rows are those of one index before the wrap and of the next after it.
+    // (An instantiation of its own: in one kernel the longer code took the aligned
+    // split pass of 512^3 at R = 32 from 95 to 111 us.)
+    const bool lead = WRAP || (kdim[0] % kKC) == 0;
     // write rank row rr, elements [32 half, 32 half + 32) of the B tile
     auto store_b_rows = [&](const float* v, int rr) {
 #pragma unroll
@@ -689,7 +693,7 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
         w.nk = (int)((p.K + kKC - 1) / kKC);
       }
       if (!p.b_resident && u >= n_units) break;
-      // lead-aligned position of this half's first element, kept incrementally:
+      // position of this half's first element, kept incrementally:
       // k = kbeg + 64 s + 32 half = lq * kd0 + lk (one 64-bit division per unit)
       const long long kb = w.kbeg + half * 32;
       long long lq = kb / kd0;
@@ -697,6 +701,26 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
       int ls = 0;                 // stage the position refers to
       long long cst_q = -1;       // slow index the cached constant belongs to
       float cst = 1.0f;
+      // WRAP: the products of the other modes' rows at slow index cst_q
+      // and at the one after it, for this lane's rank rows lane and lane + 32
+      long long nxt_q = -1;
+      float now[2] = {1.0f, 1.0f}, nxt[2] = {1.0f, 1.0f};
+      auto slow_rows = [&](long long q, float* c) {
+#pragma unroll
+        for (int it = 0; it < 2; ++it) {
+          const int rr = lane + 32 * it;
+          if (32 * it >= Rp) break;
+          long long rem = q;
+          float v = 1.0f;
+          for (int m = 1; m < nm; ++m) {
+            const uint32_t dm = kdim[m];
+            const long long qm = rem / dm;
+            v *= __ldg(kH[m] + (uint32_t)(rem - qm * dm) * (uint32_t)R + (rr < R ? rr : 0));
+            rem = qm;
+          }
+          c[it] = v;
+        }
+      };
       for (int s = 0; s < w.nk; ++s, ++t) {
         if ((int)(t % kSB) != bw) continue;
         if (p.b_resident) bt_base = b0 + s * kBBytes;
@@ -711,7 +735,7 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
           const bool got = mbar_wait(b_empty(bw), (use & 1u) ^ 1u, abort_flag, p.err);
           slot_ok = __all_sync(0xffffffffu, got);
         };
-        if (!lead_aligned) {
+        if (!lead) {
           // row offsets of the contraction element this lane owns
           const int kk = half * 32 + lane;
           const long long k = kst + lane;
@@ -729,12 +753,53 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
           }
           __syncwarp();
         }
+        int wrap = 32;  // elements before the first mode wraps
+        if constexpr (WRAP) {
+          lk += (uint32_t)(s - ls) * kKC;  // to stage s (64 elements per stage)
+          ls = s;
+          while (lk >= kd0) {
+            lk -= kd0;
+            ++lq;
+          }
+          wrap = (int)min(32u, kd0 - lk);
+          if (lq != cst_q) {
+            if (lq == nxt_q) {
+              now[0] = nxt[0];
+              now[1] = nxt[1];
+            } else {
+              slow_rows(lq, now);
+            }
+            cst_q = lq;
+          }
+          // (past the end of the contraction there is no next index)
+          if (wrap < 32 && kst + wrap < p.K && nxt_q != lq + 1) {
+            slow_rows(lq + 1, nxt);
+            nxt_q = lq + 1;
+          }
+        }
         const int iters = (Rp + 31) >> 5;
         for (int it = 0; it < iters; ++it) {
           const int rr = lane + 32 * it;           // rank row of this lane
           const int rs = rr < R ? rr : 0;
           float v[32];
-          if (lead_aligned) {
+          if constexpr (WRAP) {
+            // v(e) = H_0((lk + e) mod I_0, r) * (now or nxt)(r)
+            const float* h0 = kH[0] + (long long)lk * R + rs;
+            const float c0 = it ? now[1] : now[0], c1 = it ? nxt[1] : nxt[0];
+            if (wrap == 32 && kst + 32 <= w.kend) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) v[e] = __ldg(h0 + e * R);
+#pragma unroll
+              for (int e = 0; e < 32; ++e) v[e] = rr < R ? v[e] * c0 : 0.0f;
+            } else {
+              const float* h1 = h0 - (long long)kd0 * R;  // after the wrap
+#pragma unroll
+              for (int e = 0; e < 32; ++e) v[e] = __ldg((e < wrap ? h0 : h1) + e * R);
+#pragma unroll
+              for (int e = 0; e < 32; ++e)
+                v[e] = (rr < R && kst + e < w.kend) ? v[e] * (e < wrap ? c0 : c1) : 0.0f;
+            }
+          } else if (lead) {
             // modes after the first are constant over the stage:
             // v(e) = H_0(k0 + e, r) * prod_{m>=1} H_m(k_m, r)
             if (it == 0) {
@@ -1187,9 +1252,10 @@ bool tc_leaf_ok(int precision, int contract_fast, int64_t IL, int64_t IR, int R,
 int* tc_error_word(const TcScratch& s) { return static_cast<int*>(s.base); }
 
 cudaError_t tc_attributes_init() {
-  void (*const ks[4])(CUtensorMap, TcParams) = {
-      k_tc_partial_mttkrp<false, false>, k_tc_partial_mttkrp<false, true>,
-      k_tc_partial_mttkrp<true, false>, k_tc_partial_mttkrp<true, true>};
+  void (*const ks[6])(CUtensorMap, TcParams) = {
+      k_tc_partial_mttkrp<false, false, false>, k_tc_partial_mttkrp<false, true, false>,
+      k_tc_partial_mttkrp<false, false, true>,  k_tc_partial_mttkrp<false, true, true>,
+      k_tc_partial_mttkrp<true, false, false>,  k_tc_partial_mttkrp<true, true, false>};
   for (auto k : ks) {
     const cudaError_t e =
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
@@ -1267,9 +1333,18 @@ cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, i
     if (256 + (size_t)grid * 128 * R * sizeof(float) > scratch.bytes) return cudaErrorInvalidValue;
   }
   const bool split = precision == NNCP_SPLIT_BF16X3;
+  // A first mode that is no multiple of a stage, but long: the other modes' rows once
+  // per stage, not per element, pay for the wrap from 96 without the split (600 x 404 x 330 at R = 40:
+  // bf16 103 -> 76 us, TF32 124 -> 90; 136 x 100 x 1000 at R = 16: 29.0 -> 29.0; a mode
+  // of 77 to 90 5 to 10 % slower), and from 256 with it, whose builders also split the
+  // rows (600 x 404 x 330: 123 -> 98 us; 304 x 257 x 200 at R = 60: 38.4 -> 35.4; a mode
+  // of 250 51.6 -> 55.4, of 130 26.9 -> 28.4).
+  const bool wrap = !leaf && K.dim[0] % kKC != 0 && K.dim[0] >= (split ? 256 : 96);
   void (*const kern)(CUtensorMap, TcParams) =
-      leaf ? (split ? k_tc_partial_mttkrp<true, true> : k_tc_partial_mttkrp<true, false>)
-           : (split ? k_tc_partial_mttkrp<false, true> : k_tc_partial_mttkrp<false, false>);
+      leaf    ? (split ? k_tc_partial_mttkrp<true, true, false> : k_tc_partial_mttkrp<true, false, false>)
+      : !wrap ? (split ? k_tc_partial_mttkrp<false, true, false> : k_tc_partial_mttkrp<false, false, false>)
+      : split ? k_tc_partial_mttkrp<false, true, true>
+              : k_tc_partial_mttkrp<false, false, true>;
   cudaError_t e = launch_kernel(kern, dim3(grid), dim3(kThreads), p.sm.total, st, map, p);
   if (e != cudaSuccess) return e;
   if (leaf) {
