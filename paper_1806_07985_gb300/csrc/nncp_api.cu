@@ -577,7 +577,7 @@ nncp_status nncp_create(int N, const int64_t* dims, int R, nncp_ctx** out) {
   if (e == cudaSuccess) e = cudaMallocHost(&c->host_flags, 16 * sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost(&c->host_dbl, (16 + kMaxRank) * sizeof(double));
   if (e == cudaSuccess) c->host_lam = c->host_dbl + 16;
-  if (e == cudaSuccess) e = kernel_attributes_init();
+  if (e == cudaSuccess) e = kernel_attributes_init(R);
   if (e != cudaSuccess) {
     nncp_status s = cuda_fail(nullptr, e, "nncp_create");
     nncp_destroy(c);

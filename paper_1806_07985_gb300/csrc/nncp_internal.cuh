@@ -177,9 +177,9 @@ cudaError_t launch_to_bf16(const float* X, uint16_t* Y, int64_t n, cudaStream_t 
 
 // ---- factor update kernels (update_kernels.cu) -----------------------------
 
-// Shared-memory opt-ins of every kernel that needs them; once per process and
-// device, before any launch or capture.
-cudaError_t kernel_attributes_init();
+// Shared-memory opt-ins of every kernel that a problem of rank R needs, before any
+// launch or capture (each costs a new context about 6 us).
+cudaError_t kernel_attributes_init(int R);
 cudaError_t tc_attributes_init();
 
 // HALS sweep on W = H diag(lam) for every row, in place in H, followed by the

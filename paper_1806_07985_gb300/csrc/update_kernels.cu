@@ -2143,38 +2143,24 @@ size_t rows_smem(int R, bool sweep) {
 
 }  // namespace
 
-cudaError_t kernel_attributes_init() {
-  cudaError_t e = cudaSuccess;
-  const int rows = (int)rows_smem(kMaxRank, true);
-  auto opt_in = [&](auto k) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, rows);
+cudaError_t kernel_attributes_init(int R) {
+  // (the other row kernels stay below 48 KB; the update kernels are those of R)
+  cudaError_t e = cudaFuncSetAttribute(k_hals_gram<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)rows_smem(kMaxRank, true));
+  auto opt_in = [&](auto k, size_t bytes) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
-  opt_in(k_hals_gram<16>);
-  opt_in(k_hals_gram<32>);
-  opt_in(k_hals_gram<64>);
-  opt_in(k_hals_gram<128>);
-  opt_in(k_init_gram<16>);
-  opt_in(k_init_gram<32>);
-  opt_in(k_init_gram<64>);
-  opt_in(k_init_gram<128>);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_update_multi<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)multi_smem<16>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_update_multi<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)multi_smem<32>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_update_multi<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)multi_smem<64>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_update_cluster<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)cluster_smem<16>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_update_cluster<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)cluster_smem<32>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_update_cluster<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)cluster_smem<64>());
+  if (R <= 16) {
+    opt_in(k_update_multi<16>, multi_smem<16>());
+    opt_in(k_update_cluster<16>, cluster_smem<16>());
+  } else if (R <= 32) {
+    opt_in(k_update_multi<32>, multi_smem<32>());
+    opt_in(k_update_cluster<32>, cluster_smem<32>());
+  } else if (R <= 64) {
+    opt_in(k_update_multi<64>, multi_smem<64>());
+    opt_in(k_update_cluster<64>, cluster_smem<64>());
+  }
   if (e == cudaSuccess) e = simt_attributes_init();
   if (e == cudaSuccess) e = tc_attributes_init();
   return e;
