@@ -1339,9 +1339,12 @@ cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, i
   // 330 at R = 40: bf16 103 -> 76 us, TF32 124 -> 90; a mode of 130 27.0 -> 26.8, of 100
   // 16.6 -> 17.8, of 77 to 90 5 to 10 % slower), and from 256 with it, whose builders also
   // split the rows (600 x 404 x 330: 123 -> 98 us; 304 x 257 x 200 at R = 60: 38.4 -> 35.4;
-  // a mode of 250 51.6 -> 55.4, of 130 26.9 -> 28.4).  With no other mode there is nothing
-  // to save.
-  const bool wrap = !leaf && K.nm > 1 && K.dim[0] % kKC != 0 && K.dim[0] >= (split ? 256 : 192);
+  // a mode of 250 51.6 -> 55.4, of 130 26.9 -> 28.4).  A mode alone saves only its
+  // element offsets, which pays past 32 ranks (two rows per lane) and from 500 on (600 at
+  // R = 40: split 110 -> 89 us, bf16 53.8 -> 51.7; 276 at R = 33 44.3 -> 45.1 a sweep, 484
+  // at R = 26 59.1 -> 60.0).
+  const bool wrap = !leaf && K.dim[0] % kKC != 0 && K.dim[0] >= (split ? 256 : 192) &&
+                    (K.nm > 1 || (R > 32 && K.dim[0] >= 500));
   void (*const kern)(CUtensorMap, TcParams) =
       leaf    ? (split ? k_tc_partial_mttkrp<true, true, false> : k_tc_partial_mttkrp<true, false, false>)
       : !wrap ? (split ? k_tc_partial_mttkrp<false, true, false> : k_tc_partial_mttkrp<false, false, false>)

@@ -25,7 +25,7 @@ def _krp(fs, R):
 @pytest.mark.parametrize("prec,unit", [("split_bf16x3", 2.0 ** -17), ("tf32", 2.0 ** -11), ("bf16_stored", 2.0 ** -17)])
 @pytest.mark.parametrize("dims,R,split", [
     ((200, 193, 5), 17, 1), ((136, 195), 33, 1), ((192, 191, 3), 16, 1), ((264, 257, 3), 40, 1), ((16, 300, 5, 7), 64, 1),
-    ((296, 3, 4, 130), 24, 2), ((8, 1001, 11), 48, 1), ((520, 12, 255), 32, 2), ((1000, 8, 3), 5, 1)])
+    ((296, 3, 4, 130), 24, 2), ((8, 1001, 11), 48, 1), ((520, 12, 255), 32, 2), ((1000, 8, 3), 40, 1)])
 def test_long_ragged_first_modes(dims, R, split, prec, unit):
     ensure_built()
     rng = np.random.default_rng(sum(dims) + R)
