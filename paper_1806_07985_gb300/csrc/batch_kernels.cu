@@ -311,9 +311,13 @@ __device__ __forceinline__ void right_krp(const BTensor& t, int njk, int lg, KrD
     } else {
       unsigned rem = (unsigned)rest;
       for (int m = 2; m < N; ++m) {
-        const unsigned dm = (unsigned)t.dims[m];
-        const float4 h = ld_rank4(t.H[m] + (int)(rem % dm) * R, r0, R);
-        rem /= dm;
+        unsigned jm = rem;
+        if (m + 1 < N) {
+          const unsigned dm = (unsigned)t.dims[m];
+          rem = jm / dm;
+          jm -= rem * dm;
+        }
+        const float4 h = ld_rank4(t.H[m] + (int)jm * R, r0, R);
         w.x *= h.x;
         w.y *= h.y;
         w.z *= h.z;
@@ -1482,73 +1486,125 @@ k_b_pm_left_ws(const BTensor* __restrict__ ts, const int4* __restrict__ items, i
 // leaf M(a) from node {a..N} (Fig. 1): M(i, r) = sum_k T[(i + I_a k) R + r] KK(k, r),
 // KK = H_N (.) ... (.) H_{a+1}.  Item (tensor, chunk c of leaf_kc[a] rows k,
 // block of kLeafBlock outputs).  For each k the node slice of all (i, r) is
-// contiguous, so thread = output e = i R + r reads it coalesced; KK rows are
-// formed per tile of kLeafTileK rows in shared memory.  Writes lpart[c].
-__global__ void __launch_bounds__(256) k_b_mttv_leaf(const BTensor* __restrict__ ts,
-                                                     const int4* __restrict__ items, int a) {
-  const int4 it = items[blockIdx.x];
-  const BTensor& t = ts[it.x];
-  if (tensor_done(t)) return;
-  __shared__ float KKs[kLeafTileK * kBatchMaxRank];
+// contiguous, so threads read it coalesced, V outputs each (V = 4 when R % 4 == 0);
+// where a slice has at most 128 such reads, G groups of threads take the rows
+// k = g, g + G, ... of a tile and their sums are added in group order at the end.  KK
+// rows are formed per tile of kLeafTileK rows in shared memory, the rows' digits kept
+// by addition.  Bound by the latency of the node's loads: a thread per output and a
+// division per KK entry and mode left 10 x 8 slices to 80 threads.  Writes lpart[c].
+// (1500 tensors of four modes of 4 to 40, ranks 4, 8, 16: 364 us, this 87 us; 1024 of
+// three modes of 16 to 128 53 and 39 us; at six CTAs per SM, with 42 registers, 108 and 56.)
+template <int V>
+__device__ __forceinline__ void leaf_item(const BTensor& t, int a, int chunk, int block, float* KKs) {
+  using VT = typename std::conditional<V == 4, float4, float>::type;
+  constexpr int T = 256, Q = kLeafBlock / (T * V);
   const int tid = threadIdx.x;
-  const int R = t.R, N = t.N;
+  const int R = t.R, RV = R / V, N = t.N;
   const int E = (int)t.dims[a] * R;
   int K = 1;
   for (int m = a + 1; m < N; ++m) K *= (int)t.dims[m];
   const int kc = t.leaf_kc[a];
-  const int k0 = it.y * kc, k1 = min(K, k0 + kc);
-  int ep[4], rp[4];
+  const int k0 = chunk * kc, k1 = min(K, k0 + kc);
+  const int U = min(kLeafBlock, E - block * kLeafBlock) / V;  // reads of a row
+  const int G = U <= T / 2 ? T / U : 1;
+  const int g = G > 1 ? tid / U : 0, u0 = tid - g * U;
+  int rp[Q];
+  __align__(16) float acc[Q][V];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    ep[q] = it.z * kLeafBlock + tid + 256 * q;
-    rp[q] = ep[q] % R;
+  for (int q = 0; q < Q; ++q) {
+    rp[q] = (block * kLeafBlock / V + u0 + T * q) % RV;
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[q][v] = 0.0f;
   }
-  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  const float* T = t.node[a];
+  // this thread's KK entries: rank group kr of rows kk, kk + step, ... of a tile
+  const int step = T / RV, kk0 = tid / RV, kr = (tid - kk0 * RV) * V;
+  const int d = (int)t.dims[a + 1];
+  int dig = 0, rest = 0, sd = 0, sr = 0;  // digit of mode a + 1 and the rest; per step
+  const bool build = kk0 < step;
+  if (build) {
+    rest = (k0 + kk0) / d;
+    dig = k0 + kk0 - rest * d;
+    sr = step / d;
+    sd = step - sr * d;
+  }
+  const int tr = kLeafTileK / d, td = kLeafTileK - tr * d;  // per tile
+  const float* Ha = t.H[a + 1] + kr;
+  const float* node = t.node[a] + block * kLeafBlock;
   for (int kt = k0; kt < k1; kt += kLeafTileK) {
     const int nk = min(kLeafTileK, k1 - kt);
     __syncthreads();
-    // KK rows of the tile: entries x = kk R + r < nk R <= 4096, four per thread at a time
-    for (int x0 = tid; x0 < nk * R; x0 += 4 * 256) {
-      float w[4];
-      int rem[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        rem[u] = kt + (x0 + 256 * u) / R;
-        w[u] = 1.0f;
-      }
-      for (int m = a + 1; m < N; ++m) {
-        const int dm = (int)t.dims[m];
-        const float* Hm = t.H[m];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int x = x0 + 256 * u;
-          if (x < nk * R) {
-            const int jm = rem[u] % dm;
-            rem[u] /= dm;
-            w[u] *= __ldg(Hm + jm * R + x % R);
+    if (build) {
+      int x = dig, y = rest;
+#pragma unroll 2
+      for (int kk = kk0; kk < nk; kk += step) {
+        VT w = __ldg(reinterpret_cast<const VT*>(Ha + x * R));
+        float* wf = reinterpret_cast<float*>(&w);
+        unsigned rem = (unsigned)y;
+        for (int m = a + 2; m < N; ++m) {
+          unsigned jm = rem;
+          if (m + 1 < N) {
+            const unsigned dm = (unsigned)t.dims[m];
+            rem = jm / dm;
+            jm -= rem * dm;
           }
-        }
-      }
+          const VT h = __ldg(reinterpret_cast<const VT*>(t.H[m] + (int)jm * R + kr));
+          const float* hf = reinterpret_cast<const float*>(&h);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int x = x0 + 256 * u;
-        if (x < nk * R) KKs[x] = w[u];
+          for (int v = 0; v < V; ++v) wf[v] *= hf[v];
+        }
+        *reinterpret_cast<VT*>(KKs + kk * R + kr) = w;
+        kr_step(x, y, sd, sr, d);
       }
+      kr_step(dig, rest, td, tr, d);
     }
     __syncthreads();
-    const float* Tb = T + (long long)kt * E;
+    const float* Tb = node + (long long)(kt + g) * E + u0 * V;
+    const float* Kb = KKs + g * R;
+    if (g < G) {
 #pragma unroll 4
-    for (int kk = 0; kk < nk; ++kk) {
+      for (int kk = g; kk < nk; kk += G, Tb += G * E, Kb += G * R) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (ep[q] < E) acc[q] = fmaf(Tb[(long long)kk * E + ep[q]], KKs[kk * R + rp[q]], acc[q]);
+        for (int q = 0; q < Q; ++q)
+          if (u0 + T * q < U) {
+            const VT x = *reinterpret_cast<const VT*>(Tb + T * V * q);
+            const VT w = *reinterpret_cast<const VT*>(Kb + rp[q] * V);
+            const float* xf = reinterpret_cast<const float*>(&x);
+            const float* wf = reinterpret_cast<const float*>(&w);
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[q][v] = fmaf(xf[v], wf[v], acc[q][v]);
+          }
+      }
     }
   }
-  float* out = t.lpart + (long long)it.y * E;
+  float* out = t.lpart + (long long)chunk * E + block * kLeafBlock;
+  if (G > 1) {
+    __syncthreads();
+    if (g < G) *reinterpret_cast<VT*>(KKs + tid * V) = *reinterpret_cast<const VT*>(acc[0]);
+    __syncthreads();
+    if (tid < U) {
+#pragma unroll 1
+      for (int h = 1; h < G; ++h)
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (ep[q] < E) out[ep[q]] = acc[q];
+        for (int v = 0; v < V; ++v) acc[0][v] += KKs[(h * U + tid) * V + v];
+      *reinterpret_cast<VT*>(out + tid * V) = *reinterpret_cast<const VT*>(acc[0]);
+    }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+    if (u0 + T * q < U) *reinterpret_cast<VT*>(out + (u0 + T * q) * V) = *reinterpret_cast<const VT*>(acc[q]);
+}
+
+__global__ void __launch_bounds__(256, 4) k_b_mttv_leaf(const BTensor* __restrict__ ts,
+                                                     const int4* __restrict__ items, int a) {
+  const int4 it = items[blockIdx.x];
+  const BTensor& t = ts[it.x];
+  if (tensor_done(t)) return;
+  __shared__ __align__(16) float KKs[kLeafTileK * kBatchMaxRank];
+  if ((t.R & 3) == 0)
+    leaf_item<4>(t, a, it.y, it.z, KKs);
+  else
+    leaf_item<1>(t, a, it.y, it.z, KKs);
 }
 
 // child node {a+1..N} from node {a..N}: out(j, r) = sum_i T[(i + I_a j) R + r] H_a(i, r)
