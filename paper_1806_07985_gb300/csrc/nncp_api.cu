@@ -247,8 +247,10 @@ void drop_graph(nncp_ctx* c) {
 }
 
 // ---- one partial MTTKRP from the root (precision-dependent) ----------------
+// early: see launch_simt_mttkrp
 
-cudaError_t pm_right(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* leaf = nullptr) {
+cudaError_t pm_right(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* leaf = nullptr,
+                     bool early = false) {
   const int s = c->split, N = c->N;
   const int64_t IL = prod(c->dims, 0, s - 1), IR = prod(c->dims, s, N - 1);
   KrpDesc none;
@@ -258,10 +260,11 @@ cudaError_t pm_right(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* lea
     return tc_partial_mttkrp(c->precision, /*contract_fast=*/0, c->X, IL, IR, KQ, c->R, out,
                              c->tc, c->num_sms, st, leaf);
   return launch_simt_mttkrp(static_cast<const float*>(c->X), 1, IL, IR, none, KQ, c->R, out,
-                            c->partials, c->part_cap, c->num_sms, st);
+                            c->partials, c->part_cap, c->num_sms, st, early);
 }
 
-cudaError_t pm_left(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* leaf = nullptr) {
+cudaError_t pm_left(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* leaf = nullptr,
+                    bool early = false) {
   const int s = c->split, N = c->N;
   const int64_t IL = prod(c->dims, 0, s - 1), IR = prod(c->dims, s, N - 1);
   KrpDesc none;
@@ -271,7 +274,7 @@ cudaError_t pm_left(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* leaf
     return tc_partial_mttkrp(c->precision, /*contract_fast=*/1, c->X, IL, IR, KL, c->R, out,
                              c->tc, c->num_sms, st, leaf);
   return launch_simt_mttkrp(static_cast<const float*>(c->X), IL, IR, 1, KL, none, c->R, out,
-                            c->partials, c->part_cap, c->num_sms, st);
+                            c->partials, c->part_cap, c->num_sms, st, early);
 }
 
 cudaError_t update_mode(nncp_ctx* c, int n, cudaStream_t st) {
@@ -360,6 +363,7 @@ void node_stamp(nncp_ctx* c, int h, int d) {
   for (int k = 0; k < c->N; ++k) c->node_ver[h][d][k] = c->fver[k];
 }
 
+// (captured by capture_iterations alone, where no kernel writes the tensor)
 cudaError_t run_iteration(nncp_ctx* c, cudaStream_t st) {
   const int s = c->split, N = c->N;
   if (!c->dimtree) {
@@ -368,7 +372,8 @@ cudaError_t run_iteration(nncp_ctx* c, cudaStream_t st) {
       KrpDesc KL = krp(c, 0, n - 1), KQ = krp(c, n + 1, N - 1);
       cudaError_t e = launch_simt_mttkrp(static_cast<const float*>(c->X), prod(c->dims, 0, n - 1),
                                          c->dims[n], prod(c->dims, n + 1, N - 1), KL, KQ, c->R,
-                                         c->Mbuf, c->partials, c->part_cap, c->num_sms, st);
+                                         c->Mbuf, c->partials, c->part_cap, c->num_sms, st,
+                                         /*early=*/true);
       if (e == cudaSuccess) e = update_mode(c, n, st);
       if (e != cudaSuccess) return e;
     }
@@ -384,12 +389,12 @@ cudaError_t run_iteration(nncp_ctx* c, cudaStream_t st) {
   const bool fuse_r = c->fuse_leaf && N - s >= 2 &&
                       tc_leaf_ok(c->precision, 1, IL, IR, c->R, rf.I, c->num_sms);
   float* TL = (s == 1) ? c->Mbuf : c->node[0][0];
-  cudaError_t e = pm_right(c, TL, st, fuse_l ? &lf : nullptr);
+  cudaError_t e = pm_right(c, TL, st, fuse_l ? &lf : nullptr, /*early=*/true);
   if (e != cudaSuccess) return e;
   e = visit(c, TL, 0, s - 1, 0, 0, st, fuse_l);
   if (e != cudaSuccess) return e;
   float* TR = (N - s == 1) ? c->Mbuf : c->node[1][0];
-  e = pm_left(c, TR, st, fuse_r ? &rf : nullptr);
+  e = pm_left(c, TR, st, fuse_r ? &rf : nullptr, /*early=*/true);
   if (e != cudaSuccess) return e;
   return visit(c, TR, s, N - 1, 1, s, st, fuse_r);
 }

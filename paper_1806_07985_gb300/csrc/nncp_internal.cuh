@@ -15,7 +15,10 @@ namespace nncp {
 // calls pdl_wait() before its first access to memory that an earlier kernel
 // writes, or that a later one writes while an earlier one may still read it.  pdl_wait() returns
 // once every predecessor grid has completed and its writes are visible, so the
-// chain stays ordered transitively.  Small kernels then call pdl_trigger(), which
+// chain stays ordered transitively.  (Only the tensor may be read earlier, and only
+// in the library's own capture of an iteration, where no kernel writes it: the
+// entry points also run on a caller's stream, which may be captured behind a
+// kernel that writes the tensor and triggers early.)  Small kernels then call pdl_trigger(), which
 // lets their successor be scheduled on the SMs they leave free; large grids do
 // not, so their successor is scheduled as their CTAs exit.  Outside such a
 // launch both return at once.
@@ -119,11 +122,13 @@ struct SolveState {
 // for i < I, r < R: the generic (direct or partial) MTTKRP on CUDA cores.
 // X is float32.  When the contraction is split across CTAs the per-chunk
 // results go to `partials` (capacity `part_cap` floats) and are summed in a
-// fixed order, so results are bitwise reproducible.
+// fixed order, so results are bitwise reproducible.  early: nothing that may
+// still run when this launch starts writes X (in the library's own capture of
+// an iteration), so tensor tiles may be read before pdl_wait().
 cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
                                const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,
                                float* partials, size_t part_cap, int num_sms,
-                               cudaStream_t st);
+                               cudaStream_t st, bool early = false);
 size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms);
 cudaError_t simt_attributes_init();
 

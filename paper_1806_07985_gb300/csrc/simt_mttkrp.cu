@@ -79,6 +79,7 @@ struct SimtArgs {
   int gsh;                // 2^gsh lanes copy a factor row (all of it in one go when vecb)
   int fk, fc;             // threads / (RP / 4) and the remainder
   int vecx, vecb, veco, evict;
+  int early;              // tensor tiles before the wait for the preceding kernel
   int nm;                 // contracted modes, fastest first
   int dim[kMaxModes];     // their lengths
   int dstep, mag0, magl;  // 32 mod dim[0]; ceil(2^16 / dim[0]) and / L below 32, else 0
@@ -449,8 +450,10 @@ k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
     for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
 
   __syncthreads();
-  // the tensor is written by no kernel of an iteration: its first tiles stream
-  // in while the preceding kernel finishes
+  // the tensor is written by no kernel of an iteration: there (early) its first
+  // tiles stream in while the preceding kernel finishes; a caller's stream may
+  // hold a kernel that writes it
+  if (!p.early) pdl_wait();
   load_x(tabs[0], 0);
   load_x(tabs[1], 1);
   pdl_wait();
@@ -737,7 +740,7 @@ bool plan_simt(int64_t L, int64_t I, int64_t Q, const KrpDesc& KL, const KrpDesc
 
 // The launches for the rank columns [r0, r0 + pl.a.R) of a rank-R MTTKRP.
 cudaError_t launch_columns(const float* X, int R, int r0, float* out, float* partials,
-                           SimtPlan pl, cudaStream_t st) {
+                           SimtPlan pl, cudaStream_t st, bool early) {
   SimtArgs& a = pl.a;
   auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
   const bool KC = a.L > 1;
@@ -755,6 +758,7 @@ cudaError_t launch_columns(const float* X, int R, int r0, float* out, float* par
   // a tensor that cannot stay in the 126 MB L2 is marked evict-first, so that
   // its stream leaves the nodes and factors there
   a.evict = (double)a.I * a.K * sizeof(float) > 96e6;
+  a.early = early;
   const int copies = a.vecb ? a.R / 4 : a.R;
   while (a.gsh < 5 && (1 << a.gsh) < copies) ++a.gsh;
   cudaError_t e = launch_kernel(KC ? k_simt_mttkrp<true> : k_simt_mttkrp<false>,
@@ -804,7 +808,7 @@ size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms)
 cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
                                const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,
                                float* partials, size_t part_cap, int num_sms,
-                               cudaStream_t st) {
+                               cudaStream_t st, bool early) {
   // ranks in one launch unless the factor rows of a step (long products of short
   // modes at a high rank) do not fit in shared memory: then in column blocks
   int cols = R;
@@ -817,7 +821,7 @@ cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
     const int n = std::min(cols, R - r0);
     if (n != cols && !plan_simt(L, I, Q, KL, KQ, n, partials ? part_cap : 0, num_sms, &pl))
       return cudaErrorInvalidValue;
-    const cudaError_t e = launch_columns(X, R, r0, out, partials, pl, st);
+    const cudaError_t e = launch_columns(X, R, r0, out, partials, pl, st, early);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
