@@ -258,7 +258,7 @@ cudaError_t pm_right(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* lea
   KrpDesc KQ = krp(c, s, N - 1);
   if (c->precision != NNCP_FP32_SIMT)
     return tc_partial_mttkrp(c->precision, /*contract_fast=*/0, c->X, IL, IR, KQ, c->R, out,
-                             c->tc, c->num_sms, st, leaf);
+                             c->tc, c->num_sms, st, leaf, early);
   return launch_simt_mttkrp(static_cast<const float*>(c->X), 1, IL, IR, none, KQ, c->R, out,
                             c->partials, c->part_cap, c->num_sms, st, early);
 }
@@ -272,7 +272,7 @@ cudaError_t pm_left(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* leaf
   KrpDesc KL = krp(c, 0, s - 1);
   if (c->precision != NNCP_FP32_SIMT)
     return tc_partial_mttkrp(c->precision, /*contract_fast=*/1, c->X, IL, IR, KL, c->R, out,
-                             c->tc, c->num_sms, st, leaf);
+                             c->tc, c->num_sms, st, leaf, early);
   return launch_simt_mttkrp(static_cast<const float*>(c->X), IL, IR, 1, KL, none, c->R, out,
                             c->partials, c->part_cap, c->num_sms, st, early);
 }

@@ -104,6 +104,7 @@ struct TcParams {
   int direct;  // MMA reads the TMA stage (no converter)
   int a_mn;    // ... MN-major (bf16 tensor, contract_slow)
   int bf16x;   // tensor stored as bf16
+  int early;   // the tensor may be read before the wait for the preceding kernel
   int b_resident;  // every unit spans the whole contraction: B formed once per CTA
   // Stages accumulated in one tensor-memory accumulator before it is added into
   // float32 registers (split-BF16x3; one segment per unit otherwise).  The
@@ -415,7 +416,9 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
   // epilogue (output) touch memory that other kernels of the iteration write or
   // read, so only they wait for it (pdl_wait); the producer streams the tensor,
   // which nothing in the iteration writes, and the converters fill the tensor-
-  // memory A stages from it in the meantime.  The kernel does not trigger its
+  // memory A stages from it in the meantime.  Where that is not known (a caller's
+  // stream: p.early = 0) every thread waits before the roles part, so that no
+  // bounded wait runs on while the predecessor does.  The kernel does not trigger its
   // successor early: that one is scheduled as CTAs exit, and CTAs placed on the
   // first SMs to free up would crowd there instead of spreading over the GPU.
   extern __shared__ uint8_t smem_dyn[];
@@ -501,6 +504,8 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
 
   const long long n_units = p.n_units;
   const int R = p.R;
+
+  if (!p.early) pdl_wait();
 
   if (warp == kWarpTMA) {
     // ---------------------------------------------------------- producer --
@@ -1268,7 +1273,7 @@ cudaError_t tc_attributes_init() {
 cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, int64_t IL,
                               int64_t IR, const KrpDesc& K, int R, float* out,
                               const TcScratch& scratch, int num_sms, cudaStream_t st,
-                              const TcLeaf* leaf) {
+                              const TcLeaf* leaf, bool early) {
   if (!load_encode()) return cudaErrorNotSupported;
   if (R > kMaxRp || !scratch.base) return cudaErrorInvalidValue;
   const bool bf16x = precision == NNCP_BF16_STORED;
@@ -1303,6 +1308,7 @@ cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, i
   p.mode = precision;
   p.contract_fast = contract_fast;
   p.bf16x = bf16x;
+  p.early = early;
   p.a_mn = bf16x && !contract_fast;
   p.direct = (contract_fast && precision != NNCP_SPLIT_BF16X3) || p.a_mn;
   p.seg = precision == NNCP_SPLIT_BF16X3 ? kSegStages : (1 << 30);

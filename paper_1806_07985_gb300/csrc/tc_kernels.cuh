@@ -49,9 +49,10 @@ bool tc_leaf_ok(int precision, int contract_fast, int64_t IL, int64_t IR, int R,
 //   contract_fast = 0:  out(i, r) = sum_j X[i + IL*j] * K(j, r)   (root -> left node)
 // K is the Khatri-Rao product described by `K` (formed on the fly).  With
 // `leaf` (tc_leaf_ok), leaf->out receives the fused first multi-TTV as well.
+// early: as in launch_simt_mttkrp.
 cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, int64_t IL,
                               int64_t IR, const KrpDesc& K, int R, float* out,
                               const TcScratch& scratch, int num_sms, cudaStream_t st,
-                              const TcLeaf* leaf = nullptr);
+                              const TcLeaf* leaf = nullptr, bool early = false);
 
 }  // namespace nncp

@@ -89,3 +89,27 @@ def test_partial_fp32(side):
 def test_context_mttkrp_fp32(tree):
     Ms = [torch.empty(d, R, device="cuda") for d in DIMS]
     _context("fp32_simt", lambda c: [c.mttkrp(n + 1, tree, M) for n, M in enumerate(Ms)], Ms)
+
+
+@pytest.mark.parametrize("side", [0, 1])
+@pytest.mark.parametrize("precision", ["tf32", "split_bf16x3"])
+def test_partial_tensor_cores(precision, side):
+    T = torch.empty(DIMS[0] if side == 0 else DIMS[1] * DIMS[2], R, device="cuda")
+    _context(precision, lambda c: c.partial_mttkrp(side, T), [T])
+
+
+@pytest.mark.parametrize("side", [0, 1])
+def test_partial_bf16(side):
+    T = torch.empty(DIMS[0] if side == 0 else DIMS[1] * DIMS[2], R, device="cuda")
+
+    def make(X, stream):
+        Xb = torch.empty(X.numel(), dtype=torch.bfloat16, device="cuda")
+        c = nncp.Context(DIMS, R, precision="bf16_stored", root_split=1, stream=stream)
+        c.set_tensor(Xb)
+        c.set_factors([_rand(d, R, seed=n) for n, d in enumerate(DIMS)])
+
+        def consume():
+            nncp.nncp_tensor_to_bf16(X, Xb, stream=stream)
+            c.partial_mttkrp(side, T)
+        return consume, c.close
+    _check(make, [T])
