@@ -54,49 +54,11 @@
 #include <algorithm>
 
 #include "nncp_internal.cuh"
+#include "simt_plan.cuh"
 
 namespace nncp {
 
 namespace {
-
-constexpr int kBK = 32;        // contraction elements per step
-constexpr int kThreadsMax = 256;  // computing threads; the feeder warp comes after them
-constexpr int kStages = 3;
-constexpr int kTM = 4;         // output rows per thread
-constexpr int kTabs = 4;       // step descriptors in flight
-constexpr int kSmemMax = 232448;  // 227 KB per CTA on sm_103a
-constexpr int kSmemSM = 233472;   // 228 KB per SM, 1 KB of it reserved per CTA
-constexpr int kStaticSmem = 512; // descriptors (checked below)
-
-struct SimtArgs {
-  const float* X;
-  long long L, I, K;
-  int R, RP, ld;          // rank columns; padded to whole groups of eight; row stride of H and out
-  int CG, RGH, KG;        // rank groups, row groups, splits of a step
-  int bm_log2;            // BM = 32 RGH
-  int tl;                 // threads that load: the most whole pairs of computing warps
-  int b_all;              // the computing threads load the factor rows too
-  int gsh;                // 2^gsh lanes copy a factor row (all of it in one go when vecb)
-  int fk, fc;             // threads / (RP / 4) and the remainder
-  int vecx, vecb, veco, evict;
-  int early;              // tensor tiles before the wait for the preceding kernel
-  int nm;                 // contracted modes, fastest first
-  int dim[kMaxModes];     // their lengths
-  int dstep, mag0, magl;  // 32 mod dim[0]; ceil(2^16 / dim[0]) and / L below 32, else 0
-  long long rstep;        // 32 / dim[0]
-  const float* H[kMaxModes];
-  long long lstep, qstep;  // 32 mod L, 32 / L
-  int nrest_max;           // rest rows a stage has room for
-  int red_pairs;           // column pairs per round of the KG sums (1, 2 or 4)
-  int x_floats, stage_floats;
-  long long nk;            // steps per whole tile
-  long long whole;         // tiles taken whole
-  long long U2;            // steps of the tiles cut into runs
-  int G2, two;             // runs; partial slots per run (1 or 2)
-  float* out;
-  float* slots;
-  long long slot_floats;   // BM x R
-};
 
 // One step: the tile it belongs to and the position of its first element.
 struct StepTab {
@@ -639,103 +601,6 @@ k_simt_fixup(const float* __restrict__ slots, float* __restrict__ out, long long
     for (int k = 0; k < W; ++k) s += part[k][threadIdx.x & 31];
   }
   if (in) out[(i0 + e / R) * ld + e % R] = s;
-}
-
-long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
-
-struct SimtPlan {
-  SimtArgs a;
-  int BM, threads, grid;
-  size_t smem;
-};
-
-// Tile, thread split and work split of one MTTKRP; cap: floats of scratch for
-// partial tiles.
-bool plan_simt(int64_t L, int64_t I, int64_t Q, const KrpDesc& KL, const KrpDesc& KQ, int R,
-               size_t cap, int num_sms, SimtPlan* pl) {
-  SimtArgs& a = pl->a;
-  a = SimtArgs{};
-  a.L = L;
-  a.I = I;
-  a.K = (long long)L * Q;
-  a.R = R;
-  a.nk = cdiv(a.K, kBK);
-  for (const KrpDesc* d : {&KL, &KQ})
-    for (int m = 0; m < d->nm; ++m) {
-      if (a.nm == kMaxModes) return false;
-      a.dim[a.nm] = (int)d->dim[m];
-      a.H[a.nm++] = d->H[m];
-    }
-  if (a.nm < 1) return false;
-  a.dstep = kBK % a.dim[0];
-  a.rstep = kBK / a.dim[0];
-  a.mag0 = a.dim[0] < kBK ? (65535 + a.dim[0]) / a.dim[0] : 0;
-  a.magl = L < kBK ? (int)((65535 + L) / L) : 0;
-  a.lstep = kBK % L;
-  a.qstep = kBK / L;
-  a.nrest_max = a.nm > 1 ? std::min(kBK, (kBK - 1) / a.dim[0] + 2) : 0;
-  a.CG = (R + 7) / 8;
-  a.RP = 8 * a.CG;
-  // tile rows 32 RGH: the least work for the busiest SM, a step costing its
-  // rows plus the part that does not depend on them
-  double best = 0.0;
-  for (int c = 0; c < 4; ++c) {
-    SimtPlan t = *pl;
-    SimtArgs& b = t.a;
-    b.RGH = 1 << c;
-    b.bm_log2 = 5 + c;
-    t.BM = 32 << c;
-    if (8 * b.RGH * a.CG > kThreadsMax) break;
-    // splitting a step further than over four warps only shortens each one's
-    // share of it: 301 x 257 x 199, R = 20, 72 us at eight warps against 68
-    b.KG = 1;
-    while (b.KG < 8 && 8 * b.RGH * a.CG * b.KG * 2 <= kThreadsMax / 2) b.KG *= 2;
-    const int computing = 8 * b.RGH * a.CG * b.KG;
-    t.threads = (computing + 31) / 32 * 32;
-    b.tl = t.threads / 64 * 64;
-    const int rest = (a.nm - 1) * a.nrest_max;
-    // more copies of factor rows than a warp issues in a step's time
-    b.b_all = (kBK + rest) * (R % 4 == 0 ? R / 4 : R) > 32 * 16;
-    b.fk = t.threads / (a.RP / 4);
-    b.fc = t.threads % (a.RP / 4);
-    b.x_floats = t.BM * kBK;
-    b.stage_floats = b.x_floats + (kBK + rest) * a.RP;
-    b.red_pairs = 4;
-    while (b.red_pairs > 1 && computing / 2 * b.red_pairs * kTM * 2 > b.stage_floats) b.red_pairs /= 2;
-    t.smem = (size_t)kStages * b.stage_floats * sizeof(float);
-    if (t.smem > (size_t)(kSmemMax - kStaticSmem)) break;
-    // CTAs per SM at once: shared memory, and the registers of five warps (96 a
-    // thread) on each of its four schedulers
-    const int occ = std::max(1, std::min((int)(kSmemSM / (t.smem + kStaticSmem + 1024)),
-                                         20 / (t.threads / 32 + 1)));
-    const long long G = (long long)num_sms * occ, gx = cdiv(I, t.BM);
-    long long left = gx % G;
-    if (left * 10 >= G * 9) left = 0;  // a wave nine tenths full is left whole
-    b.whole = gx - left;
-    b.slot_floats = (long long)t.BM * R;
-    if (left > 0) {
-      // at least four steps per run; one slot per run where runs end with tiles
-      long long g2 = std::max(left, std::min(G, left * a.nk / 4));
-      const long long slots = (long long)(cap / (size_t)b.slot_floats);
-      if (g2 % left != 0 && 2 * g2 > slots) g2 = left * (g2 / left);
-      if (g2 % left == 0 && g2 > slots) g2 = left * std::max(1LL, slots / left);
-      if (g2 <= left) {
-        b.whole = gx;
-      } else {
-        b.U2 = left * a.nk;
-        b.G2 = (int)g2;
-        b.two = g2 % left != 0;
-      }
-    }
-    t.grid = (int)std::max<long long>(std::min(G, b.whole), b.G2);
-    const double steps = (double)cdiv(b.whole, G) * a.nk + (b.G2 ? (double)cdiv(b.U2, b.G2) : 0.0);
-    const double cost = steps * (double)cdiv(t.grid, num_sms) * (t.BM + 24) * (occ == 1 ? 1.15 : 1.0);
-    if (best == 0.0 || cost < best) {
-      best = cost;
-      *pl = t;
-    }
-  }
-  return best > 0.0;
 }
 
 // The launches for the rank columns [r0, r0 + pl.a.R) of a rank-R MTTKRP.
