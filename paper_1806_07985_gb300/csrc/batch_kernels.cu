@@ -58,8 +58,8 @@ __global__ void __launch_bounds__(256) k_b_sumsq(const BTensor* __restrict__ ts,
   const float4* x4 = reinterpret_cast<const float4*>(x);
   double acc = 0.0;
   for (int v0 = threadIdx.x; v0 < n4; v0 += 8 * 256) {
-    // eight loads in flight; into float64 after each eight, which keeps
-    // float32's range out of the sum
+    // eight loads in flight; into float64 after each eight (in float64 alone where
+    // their sum leaves float32's range)
     float4 a[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q)
@@ -68,7 +68,13 @@ __global__ void __launch_bounds__(256) k_b_sumsq(const BTensor* __restrict__ ts,
 #pragma unroll
     for (int q = 0; q < 8; ++q)
       s.add(a[q].x * a[q].x + a[q].y * a[q].y + a[q].z * a[q].z + a[q].w * a[q].w);
-    acc += s.value();
+    if (isfinite(s.hi)) {
+      acc += s.value();
+    } else {
+      for (int q = 0; q < 8; ++q)
+        acc += ((double)a[q].x * a[q].x + (double)a[q].y * a[q].y) +
+               ((double)a[q].z * a[q].z + (double)a[q].w * a[q].w);
+    }
   }
   if ((int)threadIdx.x < n - 4 * n4) {
     const float v = x[4 * n4 + threadIdx.x];

@@ -270,13 +270,24 @@ k_sumsq_partial(const void* __restrict__ Xv, int bf16, long long n, double* __re
       a0.add(s);
     }
   };
-  // into float64 after every eight loads, which keeps float32's range out of
-  // the sum; an infinite square stays infinite
+  // the same in float64, for sums past float32's range (and what is not finite)
+  auto square64 = [&](const uint4& v) {
+    const unsigned u[4] = {v.x, v.y, v.z, v.w};
+    double s = 0.0;
+    for (int i = 0; i < 4; ++i) {
+      const double x = __uint_as_float(bf16 ? u[i] << 16 : u[i]);
+      const double y = bf16 ? __uint_as_float(u[i] & 0xffff0000u) : 0.0f;
+      s += x * x + y * y;
+    }
+    return s;
+  };
+  // into float64 after every eight loads; false: their sum left float32's range
   double acc = 0.0;
   auto flush = [&]() {
-    const float h = a0.hi + a1.hi;
-    acc += isfinite(h) ? ((double)a0.hi + (double)a1.hi) + (double)(a0.lo + a1.lo) : (double)h;
+    const bool in = isfinite(a0.hi + a1.hi);
+    if (in) acc += ((double)a0.hi + (double)a1.hi) + (double)(a0.lo + a1.lo);
     a0 = a1 = SumFF();
+    return in;
   };
   long long t = t0;
   for (; t + 7 * stride < nv; t += 8 * stride) {  // eight loads in flight
@@ -285,16 +296,17 @@ k_sumsq_partial(const void* __restrict__ Xv, int bf16, long long n, double* __re
     for (int q = 0; q < 8; ++q) v[q] = __ldcs(V + t + q * stride);
 #pragma unroll
     for (int q = 0; q < 8; ++q) square(v[q]);
-    flush();
+    if (!flush())
+      for (int q = 0; q < 8; ++q) acc += square64(v[q]);
   }
-  for (; t < nv; t += stride) square(__ldcs(V + t));
-  flush();
+  for (long long r = t; r < nv; r += stride) square(__ldcs(V + r));
+  if (!flush())
+    for (; t < nv; t += stride) acc += square64(V[t]);
   for (long long e = nv * per + t0; e < n; e += stride) {
-    const float x = bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(Xv)[e])
-                         : static_cast<const float*>(Xv)[e];
-    a0.add(x * x);
+    const double x = bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(Xv)[e])
+                          : static_cast<const float*>(Xv)[e];
+    acc += x * x;
   }
-  flush();
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
   __syncthreads();
