@@ -202,7 +202,8 @@ struct nncp_batch {
   char* ws = nullptr;
   cudaStream_t work = nullptr;
   cudaGraphExec_t graph = nullptr;
-  int* host_done = nullptr;
+  cudaEvent_t ev_poll[2] = {};
+  int* host_done = nullptr;  // pinned: [1] error word, [2], [3] two polls of the count
   bool have_data = false;
   // schedule of the two root phases: -1 = chosen by the tuner at the next run
   int want_right = -1, want_left = -1;
@@ -409,6 +410,8 @@ nncp_status nncp_batch_create(int count, int N, const int64_t* dims, const int* 
   b->dims.assign(dims, dims + (size_t)count * N);
   b->R.assign(R, R + count);
   cudaError_t e = cudaStreamCreateWithFlags(&b->work, cudaStreamNonBlocking);
+  for (cudaEvent_t& ev : b->ev_poll)
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMallocHost(&b->host_done, 4 * sizeof(int));
   if (e == cudaSuccess) e = batch_attributes_init();
   if (e != cudaSuccess) {
@@ -523,18 +526,23 @@ nncp_status nncp_batch_run(nncp_batch* b, int max_iters, double tol, int* iters_
       return bfail(b, NNCP_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
     }
   }
-  // with tol <= 0 only a non-finite fit stops a tensor before max_iters: no
-  // count is read back before the end of a long run
-  int launched = 0, every = tol > 0.0 ? 4 : 64;
-  while (launched < max_iters) {
+  // Iterations in batches, the count of finished tensors copied back after each.
+  // With tol <= 0 only a non-finite fit stops a tensor before max_iters, so the host
+  // looks one batch behind and the GPU never waits for it.
+  const int lag = tol > 0.0 ? 0 : 1;
+  int launched = 0, every = 4;
+  for (int k = 0;; ++k) {
     const int n = std::min(every, max_iters - launched);
-    for (int k = 0; k < n; ++k) BCK(cudaGraphLaunch(b->graph, b->work));
+    for (int i = 0; i < n; ++i) BCK(cudaGraphLaunch(b->graph, b->work));
     launched += n;
     if (launched >= max_iters) break;
-    BCK(cudaMemcpyAsync(b->host_done, done, sizeof(int), cudaMemcpyDeviceToHost, b->work));
-    BCK(cudaStreamSynchronize(b->work));
-    if (b->host_done[0] >= b->count) break;
-    every = tol > 0.0 ? std::min(every * 2, 16) : 64;
+    BCK(cudaMemcpyAsync(b->host_done + 2 + (k & 1), done, sizeof(int), cudaMemcpyDeviceToHost, b->work));
+    BCK(cudaEventRecord(b->ev_poll[k & 1], b->work));
+    if (k >= lag) {
+      BCK(cudaEventSynchronize(b->ev_poll[(k - lag) & 1]));
+      if (b->host_done[2 + ((k - lag) & 1)] >= b->count) break;
+      every = std::min(every * 2, 16);
+    }
   }
   int* d_iters = at<int>(b, b->off_out_iters);
   double* d_fits = at<double>(b, b->off_out_fits);
@@ -658,6 +666,8 @@ void nncp_batch_destroy(nncp_batch* b) {
   if (!b) return;
   if (b->work) cudaStreamSynchronize(b->work);
   if (b->graph) cudaGraphExecDestroy(b->graph);
+  for (cudaEvent_t ev : b->ev_poll)
+    if (ev) cudaEventDestroy(ev);
   if (b->work) cudaStreamDestroy(b->work);
   if (b->host_done) cudaFreeHost(b->host_done);
   delete b;

@@ -46,6 +46,10 @@ struct nncp_ctx {
   cudaStream_t user_stream = nullptr;
   cudaStream_t work = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+  // the flags after a batch of iterations are copied on a stream of their own: on
+  // `work` the copy would hold up the next batch (64^3: 5 us)
+  cudaStream_t poll = nullptr;
+  cudaEvent_t ev_batch = nullptr, ev_poll[2] = {};
   int device = 0, num_sms = 148;
 
   char* ws = nullptr;
@@ -71,7 +75,7 @@ struct nncp_ctx {
   cudaGraphExec_t graph = nullptr;   // one outer iteration
   cudaGraphExec_t graph4 = nullptr;  // kGraphIters outer iterations, back to back
   int graph_kernels = 0;
-  int* host_flags = nullptr;  // pinned
+  int* host_flags = nullptr;  // pinned: [0..3] a solve's flags, [4..11] two polls, [12] error word
   double* host_dbl = nullptr; // pinned
   double* host_lam = nullptr; // pinned, kMaxRank entries after host_dbl's 16
   bool initialised = false;   // nncp_solve_begin ran on the current state
@@ -579,6 +583,10 @@ nncp_status nncp_create(int N, const int64_t* dims, int R, nncp_ctx** out) {
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->work, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->poll, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_batch, cudaEventDisableTiming);
+  for (cudaEvent_t& ev : c->ev_poll)
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMallocHost(&c->host_flags, 16 * sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost(&c->host_dbl, (16 + kMaxRank) * sizeof(double));
   if (e == cudaSuccess) c->host_lam = c->host_dbl + 16;
@@ -841,19 +849,26 @@ nncp_status nncp_solve_bound(nncp_ctx* c, int max_iters, double tol, double* lam
   if ((s = begin_on_work(c)) != NNCP_OK) return s;
   if ((s = solve_init(c, tol)) != NNCP_OK) return s;
   if ((s = ensure_graph(c)) != NNCP_OK) return s;
-  // with tol <= 0 only a non-finite fit stops a solve early, and what follows
-  // it changes nothing: no flag is read back before the end of a long run
-  int launched = 0, check_every = tol > 0.0 ? 4 : 64;
-  while (launched < max_iters) {
-    int batch = std::min(check_every, max_iters - launched);
+  // Iterations in batches, the flags copied back after each.  With tol <= 0 only a
+  // non-finite fit stops a solve, and what follows it changes nothing, so the host
+  // looks one batch behind and the GPU never waits for it.
+  const int lag = tol > 0.0 ? 0 : 1;
+  int launched = 0, check_every = 4;
+  for (int b = 0;; ++b) {
+    const int batch = std::min(check_every, max_iters - launched);
     CK(launch_iterations(c, batch));
     launched += batch;
     if (launched >= max_iters) break;
-    CK(cudaMemcpyAsync(c->host_flags, c->st.flags, 4 * sizeof(int), cudaMemcpyDeviceToHost,
-                       c->work));
-    CK(cudaStreamSynchronize(c->work));
-    if (c->host_flags[0]) break;
-    check_every = tol > 0.0 ? std::min(check_every * 2, 32) : 64;
+    CK(cudaEventRecord(c->ev_batch, c->work));
+    CK(cudaStreamWaitEvent(c->poll, c->ev_batch, 0));
+    CK(cudaMemcpyAsync(c->host_flags + 4 + 4 * (b & 1), c->st.flags, 4 * sizeof(int),
+                       cudaMemcpyDeviceToHost, c->poll));
+    CK(cudaEventRecord(c->ev_poll[b & 1], c->poll));
+    if (b >= lag) {
+      CK(cudaEventSynchronize(c->ev_poll[(b - lag) & 1]));
+      if (c->host_flags[4 + 4 * ((b - lag) & 1)]) break;
+      check_every = std::min(check_every * 2, 32);
+    }
   }
   // everything the call returns, in one round trip: the flags, the last fit
   // (scalars[5]), lambda and the tensor-core error word
@@ -866,6 +881,7 @@ nncp_status nncp_solve_bound(nncp_ctx* c, int max_iters, double tol, double* lam
     CK(cudaMemcpyAsync(c->host_flags + 12, tc_error_word(c->tc), sizeof(int), cudaMemcpyDeviceToHost,
                        c->work));
   CK(cudaStreamSynchronize(c->work));
+  CK(cudaStreamSynchronize(c->poll));  // the workspace is the caller's again
   const int iters = c->host_flags[2];
   if (lambda_out) memcpy(lambda_out, c->host_lam, c->R * sizeof(double));
   if (iters_out) *iters_out = iters;
@@ -1162,9 +1178,14 @@ const char* nncp_global_error(void) { return g_error.c_str(); }
 void nncp_destroy(nncp_ctx* c) {
   if (!c) return;
   if (c->work) cudaStreamSynchronize(c->work);
+  if (c->poll) cudaStreamSynchronize(c->poll);
   drop_graph(c);
   if (c->ev_in) cudaEventDestroy(c->ev_in);
   if (c->ev_out) cudaEventDestroy(c->ev_out);
+  if (c->ev_batch) cudaEventDestroy(c->ev_batch);
+  for (cudaEvent_t ev : c->ev_poll)
+    if (ev) cudaEventDestroy(ev);
+  if (c->poll) cudaStreamDestroy(c->poll);
   if (c->work) cudaStreamDestroy(c->work);
   if (c->host_flags) cudaFreeHost(c->host_flags);
   if (c->host_dbl) cudaFreeHost(c->host_dbl);
