@@ -91,3 +91,20 @@ def test_unaligned_output_and_bits_repeat():
             assert torch.equal(a.reshape(-1), b[1:])
     finally:
         c.close()
+
+
+# Runs of at most a few hundred additions, many of them: their roundings average out, and
+# what is left is the result's own rounding (2^-24 / sqrt(3) over uniform mantissas) and a
+# handful of additions in pairs, each level's errors sqrt(2) smaller: below 2^-24 together.
+@pytest.mark.parametrize("dims,R,n", [
+    ((301, 257, 199), 20, 0), ((10, 52, 880), 4, 0), ((130, 77, 65, 12), 20, 3), ((227, 154, 50), 4, 2)])
+def test_sums_of_many_runs(dims, R, n):
+    ensure_built()
+    rng = np.random.default_rng(17)
+    x = rng.random(math.prod(dims)).astype(np.float32)
+    H = [rng.random((d, R)).astype(np.float32) for d in dims]
+    ref = _reference(x.astype(np.float64), dims, [h.astype(np.float64) for h in H], n)
+    M = torch.empty(dims[n], R, device="cuda")
+    nncp.nncp_mttkrp_noalloc(dims, R, torch.from_numpy(x).cuda(), [torch.from_numpy(h).cuda() for h in H], n + 1, M)
+    torch.cuda.synchronize()
+    assert rel_fro(M.cpu().numpy(), ref) <= 2.0 ** -24
