@@ -658,15 +658,6 @@ cudaError_t launch_columns(const float* X, int R, int r0, float* out, float* par
                        a.whole, a.U2, a.G2, a.two);
 }
 
-// Rows, ranks and contraction chunks that bound the scratch a context sets
-// aside for the partial sums of one MTTKRP: enough chunks of at least 256
-// elements for four 128 x 32 tiles per SM.
-int scratch_chunks(long long tiles, long long Ktot, int num_sms) {
-  const long long target = 4LL * num_sms;
-  if (tiles >= target) return 1;
-  return (int)std::min(cdiv(target, tiles), std::max(1LL, cdiv(Ktot, 256)));
-}
-
 }  // namespace
 
 cudaError_t simt_attributes_init() {
@@ -683,8 +674,7 @@ cudaError_t simt_attributes_init() {
 }
 
 size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms) {
-  const int C = scratch_chunks(cdiv(I, 128) * cdiv(R, 32), (long long)L * Q, num_sms);
-  return C > 1 ? (size_t)C * I * R : 0;
+  return scratch_floats((long long)L * Q, I, R, num_sms);
 }
 
 cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,

@@ -46,7 +46,7 @@ struct SimtArgs {
   int G2, two;             // runs; partial slots per run (1 or 2)
   float* out;
   float* slots;
-  long long slot_floats;   // BM x R
+  long long slot_floats;   // min(BM, I) x R
 };
 
 inline long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
@@ -93,7 +93,7 @@ inline bool plan_tile(const SimtPlan& base, int c, size_t cap, int num_sms, Simt
   long long left = gx % G;
   if (left * 10 >= G * 9) left = 0;  // a wave nine tenths full is left whole
   b.whole = gx - left;
-  b.slot_floats = (long long)t->BM * b.R;
+  b.slot_floats = std::min<long long>(t->BM, b.I) * b.R;
   if (left > 0) {
     // at least four steps per run; one slot per run where runs end with tiles
     long long g2 = std::max(left, std::min(G, left * b.nk / 4));
@@ -150,6 +150,21 @@ inline bool plan_simt(int64_t L, int64_t I, int64_t Q, const KrpDesc& KL, const 
     found = true;
   }
   return found;
+}
+
+// Scratch (floats) that a context sets aside for the partial tiles of one MTTKRP: chunks of at
+// least 256 elements for four tiles of 128 rows x 32 ranks per SM; for up to 512 rows,
+// which leave most of the GPU idle unless they are cut finely and whose partials are
+// small, chunks of 128 elements for four tiles of 128 rows per SM.  (Longer outputs lose
+// with finer cuts: 145 x 32 x 9 x 32 x 6 at R = 13, root -> {2..5}, 21.9 us whole and 31.3
+// in runs.  11 rows of 41 x 64 x 14 x 11 at R = 81: 100 us with the coarse chunks, 34 with
+// these.)
+inline size_t scratch_floats(long long K, long long I, int R, int num_sms) {
+  const bool few = I <= 512;
+  const long long tiles = cdiv(I, 128) * (few ? 1 : cdiv(R, 32)), target = 4LL * num_sms;
+  if (tiles >= target) return 0;
+  const long long C = std::min(cdiv(target, tiles), cdiv(K, few ? 128 : 256));
+  return C > 1 ? (size_t)C * I * R : 0;
 }
 
 }  // namespace

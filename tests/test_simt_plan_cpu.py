@@ -1,7 +1,8 @@
 """The work split of the float32 MTTKRP kernel (csrc/simt_plan.cuh), compiled for the
 host: the tiles taken whole and the tiles cut into runs are the tiles of the output,
 each once; the partial slots fit the scratch; and the tile height is the cheapest of
-those planned one by one, whatever was tried before it."""
+those planned one by one, whatever was tried before it.  Short outputs keep the GPU
+busy with the scratch that a context sets aside."""
 import math
 import os
 import random
@@ -44,6 +45,8 @@ int main() {
       base.a.U2 = 0;
       base.a.G2 = base.a.two = 0;
       for (int c = 0; c < 4 && plan_tile(base, c, cap, 152, &t); ++c) show(t);
+      // with a context's scratch: CTAs at work
+      if (plan_simt(L, I, Q, KL, KQ, R, scratch_floats(L * Q, I, R, 152), 152, &p)) printf(" %d", p.grid);
     }
     printf("\n");
   }
@@ -100,7 +103,9 @@ def test_every_tile_once_and_the_cheapest_height(planner):
         assert (1 + two) * G2 * slot <= cap
         if not two and G2:
             assert G2 % (U2 // nk) == 0
-        alone = [v[k:k + 9] for k in range(9, len(v), 9)]
+        alone = [v[k:k + 9] for k in range(9, len(v) - 1, 9)]
         assert v[:9] in alone and cost == min(a[8] for a in alone), (d, R, lo, hi)
         cut += G2 > 0
+        if I <= 512:  # few rows: 128 elements of the contraction per CTA, or a CTA per SM
+            assert v[-1] >= min(150, nk // 4), (d, R, lo, hi)
     assert cut > 1000
