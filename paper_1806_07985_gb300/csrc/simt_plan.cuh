@@ -110,7 +110,12 @@ inline bool plan_tile(const SimtPlan& base, int c, size_t cap, int num_sms, Simt
   }
   t->grid = (int)std::max<long long>(std::min(G, b.whole), b.G2);
   const double steps = (double)cdiv(b.whole, G) * b.nk + (b.G2 ? (double)cdiv(b.U2, b.G2) : 0.0);
-  t->cost = steps * (double)cdiv(t->grid, num_sms) * (t->BM + 24) * (occ == 1 ? 1.15 : 1.0);
+  // each whole tile ends with log2(KG) rounds of sums over its rows: with four steps a
+  // tile (4000 x 21 x 8 x 14 at R = 8, root -> {1, 2}) eight splits of 32 rows take
+  // 47.8 us, one of 256 rows 18.8
+  double rounds = 0.0;
+  for (int k = 1; k < b.KG; k *= 2) rounds += (double)cdiv(b.whole, G);
+  t->cost = (steps * (t->BM + 24) + rounds * t->BM) * (double)cdiv(t->grid, num_sms) * (occ == 1 ? 1.15 : 1.0);
   return true;
 }
 
@@ -141,7 +146,7 @@ inline bool plan_simt(int64_t L, int64_t I, int64_t Q, const KrpDesc& KL, const 
   a.CG = (R + 7) / 8;
   a.RP = 8 * a.CG;
   // tile rows: the least work for the busiest SM, a step costing its rows plus the
-  // part that does not depend on them
+  // part that does not depend on them (24)
   bool found = false;
   for (int c = 0; c < 4; ++c) {
     SimtPlan t;

@@ -109,3 +109,11 @@ def test_every_tile_once_and_the_cheapest_height(planner):
         if I <= 512:  # few rows: 128 elements of the contraction per CTA, or a CTA per SM
             assert v[-1] >= min(150, nk // 4), (d, R, lo, hi)
     assert cut > 1000
+
+
+@pytest.mark.parametrize("case", [(4, 8, 0, 2, 0, 4000, 21, 8, 14), (4, 3, 0, 3, 0, 59, 14, 56, 22)])
+def test_few_steps_per_tile_take_one_split(planner, case):
+    # the sums over a step's splits at the end of every tile would outweigh its few steps
+    out = subprocess.run([planner], input=" ".join(map(str, case)) + "\n", capture_output=True, text=True,
+                         check=True).stdout.split()
+    assert float(out[0]) == 256
