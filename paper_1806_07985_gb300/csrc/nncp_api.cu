@@ -63,6 +63,7 @@ struct nncp_ctx {
   float* upd_part = nullptr;  // multi-CTA update partials
   float* partials = nullptr;
   size_t part_cap = 0;
+  size_t long_cap = 0;  // ... of which MTTKRPs with many output rows use this much
   double* red_part = nullptr;
   int red_nparts = 0;
   SolveState st = {};
@@ -132,7 +133,7 @@ KrpDesc krp(const nncp_ctx* c, int first, int last) {
 struct Plan {
   size_t node_off[2][kMaxModes];
   size_t node_bytes[2][kMaxModes];
-  size_t M_off, upd_off, part_off, part_cap, gram_off, G_off, S_off, S32_off, lam_off, scal_off,
+  size_t M_off, upd_off, part_off, part_cap, long_cap, gram_off, G_off, S_off, S32_off, lam_off, scal_off,
       fits_off, flags_off, red_off;
   size_t dual_off[kMaxModes];
   int red_nparts;
@@ -171,11 +172,15 @@ Plan make_plan(const nncp_ctx* c) {
   // split-K partial capacity: max over every MTTKRP this context may launch
   size_t cap = 0;
   const int64_t IL = prod(c->dims, 0, s - 1), IR = prod(c->dims, s, N - 1);
-  cap = std::max(cap, simt_mttkrp_partials(1, IL, IR, R, c->num_sms));
-  cap = std::max(cap, simt_mttkrp_partials(IL, IR, 1, R, c->num_sms));
-  for (int n = 0; n < N; ++n)
-    cap = std::max(cap, simt_mttkrp_partials(prod(c->dims, 0, n - 1), c->dims[n],
-                                             prod(c->dims, n + 1, N - 1), R, c->num_sms));
+  auto simt = [&](bool fine) {
+    size_t most = std::max(simt_mttkrp_partials(1, IL, IR, R, c->num_sms, fine),
+                           simt_mttkrp_partials(IL, IR, 1, R, c->num_sms, fine));
+    for (int n = 0; n < N; ++n)
+      most = std::max(most, simt_mttkrp_partials(prod(c->dims, 0, n - 1), c->dims[n],
+                                                 prod(c->dims, n + 1, N - 1), R, c->num_sms, fine));
+    return most;
+  };
+  cap = std::max(cap, simt(false));
   for (int a = 0; a + 1 < s; ++a)
     cap = std::max(cap, mttv_leaf_partials(c->dims[a], prod(c->dims, a + 1, s - 1), R,
                                            c->num_sms));
@@ -187,6 +192,8 @@ Plan make_plan(const nncp_ctx* c) {
     for (int b = a + 1; b < N; ++b)
       cap = std::max(cap, mttv_leaf_partials(c->dims[a], prod(c->dims, a + 1, b), R,
                                              c->num_sms));
+  p.long_cap = cap;
+  cap = std::max(cap, simt(true));
   p.part_cap = cap;
   p.part_off = take(std::max<size_t>(cap, 1) * sizeof(float));
 
@@ -219,6 +226,7 @@ void bind_workspace(nncp_ctx* c) {
   c->upd_part = reinterpret_cast<float*>(w + p.upd_off);
   c->partials = reinterpret_cast<float*>(w + p.part_off);
   c->part_cap = p.part_cap;
+  c->long_cap = p.long_cap;
   c->st.gram_part = reinterpret_cast<double*>(w + p.gram_off);
   c->st.G = reinterpret_cast<double*>(w + p.G_off);
   c->st.S = reinterpret_cast<double*>(w + p.S_off);
@@ -250,6 +258,9 @@ void drop_graph(nncp_ctx* c) {
   c->graph4 = nullptr;
 }
 
+// scratch for the partial tiles of a float32 MTTKRP with I output rows
+size_t simt_cap(const nncp_ctx* c, int64_t I) { return simt_few_rows(I) ? c->part_cap : c->long_cap; }
+
 // ---- one partial MTTKRP from the root (precision-dependent) ----------------
 // early: see launch_simt_mttkrp
 
@@ -264,7 +275,7 @@ cudaError_t pm_right(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* lea
     return tc_partial_mttkrp(c->precision, /*contract_fast=*/0, c->X, IL, IR, KQ, c->R, out,
                              c->tc, c->num_sms, st, leaf, early);
   return launch_simt_mttkrp(static_cast<const float*>(c->X), 1, IL, IR, none, KQ, c->R, out,
-                            c->partials, c->part_cap, c->num_sms, st, early);
+                            c->partials, simt_cap(c, IL), c->num_sms, st, early);
 }
 
 cudaError_t pm_left(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* leaf = nullptr,
@@ -278,7 +289,7 @@ cudaError_t pm_left(nncp_ctx* c, float* out, cudaStream_t st, const TcLeaf* leaf
     return tc_partial_mttkrp(c->precision, /*contract_fast=*/1, c->X, IL, IR, KL, c->R, out,
                              c->tc, c->num_sms, st, leaf, early);
   return launch_simt_mttkrp(static_cast<const float*>(c->X), IL, IR, 1, KL, none, c->R, out,
-                            c->partials, c->part_cap, c->num_sms, st, early);
+                            c->partials, simt_cap(c, IR), c->num_sms, st, early);
 }
 
 cudaError_t update_mode(nncp_ctx* c, int n, cudaStream_t st) {
@@ -376,7 +387,7 @@ cudaError_t run_iteration(nncp_ctx* c, cudaStream_t st) {
       KrpDesc KL = krp(c, 0, n - 1), KQ = krp(c, n + 1, N - 1);
       cudaError_t e = launch_simt_mttkrp(static_cast<const float*>(c->X), prod(c->dims, 0, n - 1),
                                          c->dims[n], prod(c->dims, n + 1, N - 1), KL, KQ, c->R,
-                                         c->Mbuf, c->partials, c->part_cap, c->num_sms, st,
+                                         c->Mbuf, c->partials, simt_cap(c, c->dims[n]), c->num_sms, st,
                                          /*early=*/true);
       if (e == cudaSuccess) e = update_mode(c, n, st);
       if (e != cudaSuccess) return e;
@@ -731,7 +742,7 @@ nncp_status nncp_mttkrp(nncp_ctx* c, int mode, int use_dimtree, float* M_dev) {
     KrpDesc KL = krp(c, 0, n - 1), KQ = krp(c, n + 1, N - 1);
     CK(launch_simt_mttkrp(static_cast<const float*>(c->X), prod(c->dims, 0, n - 1), c->dims[n],
                           prod(c->dims, n + 1, N - 1), KL, KQ, R, M_dev, c->partials,
-                          c->part_cap, c->num_sms, st));
+                          simt_cap(c, c->dims[n]), c->num_sms, st));
     return NNCP_OK;
   }
   // read-only walk down the tree to leaf n

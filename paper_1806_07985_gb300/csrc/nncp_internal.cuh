@@ -129,7 +129,9 @@ cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
                                const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,
                                float* partials, size_t part_cap, int num_sms,
                                cudaStream_t st, bool early = false);
-size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms);
+// floats of `partials` worth giving it: with `fine` where simt_few_rows(I), 0 elsewhere
+size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms, bool fine);
+bool simt_few_rows(int64_t I);
 cudaError_t simt_attributes_init();
 
 // Records a message for nncp_global_error().

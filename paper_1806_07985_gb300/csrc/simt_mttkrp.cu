@@ -673,9 +673,10 @@ cudaError_t simt_attributes_init() {
   return cudaSuccess;
 }
 
-size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms) {
-  return scratch_floats((long long)L * Q, I, R, num_sms);
+size_t simt_mttkrp_partials(int64_t L, int64_t I, int64_t Q, int R, int num_sms, bool fine) {
+  return scratch_floats((long long)L * Q, I, R, num_sms, fine);
 }
+bool simt_few_rows(int64_t I) { return I <= kFewRows; }
 
 cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
                                const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,

@@ -157,18 +157,19 @@ inline bool plan_simt(int64_t L, int64_t I, int64_t Q, const KrpDesc& KL, const 
   return found;
 }
 
-// Scratch (floats) that a context sets aside for the partial tiles of one MTTKRP: chunks of at
-// least 256 elements for four tiles of 128 rows x 32 ranks per SM; for up to 512 rows,
-// which leave most of the GPU idle unless they are cut finely and whose partials are
-// small, chunks of 128 elements for four tiles of 128 rows per SM.  (Longer outputs lose
-// with finer cuts: 145 x 32 x 9 x 32 x 6 at R = 13, root -> {2..5}, 21.9 us whole and 31.3
-// in runs.  11 rows of 41 x 64 x 14 x 11 at R = 81: 100 us with the coarse chunks, 34 with
-// these.)
-inline size_t scratch_floats(long long K, long long I, int R, int num_sms) {
-  const bool few = I <= 512;
-  const long long tiles = cdiv(I, 128) * (few ? 1 : cdiv(R, 32)), target = 4LL * num_sms;
+// Scratch (floats) that a context sets aside for the partial tiles of one MTTKRP: chunks
+// of at least 256 elements for four tiles of 128 rows x 32 ranks per SM.  Outputs of few
+// rows leave most of the GPU idle unless they are cut finely, and their partials are
+// small: fine, chunks of 128 elements for four tiles of 128 rows per SM.  (Longer outputs
+// lose with what finer cuts they have room for: 1205 x 34 x 219 at R = 67, root -> {1, 2},
+// 78.5 us whole and 94 in runs.  11 rows of 41 x 64 x 14 x 11 at R = 81: 100 us in coarse
+// chunks, 34 in fine ones.)
+constexpr long long kFewRows = 512;
+inline size_t scratch_floats(long long K, long long I, int R, int num_sms, bool fine) {
+  if (fine && I > kFewRows) return 0;
+  const long long tiles = cdiv(I, 128) * (fine ? 1 : cdiv(R, 32)), target = 4LL * num_sms;
   if (tiles >= target) return 0;
-  const long long C = std::min(cdiv(target, tiles), cdiv(K, few ? 128 : 256));
+  const long long C = std::min(cdiv(target, tiles), cdiv(K, fine ? 128 : 256));
   return C > 1 ? (size_t)C * I * R : 0;
 }
 

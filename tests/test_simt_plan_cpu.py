@@ -46,7 +46,8 @@ int main() {
       base.a.G2 = base.a.two = 0;
       for (int c = 0; c < 4 && plan_tile(base, c, cap, 152, &t); ++c) show(t);
       // with a context's scratch: CTAs at work
-      if (plan_simt(L, I, Q, KL, KQ, R, scratch_floats(L * Q, I, R, 152), 152, &p)) printf(" %d", p.grid);
+      if (plan_simt(L, I, Q, KL, KQ, R, scratch_floats(L * Q, I, R, 152, true), 152, &p))
+        printf(" %d %zu", p.grid, scratch_floats(L * Q, I, R, 152, true));
     }
     printf("\n");
   }
@@ -103,11 +104,13 @@ def test_every_tile_once_and_the_cheapest_height(planner):
         assert (1 + two) * G2 * slot <= cap
         if not two and G2:
             assert G2 % (U2 // nk) == 0
-        alone = [v[k:k + 9] for k in range(9, len(v) - 1, 9)]
+        alone = [v[k:k + 9] for k in range(9, len(v) - 2, 9)]
         assert v[:9] in alone and cost == min(a[8] for a in alone), (d, R, lo, hi)
         cut += G2 > 0
         if I <= 512:  # few rows: 128 elements of the contraction per CTA, or a CTA per SM
-            assert v[-1] >= min(150, nk // 4), (d, R, lo, hi)
+            assert v[-2] >= min(150, nk // 4), (d, R, lo, hi)
+        else:  # finer cuts of long outputs cost more in partial tiles than they save
+            assert v[-1] == 0
     assert cut > 1000
 
 
