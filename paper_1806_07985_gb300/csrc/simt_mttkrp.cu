@@ -69,6 +69,7 @@ struct StepTab {
   int nk;                // valid elements (1..32)
   int valid;             // 0: no more steps
   int last;              // 1: last step of this CTA's run over the tile
+  int seg;               // after it: 1, 2 write or add the sums to tensor memory, 3 add those to the sums
   int slot;              // partial slot of the run, -1: the whole tile (write the output)
 };
 
@@ -95,6 +96,63 @@ __device__ __forceinline__ void cpa16_hint(uint32_t dst, const float* src, uint6
 __device__ __forceinline__ void cpa4(uint32_t dst, const float* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
 }
+// sixteen columns of this thread's tensor-memory lane
+__device__ __forceinline__ void tmem_read16(uint32_t c, float (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+      "%14, %15}, [%16];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+      : "r"(c)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_write16(uint32_t c, const float (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+      "%14, %15, %16};" ::"r"(c),
+      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+      "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+      : "memory");
+}
+// the writes of the flush before have landed
+__device__ __forceinline__ void tmem_write_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// A thread's accumulators into its tensor-memory cells (a lane, columns c .. c + 31):
+// cells = acc (+ cells when ADD), then acc = 0
+template <bool ADD>
+__device__ __forceinline__ void seg_flush(u64 (&acc)[kTM][4], uint32_t c) {
+  if (ADD) tmem_write_wait();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float v[16] = {};
+    if (ADD) tmem_read16(c + 16 * h, v);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      u64& x = acc[2 * h + k / 4][k % 4];
+      const float2 a = unpack2(x);
+      v[2 * k] += a.x;
+      v[2 * k + 1] += a.y;
+      x = 0ull;
+    }
+    tmem_write16(c + 16 * h, v);
+  }
+}
+// acc += cells
+__device__ __forceinline__ void seg_add(u64 (&acc)[kTM][4], uint32_t c) {
+  tmem_write_wait();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float v[16];
+    tmem_read16(c + 16 * h, v);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      u64& x = acc[2 * h + k / 4][k % 4];
+      const float2 a = unpack2(x);
+      x = pack2(a.x + v[2 * k], a.y + v[2 * k + 1]);
+    }
+  }
+}
+
 __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 
 
@@ -110,6 +168,7 @@ struct Feeder {
   long long u, u1;          // what is left of the run over the cut tiles
   long long rest, l, q;
   int d, slot;
+  int in_run;  // steps of the run so far; from its second segment on p.seg more than of the segment
   bool cut, first;
 
   __device__ __forceinline__ explicit Feeder(const SimtArgs& p) {
@@ -119,7 +178,7 @@ struct Feeder {
       u = run_start(blockIdx.x, p.U2, p.G2);
       u1 = run_start(blockIdx.x + 1, p.U2, p.G2);
     }
-    d = 0;
+    d = in_run = 0;
     slot = -1;
     cut = false;
     first = true;
@@ -180,6 +239,20 @@ struct Feeder {
         }
       }
     }
+    const bool last = k + 1 == kend;
+    int seg = 0;
+    if (p.seg > 0) {
+      ++in_run;
+      if (last) {
+        seg = in_run > p.seg ? 3 : 0;
+        in_run = 0;
+      } else if (in_run == p.seg) {
+        seg = 1;
+      } else if (in_run == 2 * p.seg) {
+        seg = 2;
+        in_run = p.seg;
+      }
+    }
     if ((threadIdx.x & 31) == 0) {
       t.i0 = tile << p.bm_log2;
       t.k0 = k * kBK;
@@ -189,7 +262,8 @@ struct Feeder {
       t.d = d;
       t.nk = (int)min((long long)kBK, p.K - k * kBK);
       t.valid = 1;
-      t.last = k + 1 == kend;
+      t.last = last;
+      t.seg = seg;
       t.slot = slot;
     }
     ++k;
@@ -200,12 +274,14 @@ struct Feeder {
 // rows of 32 elements, their 16-byte chunks permuted by the row (chunk ^ row
 // mod 8) so that eight neighbouring rows are read without bank conflicts;
 // otherwise (L = 1) the outputs are contiguous and stage rows are contraction
-// elements of BM outputs.
-template <bool KC>
+// elements of BM outputs.  SEG: after every p.seg steps of a run a thread's sums are
+// added to 32 columns of its tensor-memory lane, which costs no register or shared memory.
+template <bool KC, bool SEG>
 __global__ void __launch_bounds__(kThreadsMax + 32, 2)
 k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
   extern __shared__ __align__(16) float sm[];
   __shared__ StepTab tabs[kTabs];
+  __shared__ uint32_t tmem_slot;
   const int tid = threadIdx.x, T = blockDim.x - 32;
   const int BM = 1 << p.bm_log2, RP = p.RP;
   const uint32_t sbase = s_u32(sm);
@@ -252,6 +328,14 @@ k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
   if (tid >= T) {
     // ------------------------------------------------------------ feeder --
     const int lane = tid - T;
+    const uint32_t cols = T > 128 ? 64 : 32;  // a warp reaches lanes 32 (w mod 4) .. + 31
+    if constexpr (SEG) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_u32(&tmem_slot)),
+                   "r"(cols)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    }
     Feeder f(p);
     for (int s = 0; s < kStages; ++s) f.next(p, tabs[s], KC);
     __syncthreads();
@@ -281,6 +365,11 @@ k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
             __syncthreads();
           }
       }
+    }
+    if constexpr (SEG) {
+      __syncthreads();  // every warp is done with its cells
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_slot), "r"(cols) : "memory");
     }
     return;
   }
@@ -403,7 +492,7 @@ k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
   const int rgh = id % p.RGH;
   const int kg = id / p.RGH;
   const bool act = kg < p.KG;
-  const int kper = kBK / p.KG, ka = kg * kper;
+  const int kper = SEG ? kBK : kBK / p.KG, ka = SEG ? 0 : kg * kper;  // SEG: KG = 1
   const int ngroup = 8 * p.CG * p.RGH;  // threads of a k group
   u64 acc[kTM][4];
 #pragma unroll
@@ -427,6 +516,9 @@ k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
   __syncthreads();
   form_b(tabs[0], 0);
 
+  if constexpr (SEG) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  // lane 32 (w mod 4) of warp w, the columns of its group of four
+  auto cells = [&]() { return tmem_slot + ((uint32_t)(tid & 96) << 16) + 32u * (tid >> 7); };
   for (int s = 0, st = 0;; ++s) {
     // step s and the factor rows of step s + 1 have landed, and every thread
     // is done with step s - 1
@@ -489,6 +581,12 @@ k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
           }
         }
       }
+    }
+    if constexpr (SEG) {
+      const int seg = t.seg;
+      if (seg == 1) seg_flush<false>(acc, cells());
+      else if (seg == 2) seg_flush<true>(acc, cells());
+      else if (seg == 3) seg_add(acc, cells());
     }
     if (!t.last) continue;
 
@@ -560,6 +658,10 @@ k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
       for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
+  if constexpr (SEG) {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+  }
 }
 
 // Adds the partial tiles of the cut tiles.  blockIdx.y: tile.  W > 1: the W warps
@@ -643,8 +745,9 @@ cudaError_t launch_columns(const float* X, int R, int r0, float* out, float* par
   a.early = early;
   const int copies = a.vecb ? a.R / 4 : a.R;
   while (a.gsh < 5 && (1 << a.gsh) < copies) ++a.gsh;
-  cudaError_t e = launch_kernel(KC ? k_simt_mttkrp<true> : k_simt_mttkrp<false>,
-                                dim3((unsigned)pl.grid), dim3(pl.threads + 32),
+  void (*const k)(SimtArgs) = KC ? (a.seg ? k_simt_mttkrp<true, true> : k_simt_mttkrp<true, false>)
+                                 : (a.seg ? k_simt_mttkrp<false, true> : k_simt_mttkrp<false, false>);
+  cudaError_t e = launch_kernel(k, dim3((unsigned)pl.grid), dim3(pl.threads + 32),
                                 pl.smem, st, a);
   if (e != cudaSuccess || a.G2 == 0) return e;
   const long long left = a.U2 / a.nk;
@@ -661,7 +764,8 @@ cudaError_t launch_columns(const float* X, int R, int r0, float* out, float* par
 }  // namespace
 
 cudaError_t simt_attributes_init() {
-  for (auto k : {k_simt_mttkrp<false>, k_simt_mttkrp<true>}) {
+  for (auto k : {k_simt_mttkrp<false, false>, k_simt_mttkrp<true, false>, k_simt_mttkrp<false, true>,
+                 k_simt_mttkrp<true, true>}) {
     cudaError_t e =
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kStaticSmem);
     // all of the SM's shared memory: the plan counts on it for its CTAs per SM

@@ -47,6 +47,7 @@ struct SimtArgs {
   float* out;
   float* slots;
   long long slot_floats;   // min(BM, I) x R
+  int seg;                 // steps per segment of a long unsplit run (0: the whole run)
 };
 
 inline long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
@@ -109,6 +110,19 @@ inline bool plan_tile(const SimtPlan& base, int c, size_t cap, int num_sms, Simt
     }
   }
   t->grid = (int)std::max<long long>(std::min(G, b.whole), b.G2);
+  const long long run = std::max(b.whole ? b.nk : 0, b.G2 ? std::min(b.nk, cdiv(b.U2, b.G2)) : 0);
+  // A run is one chain of float32 additions per output (KG of them where steps are split),
+  // whose error grows with the square root of its length.  The kernel before this one cut
+  // the contraction into `parts` chunks; whole runs of more than 1.25 times that length
+  // were up to 1.95 times as far from float64 (301 x 257 x 199 at R = 20, root -> {2, 3}:
+  // 2.6e-7, 1.3e-7 in segments of 160).  Others stay whole, since the form with segments
+  // costs more than its flushes where a thread copies 16 bytes along the contraction:
+  // 512^3 at R = 32, root -> {2, 3} 250 -> 270 us, 40000 x 48 x 40 at R = 16 92 -> 105;
+  // 301 x 257 x 199 45.3 -> 45.5.
+  const long long tiles = cdiv(b.I, 128) * cdiv(b.R, 32);
+  const long long parts = std::max(1LL, std::min(cdiv(4LL * num_sms, tiles), cdiv(b.K, 256)));
+  const long long chain = std::min(b.K, run * kBK);
+  if (b.KG == 1 && run > 5 && tiles < 4LL * num_sms && (double)chain * parts > 1.25 * b.K) b.seg = run > 32 ? 10 : 5;
   const double steps = (double)cdiv(b.whole, G) * b.nk + (b.G2 ? (double)cdiv(b.U2, b.G2) : 0.0);
   // each whole tile ends with log2(KG) rounds of sums over its rows: with four steps a
   // tile (4000 x 21 x 8 x 14 at R = 8, root -> {1, 2}) eight splits of 32 rows take

@@ -108,3 +108,35 @@ def test_sums_of_many_runs(dims, R, n):
     nncp.nncp_mttkrp_noalloc(dims, R, torch.from_numpy(x).cuda(), [torch.from_numpy(h).cuda() for h in H], n + 1, M)
     torch.cuda.synchronize()
     assert rel_fro(M.cpu().numpy(), ref) <= 2.0 ** -24
+
+
+# A chain of n float32 additions of nonnegative terms of one size is off by at most
+# 2^-24 sqrt(n) / 3 of its sum (rms; each addition rounds by up to 2^-24 / sqrt(3) of a partial
+# sum).  A run of up to 32 steps is added in segments of 160 elements, a longer one in
+# segments of 320, and the segments one after the other; then come the result's own rounding
+# and the pairs above.
+@pytest.mark.parametrize("dims,R,split,seg", [
+    ((300, 256, 200), 20, 1, 160), ((301, 257, 199), 20, 1, 160), ((33, 23, 120, 82), 93, 2, 160),
+    ((521, 110, 111), 85, 1, 160), ((1140, 130, 162), 35, 1, 320)])
+def test_long_runs_in_segments(dims, R, split, seg):
+    ensure_built()
+    rng = np.random.default_rng(23)
+    x = rng.random(math.prod(dims)).astype(np.float32)
+    H = [rng.random((d, R)).astype(np.float32) for d in dims]
+    L = math.prod(dims[:split])
+    k = np.ones((1, R))
+    for h in H[:split]:
+        k = (h.astype(np.float64)[:, None] * k).reshape(-1, R)
+    ref = x.astype(np.float64).reshape(-1, L) @ k
+    c = nncp.Context(dims, R, root_split=split)
+    try:
+        c.set_tensor(torch.from_numpy(x).cuda())
+        c.set_factors([torch.from_numpy(h).cuda() for h in H])
+        T = torch.full(ref.shape, float("nan"), device="cuda", dtype=torch.float32)
+        c.partial_mttkrp(1, T)
+        torch.cuda.synchronize()
+    finally:
+        c.close()
+    segs = [min(seg, L - a) for a in range(0, L, seg)]
+    bound = 2.0 ** -24 / 3 * math.sqrt(sum(n ** 3 for n in segs) / L ** 2 + len(segs) + 3)
+    assert rel_fro(T.cpu().numpy(), ref) <= bound
