@@ -17,8 +17,7 @@ constexpr long long kBatchMaxElems = (1LL << 31) - 1;  // per tensor (32-bit ind
 
 // Tiles of the two root partial MTTKRPs.  X_(1) of a tensor is read as rows j
 // of I_1 contiguous floats; a tile is a run of whole rows (a multiple of four
-// rows, so every tile starts 16-byte aligned), at most kTileFloats floats,
-// double-buffered in shared memory.
+// rows, so every tile starts 16-byte aligned), at most kTileFloats floats.
 constexpr int kTileFloats = 4096;
 constexpr int kWsFloats = 2048;       // Khatri-Rao tile (rows x padded rank)
 constexpr int kLeftMaxRows = 512;     // padded X tile <= kTileFloats + kLeftMaxRows

@@ -15,13 +15,19 @@ namespace nncp {
 // calls pdl_wait() before its first access to memory that an earlier kernel
 // writes, or that a later one writes while an earlier one may still read it.  pdl_wait() returns
 // once every predecessor grid has completed and its writes are visible, so the
-// chain stays ordered transitively.  (Only the tensor may be read earlier, and only
-// in the library's own capture of an iteration, where no kernel writes it: the
-// entry points also run on a caller's stream, which may be captured behind a
-// kernel that writes the tensor and triggers early.)  Small kernels then call pdl_trigger(), which
+// chain stays ordered transitively.  Small kernels then call pdl_trigger(), which
 // lets their successor be scheduled on the SMs they leave free; large grids do
 // not, so their successor is scheduled as their CTAs exit.  Outside such a
 // launch both return at once.
+// Two exceptions, both for the library's own capture of an iteration only:
+//   * the tensor, which no kernel of an iteration writes, may be read before the wait.
+//     The entry points also run on a caller's stream, which may be captured behind a
+//     kernel that writes the tensor and triggers early: there they wait first;
+//   * a mode update's row kernel reads S, lambda and its factor before the wait, all of
+//     them written no later than the update before it.  An MTTKRP or multi-TTV stands
+//     between two updates and, like every kernel here, lets its successor start only
+//     after its own wait.  A row kernel placed right after k_finish or another update
+//     would have to wait first.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -254,7 +260,9 @@ cudaError_t launch_gram_only(const float* H, int64_t In, int R, SolveState st,
 //   W^T W = sum of the partials; lam = sqrt(diag); G_n = D^-1 W^T W D^-1;
 //   H_n = W / lam (in place); if is_last: fit from the Sec. IV-B identity;
 //   S for mode next_mode.
-//   gscr: kFinishScratch doubles of device scratch.
+//   gscr: kFinishScratch doubles of device scratch, one per CTA.
+//   (The next row kernel reads S and lambda before its wait: an MTTKRP or multi-TTV
+//   has to come between, as the rule on pdl_wait() says.)
 //   U non-null: the rows' ADMM duals, divided by the new lambda along with H.
 constexpr int kFinishScratch = 304;
 cudaError_t launch_finish(float* H, int64_t In, int R, int N, int n, int next_mode, int is_last,

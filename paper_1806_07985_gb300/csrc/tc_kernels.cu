@@ -532,7 +532,7 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
               tma_load_2d(dst, &tmap, k0, m0, raw_full(sf), pol);
               tma_load_2d(dst + 16384, &tmap, k0 + 32, m0, raw_full(sf), pol);
             }
-          } else if (!SPLIT && p.a_mn) {  // (a split pass is not asked: 220 x 230 x 1818 81.4 -> 82.9 us)
+          } else if (!SPLIT && p.a_mn) {  // (never so in a split pass, which the test alone slowed by 2 %)
             tma_load_2d(dst, &tmap, m0, k0, raw_full(sf), pol);
             tma_load_2d(dst + 8192, &tmap, m0 + 64, k0, raw_full(sf), pol);
           } else {
@@ -1346,9 +1346,11 @@ cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, i
   // 16.6 -> 17.8, of 77 to 90 5 to 10 % slower), and from 256 with it, whose builders also
   // split the rows (600 x 404 x 330: 123 -> 98 us; 304 x 257 x 200 at R = 60: 38.4 -> 35.4;
   // a mode of 250 51.6 -> 55.4, of 130 26.9 -> 28.4).  A mode alone saves only its
-  // element offsets, which pays past 32 ranks (two rows per lane) and from 500 on (600 at
-  // R = 40: split 110 -> 89 us, bf16 53.8 -> 51.7; 276 at R = 33 44.3 -> 45.1 a sweep, 484
-  // at R = 26 59.1 -> 60.0).
+  // element offsets, which pays past 32 ranks (two rows per lane) and from 500 on: at R =
+  // 33 to 64 a contraction takes 0.87 to 0.97 of its time at 520 elements, 0.81 to 0.90 at
+  // 840 and 0.77 to 0.86 at 2200 in every precision and from either side; at 200 to 440 it
+  // takes 0.91 to 1.00 (276 at R = 33 44.3 -> 45.1 a sweep), at R = 24 0.87 to 1.01 (484 at
+  // R = 26 59.1 -> 60.0).
   const bool wrap = !leaf && K.dim[0] % kKC != 0 && K.dim[0] >= (split ? 256 : 192) &&
                     (K.nm > 1 || (R > 32 && K.dim[0] >= 500));
   void (*const kern)(CUtensorMap, TcParams) =
