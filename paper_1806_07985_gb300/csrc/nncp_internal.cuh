@@ -92,6 +92,12 @@ cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, c
   return launch_kernel_cluster(k, grid, block, smem, st, 0, std::forward<A>(args)...);
 }
 
+// A launch on st is ordered after everything before it without pdl_wait().
+inline bool launch_ordered(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusActive;
+  return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+}
+
 constexpr int kMaxModes = 8;
 constexpr int kMaxRank = 128;
 constexpr int kFitCapacity = 1 << 16;  // fit history slots on the device
@@ -128,9 +134,9 @@ struct SolveState {
 // for i < I, r < R: the generic (direct or partial) MTTKRP on CUDA cores.
 // X is float32.  When the contraction is split across CTAs the per-chunk
 // results go to `partials` (capacity `part_cap` floats) and are summed in a
-// fixed order, so results are bitwise reproducible.  early: nothing that may
-// still run when this launch starts writes X (in the library's own capture of
-// an iteration), so tensor tiles may be read before pdl_wait().
+// fixed order, so results are bitwise reproducible.  early: no kernel before this
+// launch in its capture writes X (the library's own capture of an iteration), so
+// tensor tiles may be read before pdl_wait(), as outside a capture.
 cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
                                const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,
                                float* partials, size_t part_cap, int num_sms,

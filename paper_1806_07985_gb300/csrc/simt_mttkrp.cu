@@ -742,7 +742,7 @@ cudaError_t launch_columns(const float* X, int R, int r0, float* out, float* par
   // a tensor that cannot stay in the 126 MB L2 is marked evict-first, so that
   // its stream leaves the nodes and factors there
   a.evict = (double)a.I * a.K * sizeof(float) > 96e6;
-  a.early = early;
+  a.early = early || launch_ordered(st);
   const int copies = a.vecb ? a.R / 4 : a.R;
   while (a.gsh < 5 && (1 << a.gsh) < copies) ++a.gsh;
   void (*const k)(SimtArgs) = KC ? (a.seg ? k_simt_mttkrp<true, true> : k_simt_mttkrp<true, false>)

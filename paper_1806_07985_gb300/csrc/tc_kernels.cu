@@ -417,7 +417,7 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
   // read, so only they wait for it (pdl_wait); the producer streams the tensor,
   // which nothing in the iteration writes, and the converters fill the tensor-
   // memory A stages from it in the meantime.  Where that is not known (a caller's
-  // stream: p.early = 0) every thread waits before the roles part, so that no
+  // capture: p.early = 0) every thread waits before the roles part, so that no
   // bounded wait runs on while the predecessor does.  The kernel does not trigger its
   // successor early: that one is scheduled as CTAs exit, and CTAs placed on the
   // first SMs to free up would crowd there instead of spreading over the GPU.
@@ -1308,7 +1308,7 @@ cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, i
   p.mode = precision;
   p.contract_fast = contract_fast;
   p.bf16x = bf16x;
-  p.early = early;
+  p.early = early || launch_ordered(st);
   p.a_mn = bf16x && !contract_fast;
   p.direct = (contract_fast && precision != NNCP_SPLIT_BF16X3) || p.a_mn;
   p.seg = precision == NNCP_SPLIT_BF16X3 ? kSegStages : (1 << 30);
