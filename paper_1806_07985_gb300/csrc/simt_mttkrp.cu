@@ -38,17 +38,18 @@
 // Work split: G CTAs (what fits on the GPU at once) take whole tiles in turn;
 // the tiles of a last, partly filled wave are cut into G equal runs of steps
 // instead (a run may straddle two tiles), whose partial tiles go to `slots` and
-// are added in run order by k_simt_fixup.  Every cut follows from the shape and
-// the scratch size alone, so results are bitwise reproducible.
+// are added in a fixed order by k_simt_fixup.  Every cut follows from the shape and
+// the scratch size alone, so results are bitwise reproducible (simt_plan.cuh).  A long
+// run whose steps are not split adds up in segments (SEG).
 //
-// Measured on a GB300 per root branch (outputs slow / fast), the 128 x 32 tile
-// kernel of one FMA per issue slot that this one replaced in brackets: 512^3
-// R = 8 117 / 104 us (358 / 411), R = 32 260 / 250 us (363 / 416), 40000x48x40
-// R = 16 121 / 95 us (292 / 230), 301x257x199 R = 20 68 / 49 us (74 / 85),
-// 220x180x150 R = 100 80 / 66 us (90 / 91).  At R = 8 it streams at 4.6 to 5.2
-// TB/s; at R = 32 it runs at 0.44 of the FMA peak, of which a step's loads,
-// Khatri-Rao rows and barrier take a quarter and the shared-memory reads (three
-// of 16 bytes per 16 packed FMAs) most of the rest.
+// Measured on a GB300 per root branch (outputs slow / fast, calls repeated on one
+// tensor), the 128 x 32 tile kernel of one FMA per issue slot that this one replaced in
+// brackets: 512^3 R = 8 102 / 101 us (358 / 411), R = 32 246 / 250 us (363 / 416),
+// 40000x48x40 R = 16 119 / 92 us (292 / 230), 301x257x199 R = 20 56 / 45 us (74 / 85),
+// 220x180x150 R = 100 70 / 66 us (90 / 91).  At R = 8 it streams at 5.3 TB/s; at R = 32 it
+// runs at 0.44 of the FMA peak, of which a step's loads, Khatri-Rao rows and barrier take
+// a quarter and the shared-memory reads (three of 16 bytes per 16 packed FMAs) most of
+// the rest.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -669,7 +670,7 @@ k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
 // tile, and warp 0 adds the warps' sums; W = 1: a thread per output adds the runs.
 // A thread's runs go to four sums in turn and everything after that is added in
 // pairs: with runs and warps added one after the other, the last 32 additions alone
-// made the error of a 301 x 257 x 199 contraction at R = 20 8.6e-8, not 5.0e-8.  (Four threads per output left 760 runs of a 12 x 20 output
+// made the error of a 301 x 257 x 199 contraction at R = 20 8.6e-8, not 4.1e-8.  (Four threads per output left 760 runs of a 12 x 20 output
 // to ten CTAs: 108 us on a GB300, more than the MTTKRP.)
 template <int W>
 __global__ void __launch_bounds__(W > 1 ? 32 * W : 256)
