@@ -20,9 +20,10 @@ namespace nncp {
 // not, so their successor is scheduled as their CTAs exit.  Outside such a
 // launch both return at once.
 // Two exceptions, both for the library's own capture of an iteration only:
-//   * the tensor, which no kernel of an iteration writes, may be read before the wait.
-//     The entry points also run on a caller's stream, which may be captured behind a
-//     kernel that writes the tensor and triggers early: there they wait first;
+//   * the tensor, which no kernel of an iteration writes, is read before the wait.  The
+//     entry points also run on a caller's stream, which may be captured behind a kernel
+//     that writes the tensor and triggers early: there the kernels that read the tensor
+//     are launched without programmatic serialization (launch_kernel_if);
 //   * a mode update's row kernel reads S, lambda and its factor before the wait, all of
 //     them written no later than the update before it.  An MTTKRP or multi-TTV stands
 //     between two updates and, like every kernel here, lets its successor start only
@@ -53,12 +54,12 @@ __device__ __forceinline__ float2 unpack2(u64 v) {
 }
 
 // Launches k(args...) on st: with programmatic stream serialization while st is
-// being captured into a graph, as an ordinary launch otherwise.  Only kernels
-// that follow the pdl_wait() rule above are launched through this.
+// being captured into a graph (and `programmatic`), as an ordinary launch otherwise.
+// Only kernels that follow the pdl_wait() rule above are launched through this.
 // cluster_x > 0 launches the grid as thread-block clusters of cluster_x CTAs.
 template <typename... P, typename... A>
-cudaError_t launch_kernel_cluster(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
-                                  cudaStream_t st, int cluster_x, A&&... args) {
+cudaError_t launch_kernel_any(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              int cluster_x, bool programmatic, A&&... args) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaStreamIsCapturing(st, &cs);
   if (e != cudaSuccess) return e;
@@ -71,7 +72,7 @@ cudaError_t launch_kernel_cluster(void (*k)(P...), dim3 grid, dim3 block, size_t
     at[na].val.clusterDim.z = 1;
     ++na;
   }
-  if (cs == cudaStreamCaptureStatusActive) {
+  if (programmatic && cs == cudaStreamCaptureStatusActive) {
     at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[na].val.programmaticStreamSerializationAllowed = 1;
     ++na;
@@ -87,15 +88,21 @@ cudaError_t launch_kernel_cluster(void (*k)(P...), dim3 grid, dim3 block, size_t
 }
 
 template <typename... P, typename... A>
-cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                          A&&... args) {
-  return launch_kernel_cluster(k, grid, block, smem, st, 0, std::forward<A>(args)...);
+cudaError_t launch_kernel_cluster(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t st, int cluster_x, A&&... args) {
+  return launch_kernel_any(k, grid, block, smem, st, cluster_x, true, std::forward<A>(args)...);
 }
 
-// A launch on st is ordered after everything before it without pdl_wait().
-inline bool launch_ordered(cudaStream_t st) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusActive;
-  return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                          A&&... args) {
+  return launch_kernel_any(k, grid, block, smem, st, 0, true, std::forward<A>(args)...);
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_kernel_if(bool programmatic, void (*k)(P...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t st, A&&... args) {
+  return launch_kernel_any(k, grid, block, smem, st, 0, programmatic, std::forward<A>(args)...);
 }
 
 constexpr int kMaxModes = 8;
@@ -135,8 +142,8 @@ struct SolveState {
 // X is float32.  When the contraction is split across CTAs the per-chunk
 // results go to `partials` (capacity `part_cap` floats) and are summed in a
 // fixed order, so results are bitwise reproducible.  early: no kernel before this
-// launch in its capture writes X (the library's own capture of an iteration), so
-// tensor tiles may be read before pdl_wait(), as outside a capture.
+// launch in its capture writes X (the library's own capture of an iteration), so it
+// may start, and read tensor tiles, while the one just before it runs.
 cudaError_t launch_simt_mttkrp(const float* X, int64_t L, int64_t I, int64_t Q,
                                const KrpDesc& KL, const KrpDesc& KQ, int R, float* out,
                                float* partials, size_t part_cap, int num_sms,

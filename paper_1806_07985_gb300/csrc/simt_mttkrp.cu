@@ -502,10 +502,9 @@ k_simt_mttkrp(const __grid_constant__ SimtArgs p) {
     for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
 
   __syncthreads();
-  // the tensor is written by no kernel of an iteration: there (early) its first
-  // tiles stream in while the preceding kernel finishes; a caller's stream may
-  // hold a kernel that writes it
-  if (!p.early) pdl_wait();
+  // the tensor is written by no kernel of an iteration, where alone the kernel may
+  // start early (launch_columns): its first tiles stream in while the preceding
+  // kernel finishes
   load_x(tabs[0], 0);
   load_x(tabs[1], 1);
   pdl_wait();
@@ -743,12 +742,11 @@ cudaError_t launch_columns(const float* X, int R, int r0, float* out, float* par
   // a tensor that cannot stay in the 126 MB L2 is marked evict-first, so that
   // its stream leaves the nodes and factors there
   a.evict = (double)a.I * a.K * sizeof(float) > 96e6;
-  a.early = early || launch_ordered(st);
   const int copies = a.vecb ? a.R / 4 : a.R;
   while (a.gsh < 5 && (1 << a.gsh) < copies) ++a.gsh;
   void (*const k)(SimtArgs) = KC ? (a.seg ? k_simt_mttkrp<true, true> : k_simt_mttkrp<true, false>)
                                  : (a.seg ? k_simt_mttkrp<false, true> : k_simt_mttkrp<false, false>);
-  cudaError_t e = launch_kernel(k, dim3((unsigned)pl.grid), dim3(pl.threads + 32),
+  cudaError_t e = launch_kernel_if(early, k, dim3((unsigned)pl.grid), dim3(pl.threads + 32),
                                 pl.smem, st, a);
   if (e != cudaSuccess || a.G2 == 0) return e;
   const long long left = a.U2 / a.nk;

@@ -30,7 +30,6 @@ struct SimtArgs {
   int gsh;                // 2^gsh lanes copy a factor row (all of it in one go when vecb)
   int fk, fc;             // threads / (RP / 4) and the remainder
   int vecx, vecb, veco, evict;
-  int early;              // tensor tiles before the wait for the preceding kernel
   int nm;                 // contracted modes, fastest first
   int dim[kMaxModes];     // their lengths
   int dstep, mag0, magl;  // 32 mod dim[0]; ceil(2^16 / dim[0]) and / L below 32, else 0

@@ -104,7 +104,6 @@ struct TcParams {
   int direct;  // MMA reads the TMA stage (no converter)
   int a_mn;    // ... MN-major (bf16 tensor, contract_slow)
   int bf16x;   // tensor stored as bf16
-  int early;   // the tensor may be read before the wait for the preceding kernel
   int b_resident;  // every unit spans the whole contraction: B formed once per CTA
   // Stages accumulated in one tensor-memory accumulator before it is added into
   // float32 registers (split-BF16x3; one segment per unit otherwise).  The
@@ -416,10 +415,9 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
   // epilogue (output) touch memory that other kernels of the iteration write or
   // read, so only they wait for it (pdl_wait); the producer streams the tensor,
   // which nothing in the iteration writes, and the converters fill the tensor-
-  // memory A stages from it in the meantime.  Where that is not known (a caller's
-  // capture: p.early = 0) every thread waits before the roles part, so that no
-  // bounded wait runs on while the predecessor does.  The kernel does not trigger its
-  // successor early: that one is scheduled as CTAs exit, and CTAs placed on the
+  // memory A stages from it in the meantime.  (A caller's capture, whose kernels may
+  // write the tensor, launches it without that serialization.)  The kernel does not
+  // trigger its successor early: that one is scheduled as CTAs exit, and CTAs placed on the
   // first SMs to free up would crowd there instead of spreading over the GPU.
   extern __shared__ uint8_t smem_dyn[];
   const uint32_t sbase_raw = smem_u32(smem_dyn);
@@ -504,8 +502,6 @@ k_tc_partial_mttkrp(const __grid_constant__ CUtensorMap tmap, TcParams p) {
 
   const long long n_units = p.n_units;
   const int R = p.R;
-
-  if (!p.early) pdl_wait();
 
   if (warp == kWarpTMA) {
     // ---------------------------------------------------------- producer --
@@ -1308,7 +1304,6 @@ cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, i
   p.mode = precision;
   p.contract_fast = contract_fast;
   p.bf16x = bf16x;
-  p.early = early || launch_ordered(st);
   p.a_mn = bf16x && !contract_fast;
   p.direct = (contract_fast && precision != NNCP_SPLIT_BF16X3) || p.a_mn;
   p.seg = precision == NNCP_SPLIT_BF16X3 ? kSegStages : (1 << 30);
@@ -1358,7 +1353,7 @@ cudaError_t tc_partial_mttkrp(int precision, int contract_fast, const void* X, i
       : !wrap ? (split ? k_tc_partial_mttkrp<false, true, false> : k_tc_partial_mttkrp<false, false, false>)
       : split ? k_tc_partial_mttkrp<false, true, true>
               : k_tc_partial_mttkrp<false, false, true>;
-  cudaError_t e = launch_kernel(kern, dim3(grid), dim3(kThreads), p.sm.total, st, map, p);
+  cudaError_t e = launch_kernel_if(early, kern, dim3(grid), dim3(kThreads), p.sm.total, st, map, p);
   if (e != cudaSuccess) return e;
   if (leaf) {
     // the CTAs' partial leaves, summed in CTA order
